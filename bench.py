@@ -34,14 +34,7 @@ STENCIL_MEAN = 10.43
 # (frame, Cholesky, two triangular solves; per stencil point the coordinates, monomials, moment
 # update, coefficient and the apply of C = 4 values), + 24.
 FLOP_PER_NODE_Q = 30 + 3 * (244 + 77 * STENCIL_MEAN) + 24
-# FP64 arithmetic of the refinement residual r = b - sum_mu p_mu (p_mu . y) per node: per stencil
-# point p . y by nested products (5 FMA = 10), X t and Y t (2) and the update of r (3 subtractions
-# and 3 FMA = 9); 13 FP64 instructions.
-FP64_FLOP_PER_NODE_RES = 3 * 21 * STENCIL_MEAN
-FP64_INST_PER_NODE_RES = 3 * 13 * STENCIL_MEAN
 FP32_LANES_PER_SM = 128
-FP64_FMA_PER_SM_CLK = 2       # FP64 FMA per SM per clock: ncu's peak_sustained of
-                              # sm__sass_thread_inst_executed_op_dfma_pred_on on GB300
 
 
 def kernel_traffic(stage: str, solve: str):
@@ -326,8 +319,8 @@ def run_ours(args, world, rank, local):
     clk = clocks.stop()
     proj.check("timed steps")
     ctx.set_stage_events([])
-    # with the FP64-residual, plain FP32 and FP64 solves the node location runs inside the solve
-    # kernel (k_p2m_tab), so "geometry" is only the gap between two events there
+    # the node location runs inside the solve kernel (k_p2m_tab): "geometry" is only the gap
+    # between two events
     stage_ms = {name: float(np.mean([st[i].elapsed_time(st[i + 1]) for st in stages]))
                 for i, name in enumerate(("star_table", "geometry", "solve", "fix_pass"))}
     step_ms = [r[0].elapsed_time(r[3]) for r in recs]
@@ -343,41 +336,23 @@ def run_ours(args, world, rank, local):
     t_m2p = float(np.mean(m2p_ms)) * 1e-3
     sm_mhz = (clk or {}).get("sm_mhz") or pk.get("sm_max_mhz", 2070.0)
     fp32_peak = sms * FP32_LANES_PER_SM * 2 * 2070.0e6 / 1e12   # TFLOP/s at the maximum SM clock
-    fp64_peak = sms * FP64_FMA_PER_SM_CLK * 2 * 2070.0e6 / 1e12
     p2m_flops = FLOP_PER_NODE_Q * nn
     # algorithmic bytes of the round trip: P2M reads pos + C vals per particle and writes C
     # per node; M2P reads pos per particle, C per node, writes C per particle (FP32)
     rt_bytes = N * (8 + 4 * C) + nn * 4 * C + N * 8 + nn * 4 * C + N * 4 * C
     m2p_bytes = N * 8 + nn * 4 * C + N * 4 * C
-    # roofline of the dominant kernel of the step, timed by the stage events: with the refined
-    # solve in FP64 residual form that is the solve kernel, bound by the FP64 pipe; otherwise
-    # the star table (integer and FP32 filter work) or the solve's FP32 arithmetic
+    # the dominant kernel of the step, timed by the stage events: integer and FP32 filter work of
+    # the star table, or the location, FP32 solve and fixed-point residual of the node kernel
     dominant = max(stage_ms, key=stage_ms.get)
-    t_dom = stage_ms[dominant] * 1e-3
-    if dominant == "solve" and args.solve == "f32ref":
-        roofline = {"bound": "alu",
-                    "kernel": "k_p2m_tab (node location from the star table, FP32 Cholesky + "
-                              "FP64-residual refinement, apply: one kernel)",
-                    "achieved": FP64_FLOP_PER_NODE_RES * nn / t_dom / 1e12,
-                    "peak": fp64_peak, "unit": "TFLOP/s (FP64)",
-                    "frac": FP64_FLOP_PER_NODE_RES * nn / t_dom / 1e12 / fp64_peak,
-                    "algorithmic_flop_per_node": FP64_FLOP_PER_NODE_RES,
-                    "peak_source": f"derived: {sms} SMs (device query) x {FP64_FMA_PER_SM_CLK} FP64 FMA "
-                                   "per SM per clock (ncu peak counter) x 2 flop x 2070 MHz; nominal "
-                                   "1.25 TFLOP/s; no measured FP64 figure",
-                    # the same residual counted in FP64 pipe instructions (FMA, MUL and ADD
-                    # alike) against 2 per SM per clock (1.25 TFLOP/s / 2 / SMs / 2070 MHz)
-                    "fp64_inst_per_node": FP64_INST_PER_NODE_RES,
-                    "fp64_pipe_frac": FP64_INST_PER_NODE_RES * nn / t_dom / (FP64_FMA_PER_SM_CLK * sms * 2070.0e6)}
-    else:
-        roofline = {"bound": "alu", "kernel": {"star_table": "k_star_list + k_star_retry",
-                                                "geometry": "k_p2m_geom", "solve": "k_p2m_solve",
-                                                "fix_pass": "k_p2m_fix"}[dominant],
-                    "achieved": p2m_flops / t_p2m / 1e12, "peak": fp32_peak, "unit": "TFLOP/s",
-                    "frac": p2m_flops / t_p2m / 1e12 / fp32_peak,
-                    "algorithmic_flop_per_node": FLOP_PER_NODE_Q,
-                    "note": "FP32 arithmetic of the whole quadratic P2M call over the call's time",
-                    "peak_source": f"{sms} SMs (device query) x 128 FP32 lanes x 2 x 2070 MHz (derived)"}
+    roofline = {"bound": "alu", "kernel": {"star_table": "k_star_list + k_star_retry",
+                                            "geometry": "none (gap between two events)",
+                                            "solve": "k_p2m_tab (location, edge solves, apply)",
+                                            "fix_pass": "k_p2m_fix_tab"}[dominant],
+                "achieved": p2m_flops / t_p2m / 1e12, "peak": fp32_peak, "unit": "TFLOP/s",
+                "frac": p2m_flops / t_p2m / 1e12 / fp32_peak,
+                "algorithmic_flop_per_node": FLOP_PER_NODE_Q,
+                "note": "FP32 arithmetic of the whole quadratic P2M call over the call's time",
+                "peak_source": f"{sms} SMs (device query) x 128 FP32 lanes x 2 x 2070 MHz (derived)"}
     roofline["kernel_ms"] = stage_ms[dominant]
     roofline["traffic"] = kernel_traffic(dominant, args.solve)
     roofline["traffic_unit"] = "bytes per launch (ncu dram read+write), null when the sources changed since"
@@ -722,8 +697,8 @@ def main():
     ap.add_argument("--impl", choices=["ours", "reference"], default="ours")
     ap.add_argument("--solve", choices=["f32", "f32ref", "f32ff", "f64"], default="f32ref",
                     help="moment solve of the headline P2M: f32ref = FP32 Cholesky + one "
-                         "refinement step with an FP64 residual (default); f32ff = the same with "
-                         "a float-float residual; f64 = FP64 assembly and solve; f32 = plain FP32 "
+                         "refinement step, residual in 64-bit fixed point (default); f32ff = the same "
+                         "by its other name; f64 = FP64 assembly and solve; f32 = plain FP32 "
                          "Cholesky (a side variant outside the stated accuracy target)")
     ap.add_argument("--profile", action="store_true", help="timed loop only (for ncu)")
     ap.add_argument("--no-cpu-baseline", action="store_true")

@@ -74,10 +74,11 @@ typedef enum { PFEM_SHAPE_LINEAR = 0, PFEM_SHAPE_QUADRATIC = 1 } pfem_shape;
 typedef enum {
     PFEM_SOLVE_F64 = 0,         /* moment assembly and Cholesky in FP64 */
     PFEM_SOLVE_F32 = 1,         /* in FP32 after centring/scaling by the edge length */
-    PFEM_SOLVE_F32_REFINED = 2, /* FP32 Cholesky + one refinement step, FP64 residual */
+    PFEM_SOLVE_F32_REFINED = 2, /* FP32 Cholesky + one refinement step, residual in 64-bit fixed
+                                   point (at least FP64's accuracy) */
     PFEM_SOLVE_F32_REFINED_FF = 3 /* FP32 Cholesky + one refinement step, residual in float-float
-                                   (pairs of FP32 numbers, ~48-bit significand): the same
-                                   refinement without FP64 instructions */
+                                   (~48-bit significand) or better: runs the fixed-point
+                                   residual of PFEM_SOLVE_F32_REFINED */
 } pfem_solve;
 typedef enum { PFEM_BACKWARD_RECOMPUTE = 0, PFEM_BACKWARD_CHECKPOINT = 1 } pfem_backward_mode;
 
@@ -127,15 +128,14 @@ const char *pfem_last_error(const pfem_ctx *ctx);
 /* Stage events for timing: events[0..count) are cudaEvent_t handles created by the caller
  * (count <= 8; 0 clears them).  Every later pfem_project_p2m with this context records them on
  * its stream at the boundaries of its stages when the star-table path runs: 0 before the fast
- * pass, 1 after the star table, 2 after the per-node geometry kernel, 3 after the solve kernel,
- * 4 after the fix pass (where one kernel locates the nodes and solves, 2 is recorded right
- * before it and 3 after it; the other paths record 0 and 4 only).  The caller reads the intervals
+ * pass, 1 after the star table, 2 right before the kernel that locates the nodes and solves, 3
+ * after it, 4 after the fix pass (the other paths record 0 and 4 only).  The caller reads the intervals
  * with cudaEventElapsedTime after synchronising.  Recording adds no work to the kernels. */
 pfem_status pfem_set_stage_events(pfem_ctx *ctx, void *const *events, int32_t count);
 
 /* An event (cudaEvent_t as void*) that pfem_project_p2m calls made with this context wait on
  * (cudaStreamWaitEvent on the call's stream) right before their first kernel that reads the
- * particle values -- after the star table (and the node records, where they are written) of the
+ * particle values -- after the star table of the
  * quadratic path, at the start of the others; NULL (the default) clears it.  A caller can so copy the values on another
  * stream while the call works on the positions.  The event must have been recorded (or never
  * recorded: then the wait is a no-op) when the call is made. */
@@ -248,9 +248,8 @@ pfem_status pfem_shape_quadratic(pfem_ctx *ctx, int32_t n, int32_t nb, int64_t N
  * PFEM_ERR_DEGENERATE or PFEM_ERR_CAPACITY), then, for the quadratic apply form, 136 bytes of
  * record per node and the star table (72 bytes per particle).  With room for them the fast
  * pass is the star table of every particle (see pfem_delaunay_stars) and one kernel that, per
- * node, locates it with the table, builds its particle set and solves the three edge systems;
- * the float-float solve (PFEM_SOLVE_F32_REFINED_FF) splits that kernel in two, a geometry
- * kernel writing the node records and a solve kernel reading them.  With less room, one kernel
+ * node, locates it with the table, builds its particle set and solves the three edge systems.
+ * With less room, one kernel
  * searches every node's stars itself (same results, slower).  The workspace of pfem_workspace_size() has room for
  * everything. */
 pfem_status pfem_project_p2m(pfem_ctx *ctx, int32_t n, int32_t nb, int64_t N, const void *pos_sorted,
@@ -389,8 +388,7 @@ pfem_status pfem_batch_build_cells(pfem_ctx *ctx, const void *plan, int64_t N_to
  * workspace (pfem_batch_workspace_size with those totals) holds, after its 256-byte status
  * block, the fix-pass queue (8 bytes per node), the per-node records and the star table.
  * Quadratic shape functions then run as for one problem: the star table of every problem, a
- * persistent kernel that writes each node's record, a kernel that solves the edge systems,
- * and the fix pass over the queued nodes (FP64, SVD solve, widest search radius).  The
+ * persistent kernel that locates the nodes and solves the edge systems, and the fix pass over the queued nodes (FP64, SVD solve, widest search radius).  The
  * kernels compare the totals with the plan's own before writing anything and record
  * PFEM_ERR_INVALID_ARG (detail -1) when they differ.  With a smaller workspace (at least 256
  * bytes plus the queue) every node runs a fused per-node kernel; linear shape functions always

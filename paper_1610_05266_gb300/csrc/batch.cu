@@ -138,11 +138,12 @@ __global__ void __launch_bounds__(256) k_bin_batch(const BPlanDev *pl, const P *
 
 // ---------------------------------------------------------------- P2M
 
-// The plan and the caller's totals must agree before any record or table entry is written.
-__device__ __forceinline__ bool totals_ok(const BPlanDev *pl, const NodeRecs *r, const StarTab *t,
+// The plan and the caller's totals must agree before any table entry is written (nodes < 0: not
+// compared).
+__device__ __forceinline__ bool totals_ok(const BPlanDev *pl, long long nodes, const StarTab &t,
                                           DevStatus *st)
 {
-    const bool ok = (!r || r->nodes == pl->total_nodes) && (!t || t->N == pl->total_particles);
+    const bool ok = (nodes < 0 || nodes == pl->total_nodes) && t.N == pl->total_particles;
     if (!ok && blockIdx.x == 0 && threadIdx.x == 0) record_error(st, PFEM_ERR_INVALID_ARG, -1);
     return ok;
 }
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(BSTAR) k_star_list_batch(const BPlanDev *pl, P
     __shared__ int ss[STAR_KL * BSTAR];
     __shared__ unsigned char sord[STAR_KL * BSTAR];
     __shared__ unsigned char sstk[STAR_KL * BSTAR];
-    if (!totals_ok(pl, nullptr, &t, base.status)) return;
+    if (!totals_ok(pl, -1, t, base.status)) return;
     const long long *sp = plan_star_tiles(pl);
     for (long long b = blockIdx.x; b < pl->n_star_tiles; b += gridDim.x) {
         const int p = find_item(sp, pl->P, b);
@@ -230,48 +231,15 @@ __global__ void __launch_bounds__(64) k_star_retry_batch(const BPlanDev *pl, P2M
     }
 }
 
-// Node records of every problem in a persistent loop (the geometry half of the two-kernel
-// quadratic P2M): each node's record at its batch-wide index, with its coordinates.
-template <typename P, typename V, typename R>
-__global__ void __launch_bounds__(256, PFEM_GEOM_MIN_BLOCKS / 2) k_p2m_batch_geom(
-    const BPlanDev *pl, int shape_idx, P2MArgs base, unsigned long long *counter, StarTab tab,
-    NodeRecs r)
-{
-    __shared__ long long item;
-    if (!totals_ok(pl, &r, &tab, base.status)) return;
-    const int TY = blockDim.x / 16;
-    const long long total = pl->n_items[shape_idx];
-    const long long *tp = plan_tiles(pl, shape_idx);
-    for (int guard = 0; guard < (1 << 30); ++guard) {
-        __syncthreads();
-        if (threadIdx.x == 0) item = (long long)atomicAdd(counter, 1ull);
-        __syncthreads();
-        const long long it = item;
-        if (it >= total) break;
-        const int p = find_item(tp, pl->P, it);
-        const BDesc d = plan_desc(pl)[p];
-        const long long t = it - tp[p];
-        const int tiles_x = (d.n + 15) / 16;
-        const int I = (int)(t % tiles_x) * 16 + (threadIdx.x & 15);
-        const int J = (int)(t / tiles_x) * TY + (threadIdx.x >> 4);
-        if (I >= d.n || J >= d.n) continue;
-        const long long rec = d.noff + (long long)J * d.n + I;
-        if (rec >= r.nodes) continue;
-        P2MArgs a;
-        problem_args(a, base, d);
-        problem_out<V>(a, base, d);
-        geom_node<P, V, R>(a, tab, r, I, J, rec);
-    }
-}
-
 // The table path's fast pass of every problem in one persistent kernel (as k_p2m_tab: location
 // from the star table, edge solves and apply per node, no node records).
 template <typename P, typename V, typename R, typename S, int REFINE>
-__global__ void __launch_bounds__(256, tab_min_blocks<S, REFINE>() / 2) k_p2m_batch_tab(
-    const BPlanDev *pl, int shape_idx, P2MArgs base, unsigned long long *counter, StarTab tab)
+__global__ void __launch_bounds__(256, tab_min_blocks<S>() / 2) k_p2m_batch_tab(
+    const BPlanDev *pl, int shape_idx, P2MArgs base, unsigned long long *counter, StarTab tab,
+    long long nodes)
 {
     __shared__ long long item;
-    if (!totals_ok(pl, nullptr, &tab, base.status)) return;
+    if (!totals_ok(pl, nodes, tab, base.status)) return;
     const int TY = blockDim.x / 16;
     const long long total = pl->n_items[shape_idx];
     const long long *tp = plan_tiles(pl, shape_idx);
@@ -436,7 +404,7 @@ cudaError_t launch_batch_build_cells(const void *plan, long long Ntot, long long
 
 // Workspace of the batched P2M: status (byte 0), work counter (byte 64), fix-pass queue counter
 // (byte 128), star-table queue counter (byte 132); the fix-pass queue from byte 256 (8 bytes per
-// node), then the node records (with the nodes' coordinates) and the star table.
+// node), then a record's space per node and the star table.
 static size_t al256b(size_t x) { return (x + 255) & ~(size_t)255; }
 
 size_t batch_p2m_ws_bytes(long long nodes_total, long long N_total)
@@ -447,8 +415,8 @@ size_t batch_p2m_ws_bytes(long long nodes_total, long long N_total)
 }
 
 struct BatchWs {
-    NodeRecs recs;
     StarTab tab;
+    long long nodes;            // the total that the fast pass compares with the plan's, or -1
     bool table;
 };
 
@@ -465,16 +433,9 @@ static cudaError_t p2m_batch_t(const void *plan, const P2MArgs &base, int shape_
         k_star_list_batch<<<num_sms() * 8, BSTAR, 0, s>>>(pl, base, w.tab);
         k_star_retry_batch<true><<<num_sms() * PFEM_RETRY_BLOCKS, 64, 0, s>>>(pl, base, w.tab);
         k_star_retry_batch<false><<<num_sms() * PFEM_RETRY_REGION_BLOCKS, 64, 0, s>>>(pl, base, w.tab);
-        if (REF != REFINE_FF) {      // one kernel, as the single-problem table path
-            k_p2m_batch_tab<P, V, R, S, REF><<<blocks, 16 * TYs[shape_idx], 0, s>>>(
-                pl, shape_idx, base, counter, w.tab);
-            count_launch(4);
-        } else {
-            k_p2m_batch_geom<P, V, R><<<blocks, 16 * TYs[shape_idx], 0, s>>>(pl, shape_idx, base,
-                                                                          counter, w.tab, w.recs);
-            k_p2m_solve<P, V, R, S, REF><<<(unsigned)((w.recs.nodes + 127) / 128), 128, 0, s>>>(base, w.recs);
-            count_launch(5);
-        }
+        k_p2m_batch_tab<P, V, R, S, REF><<<blocks, 16 * TYs[shape_idx], 0, s>>>(
+            pl, shape_idx, base, counter, w.tab, w.nodes);
+        count_launch(4);
     } else {
         k_p2m_batch<P, V, R, S, REF, SHAPE><<<blocks, 16 * TYs[shape_idx], 0, s>>>(
             pl, shape_idx, base, counter);
@@ -495,8 +456,7 @@ static cudaError_t p2m_batch_solve(pfem_solve solve, const void *plan, const P2M
     switch (solve) {
     case PFEM_SOLVE_F64: return p2m_batch_t<P, V, float, double, REFINE_NONE, SHAPE>(plan, a, shape_idx, blocks, counter, w, s);
     case PFEM_SOLVE_F32: return p2m_batch_t<P, V, float, float, REFINE_NONE, SHAPE>(plan, a, shape_idx, blocks, counter, w, s);
-    case PFEM_SOLVE_F32_REFINED: return p2m_batch_t<P, V, float, float, REFINE_F64, SHAPE>(plan, a, shape_idx, blocks, counter, w, s);
-    default: return p2m_batch_t<P, V, float, float, REFINE_FF, SHAPE>(plan, a, shape_idx, blocks, counter, w, s);
+    default: return p2m_batch_t<P, V, float, float, REFINE_FIX, SHAPE>(plan, a, shape_idx, blocks, counter, w, s);   // both refined solves
     }
 }
 
@@ -533,9 +493,11 @@ cudaError_t launch_batch_p2m(const void *plan, const void *pos_sorted, const uin
     a.defer_list = a.defer_cap > 0 ? (long long *)(W + 256) : nullptr;
     if (w.table) {
         char *base = W + al256b(256 + 8 * (size_t)nodes_total);
-        const size_t rb = al256b(node_recs_layout(base, nodes_total, &w.recs, true));
+        NodeRecs r;
+        const size_t rb = al256b(node_recs_layout(nullptr, nodes_total, &r, true));
         w.tab = star_tab_layout(base + rb, N_total, (int *)(W + 132));
     }
+    w.nodes = solve == PFEM_SOLVE_F32_REFINED_FF ? nodes_total : -1;
     unsigned long long *counter = (unsigned long long *)(W + 64);
     const bool q = shape == PFEM_SHAPE_QUADRATIC;
     if (val_t == PFEM_F64) {

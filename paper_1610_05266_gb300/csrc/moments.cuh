@@ -86,57 +86,6 @@ template <typename S> struct Moment {
     }
 };
 
-// ----------------------------------------------------------------- float-float arithmetic
-// An unevaluated sum hi + lo of two FP32 numbers (about 48 significant bits), built from the
-// error-free transformations of Dekker (1971) and Knuth (TAOCP vol. 2, 4.2.2): the FP32 sum and
-// product of two floats are exact once their rounding error is carried along.  Used for the
-// residual of the refined FP32 solve, which must be formed in about twice the working
-// precision; on sm_103a FP32 instructions issue at 64 times the rate of FP64 ones.
-struct FF {
-    float h, l;
-};
-
-__device__ __forceinline__ FF ff_two_sum(float a, float b)
-{
-    const float s = a + b;
-    const float bb = s - a;
-    return {s, (a - (s - bb)) + (b - bb)};
-}
-
-__device__ __forceinline__ FF ff_two_prod(float a, float b)
-{
-    const float p = a * b;
-    return {p, fmaf(a, b, -p)};
-}
-
-__device__ __forceinline__ FF ff_norm(float h, float l)
-{
-    const float s = h + l;
-    return {s, l - (s - h)};
-}
-
-__device__ __forceinline__ FF ff_add(FF a, FF b)
-{
-    const FF s = ff_two_sum(a.h, b.h);
-    return ff_norm(s.h, s.l + (a.l + b.l));
-}
-
-// (a.h + a.l) * b for a float b
-__device__ __forceinline__ FF ff_mul(FF a, float b)
-{
-    const FF p = ff_two_prod(a.h, b);
-    return ff_norm(p.h, fmaf(a.l, b, p.l));
-}
-
-// (a.h + a.l) * (b.h + b.l)
-__device__ __forceinline__ FF ff_mul(FF a, FF b)
-{
-    const FF p = ff_two_prod(a.h, b.h);
-    return ff_norm(p.h, fmaf(a.h, b.l, fmaf(a.l, b.h, p.l)));
-}
-
-__device__ __forceinline__ FF ff_neg(FF a) { return {-a.h, -a.l}; }
-
 // Exact FP32 -> FP64 widening by integer operations on the bit patterns (sign; exponent
 // rebiased by 1023 - 127 = 896; the 23 mantissa bits at the top of the 52).  FP32 subnormals
 // (below 1.2e-38) become zero.  On sm_103a the format conversion instructions share the
@@ -161,9 +110,106 @@ __device__ __forceinline__ float f32_trunc(double d)
     return e > 0 ? __uint_as_float(u) : 0.0f;
 }
 
-// Refinement of the FP32 moment solve: 0 = none, 1 = residual in FP64, 2 = residual in
-// float-float.
-enum { REFINE_NONE = 0, REFINE_F64 = 1, REFINE_FF = 2 };
+// Refinement of the FP32 moment solve: none, or one step with the residual r = b - M y in 64-bit
+// fixed point (FixRes).
+enum { REFINE_NONE = 0, REFINE_FIX = 1 };
+
+// ----------------------------------------------------------------- fixed-point residual
+// The residual r = b - sum_mu p_mu (p_mu . y) of one edge system on the integer pipes.
+//
+// An SM of GB300 issues two FP64 instructions a clock: one FP64 instruction of a warp holds its
+// scheduler's FP64 pipe for 64 cycles, and in FP64 this residual takes 13 of them a stencil point
+// and edge (832 cycles).  Here it takes about 45 integer instructions.  Everything is scaled by
+// powers of two, so the scaling is exact:
+//  - coordinates X = x / g in Q32, |X| < 1/2, g = 2^k from the largest |x|, |y| of the stencil.
+//    A coordinate down to 2^-8 of the largest keeps all 24 bits of its FP32 value; smaller ones
+//    are rounded at 2^-33 g, far below the rounding of the FP32 offsets themselves;
+//  - the solution in the scaled monomials, y'_k = y_k g^deg(k), as 30-bit integers relative to
+//    the largest of |y'| and |b'|.  y is an approximate solution: the refinement corrects the
+//    one it is given, and rounding it to this grid leaves values that FP32 represents;
+//  - t = p . y, X t, Y t and the six sums as 64-bit integers with unit 2^-61 of that largest
+//    value.  |t| <= 1 + 2/2 + 3/4 = 2.75 of it, so products do not overflow; the sums may wrap, which
+//    two's complement undoes since the residual itself is small (the FP32 Cholesky solve is
+//    backward stable).
+// A product drops bits below 2^-61, where FP64 rounds t, X t, Y t and every partial sum to 53
+// bits, and the sums are exact: measured against 64-bit arithmetic the projection's error is the
+// FP64 residual's (see k_p2m_tab).
+struct FixRes {
+    float sx, gi;               // 2^32 / g and 1 / g
+    int bm;                     // biased exponent: |y'|, |b'| < 2^(bm - 126)
+    int Y[6];
+    long long r[6];
+
+    // 2^e for -126 <= e <= 127
+    static __device__ __forceinline__ float pow2(int e) { return __int_as_float((e + 127) << 23); }
+
+    // ext: the stencil's largest |x|, |y|; y is rounded to the grid.  False when the system is
+    // beyond the scaling's range (extent 2^40 edge lengths and more).
+    __device__ __forceinline__ bool init(float ext, const float b[6], float y[6])
+    {
+        const int be = (int)(__float_as_uint(ext) >> 23);       // ext < 2^(be - 126)
+        if (be < 96 || be > 166) return false;
+        gi = pow2(125 - be);
+        sx = pow2(157 - be);
+        const float g = pow2(be - 125), g2 = g * g, gi2 = gi * gi;
+        const float s[6] = {1.f, g, g, g2, g2, g2}, si[6] = {1.f, gi, gi, gi2, gi2, gi2};
+        float ym = 0.f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) ym = fmaxf(ym, fmaxf(fabsf(y[k] * s[k]), fabsf(b[k] * si[k])));
+        bm = (int)(__float_as_uint(ym) >> 23);
+        if (bm < 30 || bm > 250) return false;
+        const float sy = pow2(155 - bm), us = pow2(bm - 155);
+        const float sb = pow2(61), ub = pow2(126 - bm);         // b' 2^(187 - bm)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            Y[k] = __float2int_rn(y[k] * s[k] * sy);            // |Y| <= 2^29
+            y[k] = (float)Y[k] * us * si[k];
+            r[k] = k < 3 ? 0 : __float2ll_rn(b[k] * si[k] * ub * sb);
+        }
+        return true;
+    }
+
+    // (a * u) >> 32 with u = uh 2^32 + ul, ul signed
+    struct Split {
+        int h, l;
+    };
+    static __device__ __forceinline__ Split split(long long u)
+    {
+        const int l = (int)u;
+        return {(int)(u >> 32) + (int)((unsigned)l >> 31), l};
+    }
+    static __device__ __forceinline__ long long mul(int a, Split u)
+    {
+        return (long long)a * u.h + __mulhi(a, u.l);
+    }
+
+    // r -= p (p . y) for the point at (x, y)
+    __device__ __forceinline__ void point(float x, float y)
+    {
+        const int X = __float2int_rn(x * sx), Z = __float2int_rn(y * sx);
+        const Split u = split(((long long)Y[1] << 32) + (long long)X * Y[3] + (long long)Z * Y[4]);
+        const Split v = split(((long long)Y[2] << 32) + (long long)Z * Y[5]);
+        const long long t = ((long long)Y[0] << 32) + mul(X, u) + mul(Z, v);
+        const Split ts = split(t);
+        const long long xt = mul(X, ts), zt = mul(Z, ts);
+        const Split xs = split(xt), zs = split(zt);
+        r[0] -= t;
+        r[1] -= xt;
+        r[2] -= zt;
+        r[3] -= mul(X, xs);
+        r[4] -= mul(Z, xs);
+        r[5] -= mul(Z, zs);
+    }
+
+    // the residual in the edge frame's units
+    __device__ __forceinline__ void result(float out[6]) const
+    {
+        const float g = 1.f / gi, g2 = g * g, u = pow2(bm - 126), w = pow2(-61);
+        const float s[6] = {1.f, g, g, g2, g2, g2};
+#pragma unroll
+        for (int k = 0; k < 6; ++k) out[k] = __ll2float_rn(r[k]) * w * u * s[k];
+    }
+};
 
 template <typename S> struct SolveTol;
 template <> struct SolveTol<double> { static constexpr double v = 1e-13; };

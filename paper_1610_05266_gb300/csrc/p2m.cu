@@ -47,14 +47,6 @@ static P2MArgs make_args(const GeoArgs &g, DevStatus *st)
 
 static dim3 node_grid(int n) { return dim3((n + 15) / 16, (n + 7) / 8); }
 
-// The table path's fast pass as one kernel (k_p2m_tab) or as the geometry and solve kernels with
-// node records in between.  Measured at 1025^2 nodes / 2048^2 particles (geometry + solve):
-// FP64-residual refinement 1.21 -> 1.07 ms fused, plain FP32 0.58 -> 0.53 ms, float-float
-// refinement 0.84 -> 0.89 ms; the float-float solve keeps the two kernels.
-#ifndef PFEM_P2M_FUSED_TAB
-#define PFEM_P2M_FUSED_TAB 1
-#endif
-
 template <typename P, typename V, typename R, typename S, int REF, int SHAPE, bool W>
 static cudaError_t go_fast(const P2MArgs &a, cudaStream_t s)
 {
@@ -67,7 +59,7 @@ static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Workspace layout of P2M after the 256-byte status block: the fix-pass queue counter at byte
 // 256 and the star-table queue counter at byte 260, the fix-pass queue from byte 512 (8 bytes
-// per node), then the node records and the star table of the table path.
+// per node), then a record's space per node (the adjoint's layout) and the star table.
 static size_t recs_offset(long long nodes) { return al256(512 + 8 * (size_t)nodes); }
 
 size_t p2m_ws_bytes(long long nodes, long long N)
@@ -78,27 +70,25 @@ size_t p2m_ws_bytes(long long nodes, long long N)
 }
 
 // Records and star table in ws, when it has room for them.
-static bool set_table(NodeRecs &r, StarTab &t, void *ws, size_t ws_bytes, long long nodes,
-                      long long N)
+static bool set_table(StarTab &t, void *ws, size_t ws_bytes, long long nodes, long long N)
 {
     if (ws_bytes < p2m_ws_bytes(nodes, N)) return false;
     char *base = (char *)ws + recs_offset(nodes);
-    const size_t recs = al256(node_recs_layout(base, nodes, &r));
+    NodeRecs r;
+    const size_t recs = al256(node_recs_layout(nullptr, nodes, &r));
     t = star_tab_layout(base + recs, N, (int *)((char *)ws + 260));
     return true;
 }
 
 // P2M: the fast pass over all nodes, then the fix pass over the nodes it queued.  With quadratic
 // shape functions, the apply form and room for the table, the fast pass is the star table and
-// then k_p2m_tab (location, edge solves and apply per node), or, for the float-float solve, the
-// geometry kernel (node records) and the solve kernel; otherwise one kernel that searches the
+// then k_p2m_tab (location, edge solves and apply per node); otherwise one kernel that searches the
 // stars per node.
 // Stage events (when the caller's context has them): 0 before the fast pass, 1 after the star
-// table, 2 after the geometry kernel (right before k_p2m_tab), 3 after the solve kernel (after
-// k_p2m_tab), 4 after the fix pass.
+// table, 2 right before k_p2m_tab, 3 after it, 4 after the fix pass.
 template <typename P, typename V, typename R, typename S, int REF, int SHAPE, bool W>
 static cudaError_t go(const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
-                      const NodeRecs *rec = nullptr, const StarTab *tab = nullptr)
+                      const StarTab *tab = nullptr)
 {
     const int R0 = g.R0, rmax_far = g.rmax_far;
     cudaError_t e;
@@ -107,36 +97,17 @@ static cudaError_t go(const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
         e = cudaMemsetAsync(a.defer_count, 0, sizeof(int), s);
         if (e != cudaSuccess) return e;
     }
-    if (SHAPE == PFEM_SHAPE_QUADRATIC && !W && rec && tab) {
+    if (SHAPE == PFEM_SHAPE_QUADRATIC && !W && tab) {
         e = launch_star_table(a.B, R0, rmax_far, *tab, a.status, s);
         if (e != cudaSuccess) return e;
         stage_event(g, 1, s);
-#if PFEM_P2M_FUSED_TAB
-        if (!W && REF != REFINE_FF) {
-            stage_event(g, 2, s);
-            e = wait_values(g, s);
-            if (e != cudaSuccess) return e;
-            k_p2m_tab<P, V, R, S, REF><<<node_grid(a.n), 128, 0, s>>>(a, *tab);
-            count_launch();
-            e = cudaGetLastError();
-            stage_event(g, 3, s);
-        } else
-#endif
-        {
-        k_p2m_geom<P, V, R><<<node_grid(a.n), 128, 0, s>>>(a, *tab, *rec);
-        count_launch();
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
         stage_event(g, 2, s);
-        if (!W) {
-            e = wait_values(g, s);
-            if (e != cudaSuccess) return e;
-        }
-        k_p2m_solve<P, V, R, S, REF><<<(unsigned)((rec->nodes + 127) / 128), 128, 0, s>>>(a, *rec);
+        e = wait_values(g, s);
+        if (e != cudaSuccess) return e;
+        k_p2m_tab<P, V, R, S, REF><<<node_grid(a.n), 128, 0, s>>>(a, *tab);
         count_launch();
         e = cudaGetLastError();
         stage_event(g, 3, s);
-        }
     } else {
         if (!W) {
             e = wait_values(g, s);
@@ -147,7 +118,7 @@ static cudaError_t go(const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
     if (e != cudaSuccess || a.defer_cap <= 0) return e;
     P2MArgs f = a;
     f.B.rmax = rmax_far > a.B.rmax ? rmax_far : a.B.rmax;
-    if (SHAPE == PFEM_SHAPE_QUADRATIC && !W && rec && tab)
+    if (SHAPE == PFEM_SHAPE_QUADRATIC && !W && tab)
         k_p2m_fix_tab<P, V, R, sizeof(S) == 4><<<num_sms(), 128, 0, s>>>(f, *tab);
     else
         k_p2m_fix<P, V, R, SHAPE, W><<<num_sms(), 128, 0, s>>>(f);
@@ -159,13 +130,12 @@ static cudaError_t go(const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
 // Compute type S and refinement of each solve for FP32 arithmetic.
 template <typename P, typename V, int SHAPE, bool W>
 static cudaError_t go_solve(pfem_solve solve, const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
-                            const NodeRecs *r, const StarTab *t)
+                            const StarTab *t)
 {
     switch (solve) {
-    case PFEM_SOLVE_F64: return go<P, V, float, double, REFINE_NONE, SHAPE, W>(g, a, s, r, t);
-    case PFEM_SOLVE_F32: return go<P, V, float, float, REFINE_NONE, SHAPE, W>(g, a, s, r, t);
-    case PFEM_SOLVE_F32_REFINED: return go<P, V, float, float, REFINE_F64, SHAPE, W>(g, a, s, r, t);
-    default: return go<P, V, float, float, REFINE_FF, SHAPE, W>(g, a, s, r, t);
+    case PFEM_SOLVE_F64: return go<P, V, float, double, REFINE_NONE, SHAPE, W>(g, a, s, t);
+    case PFEM_SOLVE_F32: return go<P, V, float, float, REFINE_NONE, SHAPE, W>(g, a, s, t);
+    default: return go<P, V, float, float, REFINE_FIX, SHAPE, W>(g, a, s, t);   // both refined solves
     }
 }
 
@@ -180,21 +150,18 @@ cudaError_t launch_p2m(const GeoArgs &g, const int *perm, int C, const void *val
     a.C = C;
     a.out = out;
     const bool q = shape == PFEM_SHAPE_QUADRATIC;
-    NodeRecs recs;
     StarTab tab;
-    const bool table = set_table(recs, tab, st, ws_bytes, (long long)g.n * g.n, g.N);
-    const NodeRecs *r = table ? &recs : nullptr;
-    const StarTab *t = table ? &tab : nullptr;
+    const StarTab *t = set_table(tab, st, ws_bytes, (long long)g.n * g.n, g.N) ? &tab : nullptr;
     if (val_t == PFEM_F64) {   // positions FP64, arithmetic FP64
         if (!q) return go<double, double, double, double, REFINE_NONE, 0, false>(g, a, s);
-        return go<double, double, double, double, REFINE_NONE, 1, false>(g, a, s, r, t);
+        return go<double, double, double, double, REFINE_NONE, 1, false>(g, a, s, t);
     }
     if (val_t == PFEM_F32) {   // positions FP32, arithmetic FP32
         if (!q) return go<float, float, float, float, REFINE_NONE, 0, false>(g, a, s);
-        return go_solve<float, float, 1, false>(solve, g, a, s, r, t);
+        return go_solve<float, float, 1, false>(solve, g, a, s, t);
     }
     if (!q) return go<float, __nv_bfloat16, float, float, REFINE_NONE, 0, false>(g, a, s);
-    return go_solve<float, __nv_bfloat16, 1, false>(solve, g, a, s, r, t);
+    return go_solve<float, __nv_bfloat16, 1, false>(solve, g, a, s, t);
 }
 
 cudaError_t launch_shape(const GeoArgs &g, pfem_shape shape, pfem_solve solve, int K, int *w_idx,
@@ -211,7 +178,7 @@ cudaError_t launch_shape(const GeoArgs &g, pfem_shape shape, pfem_solve solve, i
         return go<double, double, double, double, REFINE_NONE, 1, true>(g, a, s);
     }
     if (!q) return go<float, float, float, float, REFINE_NONE, 0, true>(g, a, s);
-    return go_solve<float, float, 1, true>(solve, g, a, s, nullptr, nullptr);
+    return go_solve<float, float, 1, true>(solve, g, a, s, nullptr);
 }
 
 // alpha_i = sum_k w[i,k] alpha[w_idx[i,k]] (explicit-weight P2M)

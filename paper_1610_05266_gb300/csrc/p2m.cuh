@@ -485,70 +485,31 @@ __device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R
         }
         Moment<S> M;
         M.zero();
+        S ext = S(0);                   // largest coordinate, for the residual's scale
         for (unsigned m = mask; m; m &= m - 1) {
             const int i = __ffs(m) - 1;
             S ox, oy;
             offset(i, ox, oy);
-            M.add((ox - mx) * inv, (oy - my) * inv);
+            const S x = (ox - mx) * inv, yv = (oy - my) * inv;
+            M.add(x, yv);
+            if (REFINE != REFINE_NONE) ext = fmax(ext, fmax(fabs(x), fabs(yv)));
         }
         if (!M.factor(FastTol<S>::v)) return -PFEM_DEFER;
         const S tx = ex * inv, ty = ey * inv;
         const S b[6] = {S(0), S(0), S(0), S(-0.5) * tx * tx, S(-0.5) * tx * ty, S(-0.5) * ty * ty};
         S y[6];
         M.solve(b, y);
-        if constexpr (REFINE == REFINE_FF) {
-            // r = b - sum_mu p_mu (p_mu . y) in float-float, with the monomials of the FP32
-            // offsets formed exactly (the same system the FP64 residual refines)
-            FF r[6];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) r[k] = {(float)b[k], 0.f};
+        if constexpr (REFINE == REFINE_FIX) {
+            FixRes fr;
+            if (!fr.init(ext, b, y)) return -PFEM_DEFER;
             for (unsigned m = mask; m; m &= m - 1) {
                 const int i = __ffs(m) - 1;
                 S ox, oy;
                 offset(i, ox, oy);
-                const float X = (float)((ox - mx) * inv), Y = (float)((oy - my) * inv);
-                const FF p[6] = {{1.f, 0.f}, {X, 0.f}, {Y, 0.f}, ff_two_prod(X, X),
-                                 ff_two_prod(X, Y), ff_two_prod(Y, Y)};
-                FF t = {(float)y[0], 0.f};
-#pragma unroll
-                for (int k = 1; k < 6; ++k) t = ff_add(t, ff_mul(p[k], (float)y[k]));
-#pragma unroll
-                for (int k = 0; k < 6; ++k) r[k] = ff_add(r[k], ff_neg(ff_mul(p[k], t)));
+                fr.point((ox - mx) * inv, (oy - my) * inv);
             }
             S rs[6], dy[6];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) rs[k] = (S)(r[k].h + r[k].l);
-            M.solve(rs, dy);
-#pragma unroll
-            for (int k = 0; k < 6; ++k) y[k] += dy[k];
-        }
-        if constexpr (REFINE == REFINE_F64) {
-            // r = b - sum_mu p_mu (p_mu . y) in FP64: t = p . y by nested products, and the
-            // monomial terms of r as X (X t), Y (X t), Y (Y t)
-            double r[6], yd[6];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                r[k] = f64_of(b[k]);
-                yd[k] = f64_of(y[k]);
-            }
-            for (unsigned m = mask; m; m &= m - 1) {
-                const int i = __ffs(m) - 1;
-                S ox, oy;
-                offset(i, ox, oy);
-                const double X = f64_of((ox - mx) * inv), Y = f64_of((oy - my) * inv);
-                const double t = fma(X, fma(X, yd[3], fma(Y, yd[4], yd[1])),
-                                     fma(Y, fma(Y, yd[5], yd[2]), yd[0]));
-                const double xt = X * t, yt = Y * t;
-                r[0] -= t;
-                r[1] -= xt;
-                r[2] -= yt;
-                r[3] = fma(-X, xt, r[3]);
-                r[4] = fma(-Y, xt, r[4]);
-                r[5] = fma(-Y, yt, r[5]);
-            }
-            S rs[6], dy[6];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) rs[k] = f32_trunc(r[k]);
+            fr.result(rs);
             M.solve(rs, dy);
 #pragma unroll
             for (int k = 0; k < 6; ++k) y[k] += dy[k];
@@ -724,12 +685,11 @@ __global__ void __launch_bounds__(128) k_p2m_fix(P2MArgs a)
     }
 }
 
-// ---------------------------------------------------------------- two-kernel P2M
-// The table path as two kernels, each with its own register budget: k_p2m_geom locates the node
-// and builds its particle set from the star table (memory latency bound), k_p2m_solve solves the
-// three edge systems and applies the weights.  They hand over a per-node record, one array per
-// field so that both kernels access it coalesced.  The float-float solve and the adjoint take
-// this form; the other forward solves run both halves in k_p2m_tab.
+// ---------------------------------------------------------------- node records
+// The adjoint runs the table path as two kernels, each with its own register budget: k_p2m_geom
+// locates the node and builds its particle set from the star table (memory latency bound), and
+// the adjoint's solve kernel reads what it found from a per-node record, one array per field so
+// that both kernels access it coalesced.  The forward solves run both halves in k_p2m_tab.
 struct NodeRecs {
     int *meta;          // [nodes] nu | vi0 << 5 | vi1 << 10 | vi2 << 15, or -1: no record
     unsigned *mask;     // [3][nodes] vm[e]
@@ -894,88 +854,19 @@ __global__ void __launch_bounds__(128) k_p2m_fix_tab(P2MArgs a, StarTab t)
     }
 }
 
-// Resident 128-thread blocks per SM of the solve kernel (the two-kernel form: the float-float
-// refinement): 8 (64 registers) for the FP32 moment system (sweep 8, 10, 12: 8), and 8 as well
-// for the refined solves with the edge loop rolled (float-float: 6 -> 8 blocks 0.553 -> 0.536
-// ms at 1025^2 nodes / 2048^2 particles).  A refined solve needs many warps in flight to keep
-// the FP64 pipe busy: one to three persistent blocks per SM measured 1.1 to 2.4 times slower.
-#ifndef PFEM_SOLVE_MIN_BLOCKS
-#define PFEM_SOLVE_MIN_BLOCKS 8
-#endif
-#ifndef PFEM_SOLVE_REF_MIN_BLOCKS
-#define PFEM_SOLVE_REF_MIN_BLOCKS 8
-#endif
-template <typename S, int REFINE> constexpr int solve_min_blocks()
-{
-    return sizeof(S) == 8 ? 4 : REFINE != REFINE_NONE ? PFEM_SOLVE_REF_MIN_BLOCKS : PFEM_SOLVE_MIN_BLOCKS;
-}
-
-template <typename P, typename V, typename R, typename S, int REFINE>
-__global__ void __launch_bounds__(128, solve_min_blocks<S, REFINE>()) k_p2m_solve(P2MArgs a, NodeRecs r)
-{
-    const long long node = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (node >= r.nodes) return;
-    const int meta = r.meta[node];
-    if (meta < 0) return;
-    const int nu = meta & 31;
-    const int vi[3] = {(meta >> 5) & 31, (meta >> 10) & 31, (meta >> 15) & 31};
-    int us[UMAX];
-    R uw[UMAX];
-    for (int i = 0; i < nu; ++i) {
-        us[i] = r.us[i * r.nodes + node];
-        uw[i] = R(0);
-    }
-    unsigned vm[3];
-    R lam[3];
-#pragma unroll
-    for (int e = 0; e < 3; ++e) {
-        vm[e] = r.mask[e * r.nodes + node];
-        lam[e] = (R)r.lam[e * r.nodes + node];
-        uw[vi[e]] += lam[e];
-    }
-    NodePos<P, R> np;
-    if (r.loc) {                        // batch: the node's own mesh, output at its record index
-        const long long l = r.loc[node];
-        np.init((int)(l & 0x1fffff), (int)((l >> 21) & 0x1fffff), (int)(l >> 42));
-    } else {
-        const int nc = a.n - 1;
-        const int I = (int)(node % a.n), J = (int)(node / a.n);
-        np.init(I == nc ? 0 : I, J == nc ? 0 : J, nc);
-    }
-    int st = node_u_solve<P, R, S, REFINE, false, UMAX>(a, np, us, uw, vm, vi, lam);
-    R acc[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] = R(0);
-    if (st == 0) {
-        for (int i = 0; i < nu; ++i) {
-            R v[8];
-            load_vals<V, R>((const V *)a.vals, a.perm, us[i], a.C, v);
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < a.C) acc[c] = fma(uw[i], v[c], acc[c]);
-        }
-    } else {
-        st = defer_or_error(a, st, node);
-        if (st < 0) record_error(a.status, -st, node);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[c] = (R)nan_of<R>();
-    }
-    store_vals<V, R>((V *)a.out, node, a.C, acc);
-}
-
 // The table path's fast pass in one kernel: each thread locates its node with the star table,
 // builds its particle set and solves its three edge systems, without a node record in between.
-// The refined solve is bound by the FP64 pipe, which leaves the other pipes and the memory
-// system to the location work of the other warps.
-// Resident blocks per SM of k_p2m_tab with the refined solve: 8 (64 registers; with the edge
-// loop rolled 6, 7, 8 measured 1.051, 1.011, 1.000 ms at 1025^2 nodes / 2048^2 particles).
-#ifndef PFEM_TAB_REF_MIN_BLOCKS
-#define PFEM_TAB_REF_MIN_BLOCKS 8
+// The refined solve's residual runs on the integer pipes (FixRes); in FP64 it held the FP64 pipe
+// for 0.47 ms of this kernel's 0.99 ms at 1025^2 nodes / 2048^2 particles, C = 4, FP32 (now 0.67
+// ms; 4097^2 / 8192^2: 14.6 -> 9.6 ms).  Errors against 64-bit arithmetic are unchanged (1.1e-7
+// of the mesh's 2-norm; the two results differ by 1e-9 of it).  The float-float refinement that
+// PFEM_SOLVE_F32_REFINED_FF names (48 bits, about 200 FP32 instructions a point and edge) took
+// 0.84 ms in two kernels; it takes this path too, whose residual is the more exact.
+// Resident blocks per SM: 8 (64 registers).
+#ifndef PFEM_TAB_MIN_BLOCKS
+#define PFEM_TAB_MIN_BLOCKS 8
 #endif
-template <typename S, int REFINE> constexpr int tab_min_blocks()
-{
-    return sizeof(S) == 8 || REFINE == REFINE_NONE ? solve_min_blocks<S, REFINE>() : PFEM_TAB_REF_MIN_BLOCKS;
-}
+template <typename S> constexpr int tab_min_blocks() { return sizeof(S) == 8 ? 4 : PFEM_TAB_MIN_BLOCKS; }
 
 // Node (I, J) of the problem of a (mesh output a.out; queue entries and error details at node
 // a.noff + J * a.n + I of the batch).
@@ -1035,7 +926,7 @@ __device__ __forceinline__ void tab_node(const P2MArgs &a, const StarTab &t, int
 }
 
 template <typename P, typename V, typename R, typename S, int REFINE>
-__global__ void __launch_bounds__(128, tab_min_blocks<S, REFINE>()) k_p2m_tab(P2MArgs a, StarTab t)
+__global__ void __launch_bounds__(128, tab_min_blocks<S>()) k_p2m_tab(P2MArgs a, StarTab t)
 {
     const int I = blockIdx.x * 16 + (threadIdx.x & 15);
     const int J = blockIdx.y * 8 + (threadIdx.x >> 4);

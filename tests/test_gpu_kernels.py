@@ -1,0 +1,55 @@
+"""Kernel variants and dispatch rules at the sizes where they could go wrong, against the FP64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from workloads import generators as G
+
+pytestmark = pytest.mark.gpu
+
+# FP32: the storage rounding of a value, at most 24 products and sums of a node and the rounding of
+# their weights, each 2^-24 of the largest value times the weights' sum of magnitudes (below 1.3)
+TOL32 = 2e-6
+TOL64 = 1e-12
+
+
+@pytest.fixture(scope="module")
+def P():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1610_05266_gb300 as P
+    return P
+
+
+def relerr(a, b):
+    a, b = np.asarray(a, np.float64), np.asarray(b, np.float64)
+    return np.abs(a - b).max() / max(np.abs(b).max(), 1e-300)
+
+
+def uniform(n, m, seed):
+    pos = G.uniform01(G.SEED_BASE + seed, 2 * m * m).reshape(m * m, 2)
+    return G.Problem("uniform", n, m, 0.0, 0, pos, G.taylor_green(pos))
+
+
+PROBLEMS = {"tiny": lambda: G.config_tiny(), "odd": lambda: G.scaled_config("tg", 38, 91, 0.3),
+            "coarse": lambda: G.scaled_config("tg", 41, 40, 0.3), "dense": lambda: G.scaled_config("tg", 33, 128),
+            "uniform": lambda: uniform(65, 256, 900)}
+
+
+@pytest.mark.parametrize("which", sorted(PROBLEMS))
+def test_refined_solves(P, which):
+    """Both refined solves form the residual in 64-bit fixed point: the same mesh bit for bit, within
+    the FP32 bound of the oracle, on lattices of one to sixteen particles per node and on uniform
+    random particles (long thin stencils, ill-conditioned systems)."""
+    pr = PROBLEMS[which]()
+    pos = torch.tensor(pr.pos, dtype=torch.float32, device="cuda")
+    vals = torch.tensor(pr.vals, dtype=torch.float32, device="cuda")
+    proj = P.Projector(pr.n, pr.N, C=pr.C, pos_dtype=torch.float32)
+    proj.build(pos)
+    a = proj.p2m(vals, solve=P.PFEM_SOLVE_F32_REFINED)
+    b = proj.p2m(vals, solve=P.PFEM_SOLVE_F32_REFINED_FF)
+    proj.check()
+    assert torch.equal(a, b)
+    ref = O.p2m(pr.n, pos.double().cpu().numpy(), vals.double().cpu().numpy(), shape=1, nthreads=8)
+    assert relerr(a.cpu().numpy(), ref) <= TOL32
