@@ -9,6 +9,7 @@
 // Because the image row and column are stored, i+1 and j+1 never wrap.  The kernel is a
 // bandwidth-bound gather: positions and outputs stream once; the mesh is read through L2.
 #include <cmath>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -223,21 +224,40 @@ cudaError_t launch_m2p_backward(int n, int nb, long long N, const void *pos, pfe
 // coefficients once, Sec. 3.1).  With every cell split along (i,j)->(i+1,j+1), node (I,J) has
 // neighbours (I+-1,J), (I,J+-1), (I+1,J+1), (I-1,J-1); an edge's stencil is the closed
 // neighbourhood of both endpoints (10 nodes) and its minimum-norm coefficients depend only
-// on the edge's direction.  For each of the two triangles of a cell the host folds the three
-// edges into one table: the distinct stencil nodes (offsets from the cell corner), the
-// coefficient of each node in each edge, and which nodes are the triangle's vertices.  Then
+// on the edge's direction.  For the triangle of a cell the host folds the three
+// edges into one table: the coefficient of each stencil node in each edge.  Then
 //   w_k = lambda_k [k vertex] + sum_e 2 lambda_P(e) lambda_Q(e) A_{k,e}.
 // Node values are read at the unique nodes (I mod (n-1), J mod (n-1)).
 
-constexpr int MQ_NODES = 16;
+//
+// The triangle above the diagonal is the one below it with x and y exchanged, so the kernel
+// works in coordinates (hi, lo) = (max, min) of the particle's cell coordinates, with vertices
+// (0,0), (1,0), (1,1) and one table for both: its index is the same in every lane and the
+// coefficients are operands from the constant bank.  (Two tables chosen per lane made every
+// table read a divergent constant load: 140 us for 2048^2 particles on 1025^2 nodes, C = 4, FP32.)
 
-struct MQTable {
-    int count[2];
-    signed char ox[2][MQ_NODES], oy[2][MQ_NODES];
-    signed char vertex[2][MQ_NODES];      // 0..2 = lambda index, -1 = not a vertex
-    float A32[2][MQ_NODES][3];
-    double A64[2][MQ_NODES][3];
-    signed char ep[2][3], eq[2][3];       // edge e joins vertices ep[e], eq[e]
+// The 12 nodes around the triangle: its vertices, then the rest of their neighbours.
+constexpr int MQ_NODES = 12;
+__host__ __device__ constexpr int mq_x(int k)
+{
+    constexpr int X[MQ_NODES] = {0, 1, 1, 0, -1, 0, -1, 2, 1, 2, 1, 2};
+    return X[k];
+}
+__host__ __device__ constexpr int mq_y(int k)
+{
+    constexpr int Y[MQ_NODES] = {0, 0, 1, 1, 0, -1, -1, 0, -1, 1, 2, 2};
+    return Y[k];
+}
+
+// Is node k in the stencil of edge e?  (All but the two neighbours that only the vertex opposite
+// the edge has.)
+__host__ __device__ constexpr bool mq_in(int k, int e)
+{
+    return e == 0 ? k != 10 && k != 11 : e == 1 ? k != 4 && k != 6 : k != 7 && k != 8;
+}
+
+template <typename R> struct MQTable {
+    R A[MQ_NODES][3];           // coefficient of node k in edge e, which joins vertices e and e + 1
 };
 
 // Minimum-norm coefficients of the mesh edge from (0,0) to (ex,ey) over its 10-node
@@ -297,60 +317,38 @@ static int mesh_edge_host(int ex, int ey, int S[16][2], double A[16])
     return k;
 }
 
-static MQTable build_mq_table()
+template <typename R> static MQTable<R> build_mq_table()
 {
-    MQTable T;
-    int S[3][16][2];
-    double A[3][16];
-    int K[3];
-    const int D[3][2] = {{1, 0}, {0, 1}, {1, 1}};
-    for (int t = 0; t < 3; ++t) K[t] = mesh_edge_host(D[t][0], D[t][1], S[t], A[t]);
-    // triangle 0 (s >= t): (0,0), (1,0), (1,1); triangle 1: (0,0), (1,1), (0,1)
-    const int V[2][3][2] = {{{0, 0}, {1, 0}, {1, 1}}, {{0, 0}, {1, 1}, {0, 1}}};
-    for (int tr = 0; tr < 2; ++tr) {
-        int cnt = 0;
-        for (int i = 0; i < MQ_NODES; ++i) {
-            T.vertex[tr][i] = -1;
-            for (int e = 0; e < 3; ++e) { T.A32[tr][i][e] = 0.f; T.A64[tr][i][e] = 0.0; }
+    MQTable<R> T;
+    const int E[3][4] = {{0, 0, 1, 0}, {1, 0, 0, 1}, {0, 0, 1, 1}};     // origin and direction
+    for (int e = 0; e < 3; ++e) {
+        int S[16][2];
+        double A[16];
+        const int K = mesh_edge_host(E[e][2], E[e][3], S, A);
+        for (int k = 0; k < MQ_NODES; ++k) {
+            T.A[k][e] = R(0);
+            for (int i = 0; i < K; ++i)
+                if (S[i][0] + E[e][0] == mq_x(k) && S[i][1] + E[e][1] == mq_y(k)) T.A[k][e] = (R)A[i];
         }
-        auto slot = [&](int x, int y) {
-            for (int i = 0; i < cnt; ++i)
-                if (T.ox[tr][i] == x && T.oy[tr][i] == y) return i;
-            T.ox[tr][cnt] = (signed char)x;
-            T.oy[tr][cnt] = (signed char)y;
-            return cnt++;
-        };
-        for (int v = 0; v < 3; ++v) T.vertex[tr][slot(V[tr][v][0], V[tr][v][1])] = (signed char)v;
-        for (int e = 0; e < 3; ++e) {
-            const int f = (e + 1) % 3;
-            int dx = V[tr][f][0] - V[tr][e][0], dy = V[tr][f][1] - V[tr][e][1];
-            int bx = V[tr][e][0], by = V[tr][e][1];
-            if (dx < 0 || dy < 0) { dx = -dx; dy = -dy; bx = V[tr][f][0]; by = V[tr][f][1]; }
-            const int type = (dx == 1 && dy == 0) ? 0 : (dx == 0 && dy == 1) ? 1 : 2;
-            T.ep[tr][e] = (signed char)e;
-            T.eq[tr][e] = (signed char)f;
-            for (int k = 0; k < K[type]; ++k) {
-                const int i = slot(bx + S[type][k][0], by + S[type][k][1]);
-                T.A64[tr][i][e] = A[type][k];
-                T.A32[tr][i][e] = (float)A[type][k];
-            }
-        }
-        T.count[tr] = cnt;
     }
     return T;
 }
 
 // built once per process (thread-safe initialisation of a function-local static)
-static const MQTable &mq_table()
+template <typename R> static const MQTable<R> &mq_table()
 {
-    static const MQTable T = build_mq_table();
+    static const MQTable<R> T = build_mq_table<R>();
     return T;
 }
 
+// One particle per thread.  Bound by the L1: twelve gathers a particle, which neighbouring
+// particles share; the weights are 30 FMAs with constant operands.  2048^2 particles on 1025^2
+// nodes, C = 4, FP32: 49 us (17 us of it is what the bytes take); 58 us before the lanes of both
+// triangles read the nodes they share together.
 template <typename P, typename V, typename R, int CT>
 __global__ void __launch_bounds__(256) k_m2p_q(int n, long long N, const P *__restrict__ pos, int Crt,
                                                const V *__restrict__ mesh, V *__restrict__ vals,
-                                               const MQTable T)
+                                               const MQTable<R> T)
 {
     const int C = CT > 0 ? CT : Crt;
     const int nc = n - 1;
@@ -360,69 +358,100 @@ __global__ void __launch_bounds__(256) k_m2p_q(int n, long long N, const P *__re
         load_pos(pos, m, px, py);
         const int i = bin_of(fx_of(px), nc), j = bin_of(fx_of(py), nc);
         const P s = local_coord<P>(px, i, nc), t = local_coord<P>(py, j, nc);
-        const int tr = s >= t ? 0 : 1;
-        R lam[3];
-        if (tr == 0) { lam[0] = R(P(1) - s); lam[1] = R(s - t); lam[2] = R(t); }
-        else         { lam[0] = R(P(1) - t); lam[1] = R(s); lam[2] = R(t - s); }
-        R ce[3];
+        const bool below = s >= t;
+        const P hi = below ? s : t, lo = below ? t : s;
+        const R lam[3] = {R(P(1) - hi), R(hi - lo), R(lo)};
+        const R ce[3] = {R(2) * lam[0] * lam[1], R(2) * lam[1] * lam[2], R(2) * lam[2] * lam[0]};
+        R w[MQ_NODES];
 #pragma unroll
-        for (int e = 0; e < 3; ++e) ce[e] = R(2) * lam[T.ep[tr][e]] * lam[T.eq[tr][e]];
-        R acc[8];
+        for (int k = 0; k < MQ_NODES; ++k) {
+            w[k] = R(0);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc[c] = R(0);
-        const int cnt = T.count[tr];
-        for (int k = 0; k < cnt; ++k) {
-            R w;
-            if (sizeof(R) == 8)
-                w = R(T.A64[tr][k][0]) * ce[0] + R(T.A64[tr][k][1]) * ce[1] + R(T.A64[tr][k][2]) * ce[2];
-            else
-                w = R(T.A32[tr][k][0]) * ce[0] + R(T.A32[tr][k][1]) * ce[1] + R(T.A32[tr][k][2]) * ce[2];
-            const int vk = T.vertex[tr][k];
-            if (vk >= 0) w += lam[vk];
-            int I = i + T.ox[tr][k], J = j + T.oy[tr][k];
+            for (int e = 0; e < 3; ++e)
+                if (mq_in(k, e)) w[k] = fma(T.A[k][e], ce[e], w[k]);
+            if (k < 3) w[k] += lam[k];
+        }
+        // the four columns and rows around the cell (unique nodes)
+        int col[4];
+        const V *row[4];
+#pragma unroll
+        for (int d = 0; d < 4; ++d) {
+            int I = i + d - 1, J = j + d - 1;
             I += I < 0 ? nc : 0;
             I -= I >= nc ? nc : 0;
             J += J < 0 ? nc : 0;
             J -= J >= nc ? nc : 0;
-            const long long node = (long long)J * n + I;
-            if constexpr (CT == 4 && sizeof(V) == 4 && sizeof(R) == 4) {
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(mesh) + node);
-                acc[0] = fmaf(w, v.x, acc[0]);
-                acc[1] = fmaf(w, v.y, acc[1]);
-                acc[2] = fmaf(w, v.z, acc[2]);
-                acc[3] = fmaf(w, v.w, acc[3]);
+            col[d] = I * C;
+            row[d] = mesh + (long long)J * n * C;
+        }
+        R acc[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[c] = R(0);
+#pragma unroll
+        for (int k = 0; k < MQ_NODES; ++k) {
+            // node k of the triangle's own coordinates is read together with its mirror image, so
+            // that the lanes of both triangles read the nodes they share in the same instruction
+            constexpr int MIRROR[MQ_NODES] = {0, 3, 2, 1, 5, 4, 6, -1, -1, 10, 9, 11};
+            const int x = mq_x(k) + 1, y = mq_y(k) + 1;
+            const V *mp;
+            R wk;
+            if (MIRROR[k] >= 0) {
+                mp = row[y] + col[x];
+                wk = below ? w[k] : w[MIRROR[k]];
             } else {
-                const V *mp = mesh + node * C;
-                for (int c = 0; c < C; ++c) acc[c] = fma(w, load_val<V, R>(mp + c), acc[c]);
+                mp = below ? row[y] + col[x] : row[x] + col[y];
+                wk = w[k];
+            }
+            if constexpr (CT == 4 && sizeof(V) == 4 && sizeof(R) == 4) {
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(mp));
+                acc[0] = fmaf(wk, v.x, acc[0]);
+                acc[1] = fmaf(wk, v.y, acc[1]);
+                acc[2] = fmaf(wk, v.z, acc[2]);
+                acc[3] = fmaf(wk, v.w, acc[3]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (c < C) acc[c] = fma(wk, load_val<V, R>(mp + c), acc[c]);
             }
         }
         if constexpr (CT == 4 && sizeof(V) == 4 && sizeof(R) == 4)
             __stcs(reinterpret_cast<float4 *>(vals) + m, make_float4(acc[0], acc[1], acc[2], acc[3]));
         else
-            for (int c = 0; c < C; ++c) store_val<V, R>(vals + m * C + c, acc[c]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c < C) store_val<V, R>(vals + m * C + c, acc[c]);
     }
+}
+
+template <typename P, typename V, typename R>
+static cudaError_t m2p_q_t(int n, long long N, const void *pos, int C, const void *mesh, void *vals,
+                           cudaStream_t s)
+{
+    long long blocks = (N + 255) / 256;
+    if (blocks > num_sms() * 16LL) blocks = num_sms() * 16LL;
+    // four FP32 components as one 16-byte access when the arrays allow it; one to three (and
+    // four in the other types) with the component loop unrolled
+    const bool aligned = ((reinterpret_cast<uintptr_t>(mesh) | reinterpret_cast<uintptr_t>(vals)) & 15) == 0;
+    auto go = [&](auto ct) {
+        k_m2p_q<P, V, R, decltype(ct)::value><<<(unsigned)blocks, 256, 0, s>>>(
+            n, N, (const P *)pos, C, (const V *)mesh, (V *)vals, mq_table<R>());
+    };
+    if (C == 1) go(std::integral_constant<int, 1>());
+    else if (C == 3) go(std::integral_constant<int, 3>());
+    else if (C == 4 && (aligned || sizeof(V) != 4)) go(std::integral_constant<int, 4>());
+    else go(std::integral_constant<int, 0>());
+    count_launch();
+    return cudaGetLastError();
 }
 
 cudaError_t launch_m2p_quadratic(int n, long long N, const void *pos, pfem_dtype pos_t, int C,
                                  const void *mesh, void *vals, pfem_dtype val_t, cudaStream_t s)
 {
     if (N == 0) return cudaSuccess;
-    const MQTable &T = mq_table();
-    long long blocks = (N + 255) / 256;
-    if (blocks > num_sms() * 16LL) blocks = num_sms() * 16LL;
-    const bool aligned = ((reinterpret_cast<uintptr_t>(mesh) | reinterpret_cast<uintptr_t>(vals)) & 15) == 0;
-    if (val_t == PFEM_F64 && pos_t == PFEM_F64)
-        k_m2p_q<double, double, double, 0><<<(unsigned)blocks, 256, 0, s>>>(n, N, (const double *)pos, C, (const double *)mesh, (double *)vals, T);
-    else if (val_t == PFEM_F32 && pos_t == PFEM_F32 && C == 4 && aligned)
-        k_m2p_q<float, float, float, 4><<<(unsigned)blocks, 256, 0, s>>>(n, N, (const float *)pos, C, (const float *)mesh, (float *)vals, T);
-    else if (val_t == PFEM_F32 && pos_t == PFEM_F32)
-        k_m2p_q<float, float, float, 0><<<(unsigned)blocks, 256, 0, s>>>(n, N, (const float *)pos, C, (const float *)mesh, (float *)vals, T);
-    else if (val_t == PFEM_BF16 && pos_t == PFEM_F32)
-        k_m2p_q<float, __nv_bfloat16, float, 0><<<(unsigned)blocks, 256, 0, s>>>(n, N, (const float *)pos, C, (const __nv_bfloat16 *)mesh, (__nv_bfloat16 *)vals, T);
-    else
-        return cudaErrorInvalidValue;
-    count_launch();
-    return cudaGetLastError();
+    if (val_t == PFEM_F64 && pos_t == PFEM_F64) return m2p_q_t<double, double, double>(n, N, pos, C, mesh, vals, s);
+    if (val_t == PFEM_F32 && pos_t == PFEM_F32) return m2p_q_t<float, float, float>(n, N, pos, C, mesh, vals, s);
+    if (val_t == PFEM_BF16 && pos_t == PFEM_F32) return m2p_q_t<float, __nv_bfloat16, float>(n, N, pos, C, mesh, vals, s);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace pfem

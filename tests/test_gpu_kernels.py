@@ -53,3 +53,27 @@ def test_refined_solves(P, which):
     assert torch.equal(a, b)
     ref = O.p2m(pr.n, pos.double().cpu().numpy(), vals.double().cpu().numpy(), shape=1, nthreads=8)
     assert relerr(a.cpu().numpy(), ref) <= TOL32
+
+
+@pytest.mark.parametrize("C", [1, 2, 3, 4, 5, 8])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_mesh_quadratic_m2p(P, C, dtype):
+    """Mesh QCSF M2P for every component count, on particles of both triangles of a cell, the first
+    and last rows and columns among them, reading the distinct nodes only (the image row and
+    column hold something else)."""
+    n, N = 38, 4097
+    pos = G.uniform01(G.SEED_BASE + 910, 2 * N).reshape(N, 2)
+    pos[:64, 0] = np.repeat([0.0, 1e-7, 1.0 - 1e-7, 0.999], 16)
+    pos[64:128, 1] = np.repeat([0.0, 1e-7, 1.0 - 1e-7, 0.999], 16)
+    pos[128:160, 1] = pos[128:160, 0]
+    pos = torch.tensor(pos, dtype=dtype, device="cuda")
+    mesh = G.uniform01(G.SEED_BASE + 911, n * n * C).reshape(n, n, C)
+    mesh[-1], mesh[:, -1] = mesh[0], mesh[:, 0]
+    mesh = torch.tensor(mesh, dtype=dtype, device="cuda")
+    proj = P.Projector(n, N, C=C, pos_dtype=dtype)
+    spoilt = mesh.clone()
+    spoilt[-1] = 7.0
+    spoilt[:, -1] = 7.0
+    got = proj.m2p(pos, spoilt, shape=P.PFEM_SHAPE_QUADRATIC)
+    ref = O.m2p_quadratic(n, pos.double().cpu().numpy(), mesh.double().cpu().numpy())
+    assert relerr(got.cpu().numpy(), ref) <= (TOL64 if dtype == torch.float64 else TOL32)
