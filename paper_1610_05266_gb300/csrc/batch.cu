@@ -178,14 +178,12 @@ __global__ void __launch_bounds__(256, PFEM_P2M_MIN_BLOCKS / 2) k_p2m_batch(cons
 }
 
 // Star table of every problem: block b takes 128 consecutive particles of one problem.
-__global__ void __launch_bounds__(BSTAR) k_star_list_batch(const BPlanDev *pl, P2MArgs base,
-                                                           StarTab t)
+__global__ void __launch_bounds__(BSTAR, PFEM_STAR_MIN_BLOCKS) k_star_list_batch(const BPlanDev *pl,
+                                                                                 P2MArgs base, StarTab t)
 {
-    __shared__ float2 sxy[STAR_KL * BSTAR];
-    __shared__ unsigned skey[STAR_KL * BSTAR];
-    __shared__ int ss[STAR_KL * BSTAR];
-    __shared__ unsigned char sord[STAR_KL * BSTAR];
-    __shared__ unsigned char sstk[STAR_KL * BSTAR];
+    static_assert(BSTAR == STAR_TPB, "HullList's columns");
+    __shared__ float2 sxy[STAR_ROWS * BSTAR];
+    __shared__ int ss[STAR_ROWS * BSTAR];
     if (!totals_ok(pl, -1, t, base.status)) return;
     const long long *sp = plan_star_tiles(pl);
     for (long long b = blockIdx.x; b < pl->n_star_tiles; b += gridDim.x) {
@@ -195,39 +193,29 @@ __global__ void __launch_bounds__(BSTAR) k_star_list_batch(const BPlanDev *pl, P
         if (i >= d.N) continue;
         P2MArgs a;
         problem_args(a, base, d);
-        const HullList L{sxy + threadIdx.x, skey + threadIdx.x, ss + threadIdx.x, sord + threadIdx.x,
-                      sstk + threadIdx.x, BSTAR};
+        const HullList L{sxy + threadIdx.x, ss + threadIdx.x};
         star_list_slot(a.B, a.R0, t, d.poff + i, L, a.status);
     }
 }
 
-// The queued particles of the table, each with its problem's bins and the widest radius: the
-// hull attempt for a short queue, then the region search for the stars still queued.
-template <bool HULL>
-__global__ void __launch_bounds__(64) k_star_retry_batch(const BPlanDev *pl, P2MArgs base, StarTab t)
+// The queued particles of the table, a warp each, with its problem's bins and the widest radius.
+__global__ void __launch_bounds__(RETRY_TPB, PFEM_RETRY_BLOCKS) k_star_retry_batch(const BPlanDev *pl,
+                                                                                   P2MArgs base, StarTab t)
 {
-    __shared__ float2 sxy[HULL ? STAR_KL_RETRY * 64 : 1];
-    __shared__ unsigned skey[HULL ? STAR_KL_RETRY * 64 : 1];
-    __shared__ int ss[HULL ? STAR_KL_RETRY * 64 : 1];
-    __shared__ unsigned char sord[HULL ? STAR_KL_RETRY * 64 : 1];
-    __shared__ unsigned char sstk[HULL ? STAR_KL_RETRY * 64 : 1];
+    __shared__ int2 sd[RETRY_TPB / 32 * WSTAR_CAP];
+    __shared__ int ss[RETRY_TPB / 32 * WSTAR_CAP];
+    const int w = threadIdx.x >> 5;
+    const WarpList L{sd + w * WSTAR_CAP, ss + w * WSTAR_CAP};
     const int n = min(*t.qcount, (int)min(t.N, (long long)0x7fffffff));
-    if (HULL && !short_queue(n, t.N)) return;
     const BDesc *D = plan_desc(pl);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (int i = blockIdx.x * (RETRY_TPB / 32) + w; i < n; i += gridDim.x * (RETRY_TPB / 32)) {
         const int v = t.queue[i];
         const int p = find_problem(pl->P, v, [&](int k) { return D[k].poff; });
         const BDesc d = D[p];
         P2MArgs a;
         problem_args(a, base, d);
         a.B.rmax = max(d.rmax, d.nb / 4 - 1);
-        if constexpr (HULL) {
-            const HullList L{sxy + threadIdx.x, skey + threadIdx.x, ss + threadIdx.x,
-                             sord + threadIdx.x, sstk + threadIdx.x, 64};
-            star_retry_hull_slot(a.B, a.R0, t, v, L, a.status);
-        } else {
-            star_retry_slot(a.B, a.R0, t, v, a.status);
-        }
+        star_retry_slot(a.B, a.R0, t, v, L, a.status);
     }
 }
 
@@ -430,12 +418,13 @@ static cudaError_t p2m_batch_t(const void *plan, const P2MArgs &base, int shape_
     if (e != cudaSuccess) return e;
     const int TYs[BT_SHAPES] = {4, 8, 16};
     if (SHAPE == PFEM_SHAPE_QUADRATIC && w.table) {
-        k_star_list_batch<<<num_sms() * 8, BSTAR, 0, s>>>(pl, base, w.tab);
-        k_star_retry_batch<true><<<num_sms() * PFEM_RETRY_BLOCKS, 64, 0, s>>>(pl, base, w.tab);
-        k_star_retry_batch<false><<<num_sms() * PFEM_RETRY_REGION_BLOCKS, 64, 0, s>>>(pl, base, w.tab);
+        // a block per tile of 128 particles (the problems' ragged last tiles are taken by the
+        // blocks that are done first)
+        k_star_list_batch<<<(unsigned)((w.tab.N + BSTAR - 1) / BSTAR), BSTAR, 0, s>>>(pl, base, w.tab);
+        k_star_retry_batch<<<num_sms() * PFEM_RETRY_BLOCKS, RETRY_TPB, 0, s>>>(pl, base, w.tab);
         k_p2m_batch_tab<P, V, R, S, REF><<<blocks, 16 * TYs[shape_idx], 0, s>>>(
             pl, shape_idx, base, counter, w.tab, w.nodes);
-        count_launch(4);
+        count_launch(3);
     } else {
         k_p2m_batch<P, V, R, S, REF, SHAPE><<<blocks, 16 * TYs[shape_idx], 0, s>>>(
             pl, shape_idx, base, counter);

@@ -77,3 +77,47 @@ def test_mesh_quadratic_m2p(P, C, dtype):
     got = proj.m2p(pos, spoilt, shape=P.PFEM_SHAPE_QUADRATIC)
     ref = O.m2p_quadratic(n, pos.double().cpu().numpy(), mesh.double().cpu().numpy())
     assert relerr(got.cpu().numpy(), ref) <= (TOL64 if dtype == torch.float64 else TOL32)
+
+
+def _disk(M, R, fill, seed):
+    """M x M lattice with the disk of radius R emptied and refilled with `fill` uniform particles."""
+    pos = G.jittered_lattice(M, 0.2, G.SEED_BASE + seed)
+    d = pos - 0.5
+    d -= np.rint(d)
+    pos = pos[(d ** 2).sum(1) >= R * R]
+    u = G.uniform01(G.SEED_BASE + seed + 1, 2 * fill)
+    r, a = R * np.sqrt(u[0::2]), 2 * np.pi * u[1::2]
+    return np.concatenate([pos, 0.5 + np.stack([r * np.cos(a), r * np.sin(a)], 1)])
+
+
+def _rays(M):
+    """A lattice whose rows and columns are stretched unevenly: every particle shares its rays with
+    others at different distances, at exactly equal angles."""
+    g = np.cumsum(1.0 + 0.5 * (np.arange(M) % 3))
+    g = np.floor((g - 0.5) / g[-1] * 4096) / 4096
+    return np.stack([np.tile(g, M), np.repeat(g, M)], 1)
+
+
+STARS = {"dense_disk": lambda: _disk(32, 0.1, 700, 920),      # lists over their capacity
+         "sparse_disk": lambda: _disk(96, 0.06, 4, 930),      # circles wider than every list's cutoff
+         "rays": lambda: _rays(33),                           # equal angles: the exact order
+         "few": lambda: G.jittered_lattice(24, 0.3, G.SEED_BASE + 940),
+         "ragged": lambda: G.jittered_lattice(37, 0.3, G.SEED_BASE + 941)[:-3]}
+
+
+@pytest.mark.parametrize("which", sorted(STARS))
+def test_stars_of_uneven_sets(P, which):
+    """The list kernel and the warp search for queued stars, bit for bit against the oracle's stars."""
+    pos = STARS[which]()
+    proj = P.Projector(33, len(pos), pos_dtype=torch.float64)
+    proj.build(torch.tensor(pos, device="cuda"))
+    nbrs, counts = proj.stars()
+    proj.check(which)
+    nbrs, counts, perm = nbrs.cpu().numpy(), counts.cpu().numpy(), proj.cells.perm.cpu().numpy()
+    cells = O.build_cells(33, pos)
+    assert counts.sum() == 6 * len(pos)
+    for s in range(len(pos)):
+        mine, ref = list(perm[nbrs[s, :counts[s]]]), list(O.star(cells, int(perm[s])))
+        assert mine[mine.index(min(mine)):] + mine[:mine.index(min(mine))] == \
+            ref[ref.index(min(ref)):] + ref[:ref.index(min(ref))], s
+        assert (nbrs[s, counts[s]:] == -1).all()
