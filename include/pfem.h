@@ -72,7 +72,8 @@ typedef enum {
 typedef enum { PFEM_F64 = 0, PFEM_F32 = 1, PFEM_BF16 = 2 } pfem_dtype;
 typedef enum { PFEM_SHAPE_LINEAR = 0, PFEM_SHAPE_QUADRATIC = 1 } pfem_shape;
 typedef enum {
-    PFEM_SOLVE_F64 = 0,         /* moment assembly and Cholesky in FP64 */
+    PFEM_SOLVE_F64 = 0,         /* FP64 accuracy: FP32 Cholesky, the solution refined to the last bits
+                                   of 64-bit fixed point; FP64 Cholesky or SVD where that fails */
     PFEM_SOLVE_F32 = 1,         /* in FP32 after centring/scaling by the edge length */
     PFEM_SOLVE_F32_REFINED = 2, /* FP32 Cholesky + one refinement step, residual in 64-bit fixed
                                    point (at least FP64's accuracy) */
@@ -239,10 +240,11 @@ pfem_status pfem_shape_quadratic(pfem_ctx *ctx, int32_t n, int32_t nb, int64_t N
  * factorisation of its 6x6 moment matrix.  The call runs a fast pass over every node and a fix
  * pass over the nodes the fast pass queued: a node with an edge whose pivot falls below the
  * fast tolerance (rank deficient, e.g. a stencil of five particles, or too ill-conditioned for
- * the precision: 3e-4 of the trace in FP32, 1e-6 in FP64), with more than the context's
+ * the FP32 factor: 3e-4 of the trace), with more than the context's
  * node_capacity distinct particles, or whose search ran out of its first region (a sparse
- * region or a void), is recomputed in FP64 with the minimum-norm least-squares solution by SVD
- * (App. A) and searches up to the context's search_radius_max.  Linear shape functions queue
+ * region or a void), is recomputed in FP64, each edge by Cholesky down to a pivot of 1e-6 of the
+ * trace and below that with the minimum-norm least-squares solution by SVD (App. A), and
+ * searches up to the context's search_radius_max.  Linear shape functions queue
  * only the last kind.  Workspace layout after the 256-byte status block: the fix-pass queue
  * from byte 512 (8 bytes per node; with ws_bytes < 520 there is no queue and such nodes record
  * PFEM_ERR_DEGENERATE or PFEM_ERR_CAPACITY), then, for the quadratic apply form, 136 bytes of

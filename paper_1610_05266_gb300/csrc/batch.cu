@@ -15,6 +15,7 @@
 // the stage launches allocate nothing and can be captured in a CUDA graph.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(RETRY_TPB, PFEM_RETRY_BLOCKS) k_star_retry_bat
 // The table path's fast pass of every problem in one persistent kernel (as k_p2m_tab: location
 // from the star table, edge solves and apply per node, no node records).
 template <typename P, typename V, typename R, typename S, int REFINE>
-__global__ void __launch_bounds__(256, tab_min_blocks<S>() / 2) k_p2m_batch_tab(
+__global__ void __launch_bounds__(256, tab_min_blocks<REFINE>() / 2) k_p2m_batch_tab(
     const BPlanDev *pl, int shape_idx, P2MArgs base, unsigned long long *counter, StarTab tab,
     long long nodes)
 {
@@ -422,11 +423,14 @@ static cudaError_t p2m_batch_t(const void *plan, const P2MArgs &base, int shape_
         // blocks that are done first)
         k_star_list_batch<<<(unsigned)((w.tab.N + BSTAR - 1) / BSTAR), BSTAR, 0, s>>>(pl, base, w.tab);
         k_star_retry_batch<<<num_sms() * PFEM_RETRY_BLOCKS, RETRY_TPB, 0, s>>>(pl, base, w.tab);
-        k_p2m_batch_tab<P, V, R, S, REF><<<blocks, 16 * TYs[shape_idx], 0, s>>>(
+        constexpr int TREF = sizeof(S) == 8 ? REFINE_FIX64 : REF;    // as for one problem
+        k_p2m_batch_tab<P, V, R, float, TREF><<<blocks, 16 * TYs[shape_idx], 0, s>>>(
             pl, shape_idx, base, counter, w.tab, w.nodes);
         count_launch(3);
     } else {
-        k_p2m_batch<P, V, R, S, REF, SHAPE><<<blocks, 16 * TYs[shape_idx], 0, s>>>(
+        constexpr bool F64 = sizeof(S) == 8 && SHAPE == PFEM_SHAPE_QUADRATIC;
+        k_p2m_batch<P, V, R, std::conditional_t<F64, float, S>, F64 ? REFINE_FIX64 : REF, SHAPE>
+            <<<blocks, 16 * TYs[shape_idx], 0, s>>>(
             pl, shape_idx, base, counter);
         count_launch();
     }

@@ -1,0 +1,249 @@
+// fix64.cuh -- the FP64 moment solve of the table path without the FP64 pipe.
+//
+// An SM of GB300 issues two FP64 instructions a clock, so a warp's FP64 instruction takes its
+// scheduler 64 cycles; assembling, factoring and solving the three 6 x 6 systems of a node in FP64
+// took about 2600 of them.  Here each edge system is factored in FP32 and its solution y
+// refined until it is exact to the last bits of a 64-bit fixed-point number: residuals r = b - M y in
+// 64-bit fixed point on the integer pipes, corrections through the FP32 factor.  Each step gains
+// the bits that FP32 has over the system's condition (about 11 on jittered lattices: four
+// steps), at about 100 integer instructions a stencil point.  Positions enter as 64-bit fixed
+// point too: an offset between two of them is exact where FP64 rounds it.
+//
+// Scaling, all by powers of two: coordinates X in Q64, |X| < 1/2, from the largest of the
+// stencil; y'_k = y_k g^deg(k) and b' likewise, as integers with unit 2^-s, |y'|, |b'| <= 2^(60 - s); t
+// = p . y, X t, Y t and the sums in the same unit.  |t| <= 2.75 of the largest |y'|.  A product is
+// rounded within 1.5 units; with the largest coordinate at 1/4 to 1/2 and an edge of a fifth of
+// the stencil the unit is 2^-57 or below against coefficients A = p . y of about 0.3: FP64's
+// rounding of the same sums is 2^-53 of their largest terms.  The sums may wrap: the residual
+// itself is small.
+//
+// Measured (round trip, FP64 values): 513^2 nodes / 1024^2 particles 1798 -> 700 us (node kernel
+// 1475 -> 455), 33^2 / 64^2 200 -> 101 us with four lanes a node; the mesh's error against 64-bit
+// arithmetic 2.6e-16 -> 1.6e-16 of its 2-norm.
+#pragma once
+
+#include "moments.cuh"
+
+namespace pfem {
+
+// x mod 1 in Q64 (rounded to nearest below 2^-11, exact above), by integer operations.
+__device__ __forceinline__ long long fx64(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)(b >> 52) & 0x7ff, s = e - 1011;
+    const unsigned long long m = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+    unsigned long long q = 0;
+    if (s >= 0) q = s < 64 ? m << s : 0ull;
+    else if (s > -54) q = (m + (1ull << (-s - 1))) >> -s;
+    return (long long)((b >> 63) ? 0ull - q : q);
+}
+__device__ __forceinline__ long long fx64(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    const int e = (int)(b >> 23) & 0xff, s = e - 86;
+    const unsigned long long m = (b & 0x7fffffu) | (e ? 1u << 23 : 0u);
+    unsigned long long q = 0;
+    if (s >= 0) q = s < 64 ? m << s : 0ull;
+    else if (s > -25) q = (m + (1ull << (-s - 1))) >> -s;
+    return (long long)((b >> 31) ? 0ull - q : q);
+}
+
+// I / nc in Q64, rounded to nearest (0 <= I < nc < 2^31).
+__device__ __forceinline__ long long node_fx64(int I, int nc)
+{
+    const unsigned long long d = (unsigned long long)nc, a = (unsigned long long)I << 32;
+    const unsigned long long h = a / d, r = (a - h * d) << 32, l = r / d, r2 = r - l * d;
+    return (long long)((h << 32) + l + (2 * r2 >= d ? 1 : 0));
+}
+
+// A 64-bit integer as h 2^32 + l with both parts signed.
+struct Split64 {
+    int h, l;
+};
+__device__ __forceinline__ Split64 split64(long long u)
+{
+    const int l = (int)u;
+    return {(int)(u >> 32) + (int)((unsigned)l >> 31), l};
+}
+// a b / 2^64 within 1.5 (|a| < 2^63 - 2^31, |b| < 2^62)
+__device__ __forceinline__ long long mul64(Split64 a, Split64 b)
+{
+    return (long long)a.h * b.h + (long long)(__mulhi(a.h, b.l) + __mulhi(a.l, b.h) + 1);
+}
+
+struct EdgeFix64 {
+    Split64 Y[6];
+    long long Y0, Y1, Y2;
+
+    __device__ __forceinline__ void set(const long long y[6])
+    {
+        Y0 = y[0];
+        Y1 = y[1];
+        Y2 = y[2];
+#pragma unroll
+        for (int k = 3; k < 6; ++k) Y[k] = split64(y[k]);
+    }
+    // t = p . y at (X, Z)
+    __device__ __forceinline__ long long value(Split64 X, Split64 Z) const
+    {
+        const Split64 u = split64(Y1 + mul64(X, Y[3]) + mul64(Z, Y[4]));
+        const Split64 v = split64(Y2 + mul64(Z, Y[5]));
+        return Y0 + mul64(X, u) + mul64(Z, v);
+    }
+    // r -= p (p . y)
+    __device__ __forceinline__ void residual(Split64 X, Split64 Z, long long r[6]) const
+    {
+        const long long t = value(X, Z);
+        const Split64 ts = split64(t);
+        const long long xt = mul64(X, ts), zt = mul64(Z, ts);
+        const Split64 xs = split64(xt), zs = split64(zt);
+        r[0] -= t;
+        r[1] -= xt;
+        r[2] -= zt;
+        r[3] -= mul64(X, xs);
+        r[4] -= mul64(Z, xs);
+        r[5] -= mul64(Z, zs);
+    }
+};
+
+// Offsets of a node's particles from it in fixed point, scaled up by a common power of two so that
+// every |offset| < 2^60: o[0..nu) in Q64.
+template <typename P, int UM>
+__device__ __forceinline__ void node_offsets64(const void *pos, int Iu, int Ju, int nc, const int *us,
+                                               int nu, longlong2 (&o)[UM])
+{
+    const long long nx = node_fx64(Iu, nc), ny = node_fx64(Ju, nc);
+    unsigned long long m = 0;
+    for (int i = 0; i < nu; ++i) {
+        P px, py;
+        load_pos((const P *)pos, us[i], px, py);
+        const long long x = fx64(px) - nx, y = fx64(py) - ny;
+        m |= (unsigned long long)(x ^ (x >> 63)) | (unsigned long long)(y ^ (y >> 63));
+        o[i] = make_longlong2(x, y);
+    }
+    const int L = __clzll((long long)m) - 4;
+    for (int i = 0; i < nu; ++i) {
+        if (L >= 0) o[i] = make_longlong2(o[i].x << L, o[i].y << L);
+        else o[i] = make_longlong2(o[i].x >> -L, o[i].y >> -L);
+    }
+}
+
+// Weights of the quadratic part in fixed point: w[i] += 2 lambda_nu lambda_sg A_{i e} 2^56 over the
+// edges e0 <= e < e1.  Returns 0, or -PFEM_DEFER for a system below the FP32 fast-solve
+// tolerance (moments.cuh) or beyond the fixed-point range.
+constexpr int W64_SHIFT = 56;            // weights up to 2^7
+constexpr double W64_UNIT = 1.3877787807814457e-17;
+template <int UM>
+__device__ __forceinline__ int node_solve64(const longlong2 (&o)[UM], const unsigned vm[3],
+                                            const int vi[3], const double lam[3], int e0, int e1,
+                                            long long *w, int defer)
+{
+    auto pow2 = [](int e) { return __int_as_float((e + 127) << 23); };
+#pragma unroll 1
+    for (int e = e0; e < e1; ++e) {
+        const int f = e == 2 ? 0 : e + 1;
+        const unsigned mask = vm[e] | vm[f];
+        const longlong2 on = o[vi[e]], os = o[vi[f]];
+        const long long mx = on.x + os.x, my = on.y + os.y;
+        // FP32 system in units of 2^63: coordinates about the edge's midpoint, doubled
+        Moment<float> M;
+        M.zero();
+        int hm = 0;
+        for (unsigned m = mask; m; m &= m - 1) {
+            const longlong2 p = o[__ffs(m) - 1];
+            const int hx = (int)((2 * p.x - mx) >> 32), hy = (int)((2 * p.y - my) >> 32);
+            hm = max(hm, max(hx ^ (hx >> 31), hy ^ (hy >> 31)));
+            M.add((float)hx * 4.656612873077393e-10f, (float)hy * 4.656612873077393e-10f);
+        }
+        const long long dx = on.x - os.x, dy = on.y - os.y;      // half the edge, as X of nu
+        const float ex = (float)dx * 2.168404344971009e-19f, ey = (float)dy * 2.168404344971009e-19f;
+        const float l2 = fmaf(ex, ex, ey * ey);
+        // the tolerance of the system scaled by the edge length: pivots of degree d carry l^2d
+        const float i2 = 1.f / l2, i4 = i2 * i2;
+        const float tol = FastTol<float>::v *
+                          (M.m[tri_ix(0, 0)] + (M.m[tri_ix(1, 1)] + M.m[tri_ix(2, 2)]) * i2 +
+                           (M.m[tri_ix(3, 3)] + M.m[tri_ix(4, 4)] + M.m[tri_ix(5, 5)]) * i4);
+        const float t1 = tol * l2, t2 = t1 * l2;
+        const float tols[6] = {tol, t1, t1, t2, t2, t2};
+        if (!M.factor_tol(tols)) return defer;
+        const float b[6] = {0.f, 0.f, 0.f, -0.5f * ex * ex, -0.5f * ex * ey, -0.5f * ey * ey};
+        float y[6];
+        M.solve(b, y);
+        // to Q64: X' = x 2^(k - 1) with k the left shift that brings the largest coordinate up to
+        // a half; c[d]: the factor of degree d from the FP32 to the fixed-point units of y
+        const int k = __clz(hm + 1) - 1;
+        if (k > 20) return defer;
+        const float c1 = pow2(1 - k), c2 = c1 * c1;
+        const float c[6] = {1.f, c1, c1, c2, c2, c2};
+        const float ic1 = pow2(k - 1), ic2 = ic1 * ic1;
+        float ym = 0.f;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) ym = fmaxf(ym, fmaxf(fabsf(y[q] * c[q]), fabsf(b[q] * ic2)));
+        const int bm = max((int)(__float_as_uint(ym) >> 23), 124);     // ym < 2^(bm - 126)
+        if (bm > 166) return defer;
+        const int s = 186 - bm;
+        const float us = pow2(-s), sc = pow2(s - 30);
+        long long Y[6], r[6], B[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) Y[q] = __float2ll_rn(y[q] * c[q] * sc * 1073741824.0f);
+        const long long xn = dx << k, yn = dy << k;              // X' of nu; b' = -2 (X'^2, X'Y', Y'^2)
+        B[0] = B[1] = B[2] = 0;
+        const long long half = 1ll << (62 - s);
+        B[3] = -((__mul64hi(xn, xn) + half) >> (63 - s));
+        B[4] = -((__mul64hi(xn, yn) + half) >> (63 - s));
+        B[5] = -((__mul64hi(yn, yn) + half) >> (63 - s));
+        auto coords = [&](int i, Split64 &X, Split64 &Z) {
+            const longlong2 p = o[i];
+            X = split64((2 * p.x - mx) << k);
+            Z = split64((2 * p.y - my) << k);
+        };
+        EdgeFix64 E;
+        bool done = false;
+        float last = ym;                 // the correction before
+        for (int it = 0; it < 12 && !done; ++it) {
+            E.set(Y);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) r[q] = B[q];
+            for (unsigned m = mask; m; m &= m - 1) {
+                Split64 X, Z;
+                coords(__ffs(m) - 1, X, Z);
+                E.residual(X, Z, r);
+            }
+            float rf[6], d[6], dm = 0.f;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) rf[q] = __ll2float_rn(r[q]) * us * c[q];
+            M.solve(rf, d);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                d[q] *= c[q];
+                dm = fmaxf(dm, fabsf(d[q]));
+                Y[q] += __float2ll_rn(d[q] * sc * 1073741824.0f);
+            }
+            // 2^-43: the next correction would be smaller by this one's ratio to the last; or the
+            // floor that the rounding of the residual sets, if it is below 2^-36
+            done = dm <= 1.1368683772161603e-13f * ym || (dm > 0.5f * last && dm <= 1.4551915228366852e-11f * ym);
+            last = dm;
+        }
+        if (!done) return defer;
+        E.set(Y);
+        const double coef = 2.0 * lam[e] * lam[f];
+        const Split64 cf = split64(__double2ll_rn(coef * 2305843009213693952.0));   // 2^61
+        const int sh = W64_SHIFT + 3 - s;                        // product: coef A 2^(s - 3)
+        int tm = 0;
+        for (unsigned m = mask; m; m &= m - 1) {
+            const int i = __ffs(m) - 1;
+            Split64 X, Z;
+            coords(i, X, Z);
+            const long long t = E.value(X, Z);
+            const int h = (int)(t >> 32);
+            tm = max(tm, h ^ (h >> 31));
+            const long long ct = mul64(split64(t), cf);
+            w[i] += sh >= 0 ? ct << sh : ct >> -sh;
+        }
+        // |A| <= (tm + 1) 2^(32 - s): keep the weights well inside their range
+        if (((float)tm + 1.f) * pow2(32 - s) * fabsf((float)coef) > 30.f) return defer;
+    }
+    return 0;
+}
+
+}  // namespace pfem

@@ -44,12 +44,20 @@ template <typename S> struct Moment {
 #pragma unroll
         for (int r = 0; r < 6; ++r) tr += m[tri_ix(r, r)];
         const S tol = rel_tol * tr;
+        const S tols[6] = {tol, tol, tol, tol, tol, tol};
+        return factor_tol(tols);
+    }
+
+    // The same with a tolerance for each pivot.
+    __device__ __forceinline__ bool factor_tol(const S tols[6])
+    {
         bool ok = true;
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
             S s = m[tri_ix(j, j)];
 #pragma unroll
             for (int k = 0; k < j; ++k) s = fma(-m[tri_ix(j, k)], m[tri_ix(j, k)], s);
+            const S tol = tols[j];
             ok &= s > tol;
             const S d = sqrt(s > tol ? s : tol);
             const S inv = S(1) / d;
@@ -110,9 +118,9 @@ __device__ __forceinline__ float f32_trunc(double d)
     return e > 0 ? __uint_as_float(u) : 0.0f;
 }
 
-// Refinement of the FP32 moment solve: none, or one step with the residual r = b - M y in 64-bit
-// fixed point (FixRes).
-enum { REFINE_NONE = 0, REFINE_FIX = 1 };
+// Refinement of the FP32 moment solve: none, one step with the residual r = b - M y in 64-bit
+// fixed point (FixRes), or steps until the solution has FP64's accuracy (fix64.cuh).
+enum { REFINE_NONE = 0, REFINE_FIX = 1, REFINE_FIX64 = 2 };
 
 // ----------------------------------------------------------------- fixed-point residual
 // The residual r = b - sum_mu p_mu (p_mu . y) of one edge system on the integer pipes.

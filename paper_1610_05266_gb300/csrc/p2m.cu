@@ -2,6 +2,7 @@
 // from explicit weights) and of the Delaunay-star diagnostic.
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "internal.h"
 #include "p2m.cuh"
@@ -45,12 +46,21 @@ static P2MArgs make_args(const GeoArgs &g, DevStatus *st)
     return a;
 }
 
+// Meshes of up to this many nodes per SM run four lanes a node: their warps are too few to cover one
+// lane's serial work.  Round trips on 152 SMs (24,320 nodes at the line), one lane / four: 33^2 FP64
+// 136 / 102 us, 129^2 113 / 102 (FP64 153 / 140), 138^2 123 / 111, 200^2 139 / 150, 257^2 three loop
+// steps 523 / 600.
+constexpr int TAB_QUAD_NODES = 160;
+
 static dim3 node_grid(int n) { return dim3((n + 15) / 16, (n + 7) / 8); }
 
 template <typename P, typename V, typename R, typename S, int REF, int SHAPE, bool W>
 static cudaError_t go_fast(const P2MArgs &a, cudaStream_t s)
 {
-    k_p2m<P, V, R, S, REF, SHAPE, W><<<node_grid(a.n), 128, 0, s>>>(a);
+    // FP64 solves take the FP32 factor with the solution refined to FP64 (fix64.cuh)
+    constexpr bool F64 = sizeof(S) == 8 && SHAPE == PFEM_SHAPE_QUADRATIC;
+    k_p2m<P, V, R, std::conditional_t<F64, float, S>, F64 ? REFINE_FIX64 : REF, SHAPE, W>
+        <<<node_grid(a.n), 128, 0, s>>>(a);
     count_launch();
     return cudaGetLastError();
 }
@@ -104,7 +114,11 @@ static cudaError_t go(const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
         stage_event(g, 2, s);
         e = wait_values(g, s);
         if (e != cudaSuccess) return e;
-        k_p2m_tab<P, V, R, S, REF><<<node_grid(a.n), 128, 0, s>>>(a, *tab);
+        constexpr int TREF = sizeof(S) == 8 ? REFINE_FIX64 : REF;
+        if ((long long)a.n * a.n <= (long long)TAB_QUAD_NODES * num_sms())
+            k_p2m_tab<P, V, R, float, TREF, 4><<<dim3((a.n + 7) / 8, (a.n + 3) / 4), 128, 0, s>>>(a, *tab);
+        else
+            k_p2m_tab<P, V, R, float, TREF, 1><<<node_grid(a.n), 128, 0, s>>>(a, *tab);
         count_launch();
         e = cudaGetLastError();
         stage_event(g, 3, s);
@@ -119,7 +133,7 @@ static cudaError_t go(const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
     P2MArgs f = a;
     f.B.rmax = rmax_far > a.B.rmax ? rmax_far : a.B.rmax;
     if (SHAPE == PFEM_SHAPE_QUADRATIC && !W && tab)
-        k_p2m_fix_tab<P, V, R, sizeof(S) == 4><<<num_sms(), 128, 0, s>>>(f, *tab);
+        k_p2m_fix_tab<P, V, R><<<num_sms() * 2, 128, 0, s>>>(f, *tab);
     else
         k_p2m_fix<P, V, R, SHAPE, W><<<num_sms(), 128, 0, s>>>(f);
     count_launch();

@@ -9,6 +9,7 @@
 // and alpha_i = sum_mu w_{i mu} alpha_mu for every field component in one pass.
 #pragma once
 
+#include "fix64.cuh"
 #include "geom.cuh"
 #include "moments.cuh"
 #include "startab.cuh"
@@ -430,12 +431,13 @@ __device__ __forceinline__ int node_u_sets(const int tri[3], const SA *st, int *
     return over ? -1 : 0;
 }
 
-// The three edge systems of a node over its particle set: uw[u] += 2 lambda_nu lambda_sg A_{u e}.
+// The edge systems e0 <= e < e1 of a node over its particle set: uw[u] += 2 lambda_nu lambda_sg
+// A_{u e}, or with RAW (one edge) uw[u] = A_{u e}.
 // Returns 0, or -PFEM_DEFER when a moment matrix is below the fast-solve tolerance.
-template <typename P, typename R, typename S, int REFINE, bool SVD, int UM>
+template <typename P, typename R, typename S, int REFINE, bool SVD, int UM, bool RAW = false>
 __device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R> &np,
                                             const int *us, R *uw, const unsigned vm[3],
-                                            const int vi[3], const R lam[3])
+                                            const int vi[3], const R lam[3], int e0 = 0, int e1 = 3)
 {
     // Offsets are re-read from the positions, which neighbouring nodes share in L1, instead of
     // being copied into thread-private memory.
@@ -453,7 +455,7 @@ __device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R
 #endif
     constexpr int edge_unroll = PFEM_EDGE_UNROLL;
 #pragma unroll edge_unroll
-    for (int e = 0; e < 3; ++e) {
+    for (int e = e0; e < e1; ++e) {
         const int f = e == 2 ? 0 : e + 1;
         const unsigned mask = vm[e] | vm[f];
         S rnx, rny, rsx, rsy;
@@ -521,7 +523,7 @@ __device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R
             offset(i, ox, oy);
             const S x = (ox - mx) * inv, yv = (oy - my) * inv;
             const S A = y[0] + x * y[1] + yv * y[2] + x * x * y[3] + x * yv * y[4] + yv * yv * y[5];
-            uw[i] = fma(coef, R(A), uw[i]);
+            uw[i] = RAW ? R(A) : fma(coef, R(A), uw[i]);
         }
     }
     return 0;
@@ -544,6 +546,30 @@ __device__ __forceinline__ int node_quadratic(const P2MArgs &a, const NodePos<P,
     const int r = node_u_solve<P, R, S, REFINE, SVD, UM>(a, np, us, uw, vm, vi, lam);
     if (r != 0) return r;
     for (int i = 0; i < nu; ++i) emit(us[i], uw[i]);
+    return 0;
+}
+
+// node_quadratic with the solution refined in 64-bit fixed point (fix64.cuh): calls emit(slot, w) for
+// the quadratic part of every particle of U, then for the linear part of the vertices.
+template <typename P, typename R, typename SA, typename Emit>
+__device__ __forceinline__ int node_quadratic64(const P2MArgs &a, int Iu, int Ju, const int tri[3],
+                                                const SA *st, const R lam[3], Emit &&emit)
+{
+    int us[UMAX];
+    int nu;
+    unsigned vm[3];
+    int vi[3];
+    if (node_u_sets<UMAX>(tri, st, us, nu, vm, vi, min(a.ucap, UMAX)) != 0) return -PFEM_DEFER;
+    longlong2 o[UMAX];
+    long long w[UMAX];
+    node_offsets64<P>(a.pos, Iu, Ju, a.n - 1, us, nu, o);
+    for (int i = 0; i < nu; ++i) w[i] = 0;
+    const double l64[3] = {(double)lam[0], (double)lam[1], (double)lam[2]};
+    const int r = node_solve64(o, vm, vi, l64, 0, 3, w, -PFEM_DEFER);
+    if (r != 0) return r;
+    for (int i = 0; i < nu; ++i) emit(us[i], (R)(__ll2double_rn(w[i]) * W64_UNIT));
+#pragma unroll
+    for (int e = 0; e < 3; ++e) emit(tri[e], lam[e]);
     return 0;
 }
 
@@ -606,7 +632,14 @@ __device__ __forceinline__ void p2m_node(const P2MArgs &a, int I, int J)
         if (st == 0) {
             if (SHAPE == PFEM_SHAPE_QUADRATIC) {
                 const ArrStar sa[3] = {{stars[0], ns[0]}, {stars[1], ns[1]}, {stars[2], ns[2]}};
-                st = node_quadratic<P, R, S, REFINE, SVD>(a, np, tri, sa, lam, emit);
+                if constexpr (REFINE == REFINE_FIX64) {
+                    st = node_quadratic64<P, R>(a, Iu, Ju, tri, sa, lam, emit);
+                    // no fix pass to leave it to: FP64's own pivot tolerance decides (nothing was emitted)
+                    if (st == -PFEM_DEFER && a.defer_cap <= 0)
+                        st = node_quadratic<P, R, double, REFINE_NONE, false>(a, np, tri, sa, lam, emit);
+                } else {
+                    st = node_quadratic<P, R, S, REFINE, SVD>(a, np, tri, sa, lam, emit);
+                }
             } else {
                 for (int e = 0; e < 3; ++e) emit(tri[e], lam[e]);
             }
@@ -632,7 +665,14 @@ __device__ __forceinline__ void p2m_node(const P2MArgs &a, int I, int J)
         if (st == 0) {
             if (SHAPE == PFEM_SHAPE_QUADRATIC) {
                 const ArrStar sa[3] = {{stars[0], ns[0]}, {stars[1], ns[1]}, {stars[2], ns[2]}};
-                st = node_quadratic<P, R, S, REFINE, SVD>(a, np, tri, sa, lam, emit);
+                if constexpr (REFINE == REFINE_FIX64) {
+                    st = node_quadratic64<P, R>(a, Iu, Ju, tri, sa, lam, emit);
+                    // no fix pass to leave it to: FP64's own pivot tolerance decides (nothing was emitted)
+                    if (st == -PFEM_DEFER && a.defer_cap <= 0)
+                        st = node_quadratic<P, R, double, REFINE_NONE, false>(a, np, tri, sa, lam, emit);
+                } else {
+                    st = node_quadratic<P, R, S, REFINE, SVD>(a, np, tri, sa, lam, emit);
+                }
             } else {
                 for (int e = 0; e < 3; ++e) emit(tri[e], lam[e]);
             }
@@ -796,21 +836,42 @@ __global__ void __launch_bounds__(128, PFEM_GEOM_MIN_BLOCKS) k_p2m_geom(P2MArgs 
     geom_node<P, V, R>(a, t, r, I, J, (long long)J * a.n + I);
 }
 
+// The lanes of a node (a group of Q consecutive ones that run the same control flow), and the sum
+// and the least of their values.
+template <int Q> __device__ __forceinline__ unsigned group_mask()
+{
+    return ((1u << Q) - 1u) << (threadIdx.x & 31 & ~(Q - 1));
+}
+template <int Q, typename T> __device__ __forceinline__ T group_sum(T v)
+{
+#pragma unroll
+    for (int o = 1; o < Q; o <<= 1) v += __shfl_xor_sync(group_mask<Q>(), v, o);
+    return v;
+}
+template <int Q> __device__ __forceinline__ int group_min(int v)
+{
+#pragma unroll
+    for (int o = 1; o < Q; o <<= 1) v = min(v, __shfl_xor_sync(group_mask<Q>(), v, o));
+    return v;
+}
+
 // The fix pass of the table path: the queued nodes located with the star table (complete after
-// the retry kernels; the launcher passes the widest search radius for the nearest particle) and
-// every edge solved in FP64 by the SVD, as k_p2m_fix does with stars searched per thread.  With
-// CHOL (runs whose fast pass solved in FP32) a node first takes the FP64 Cholesky solve of the
-// FP64 fast path, pivot tolerance included: a system too ill-conditioned for the FP32 solve is
-// usually well within FP64's, and only the nodes below that tolerance (rank deficient, or
-// conditioned beyond it) take the SVD.
-template <typename P, typename V, typename R, bool CHOL>
+// the retry kernels; the launcher passes the widest search radius for the nearest particle),
+// four lanes a node as in tab_node.  Each edge system is solved in FP64: by Cholesky down to the
+// FP64 pivot tolerance -- a system too ill-conditioned for the FP32 factor is usually well within
+// FP64's -- and below it (rank deficient, or conditioned beyond it) by the SVD.  A queued node's
+// time is one thread's chain of FP64 instructions, so the edges of a node run side by side: about
+// 1500 queued nodes of 513^2 over 1024^2 uniform random particles 1150 -> 434 us.
+template <typename P, typename V, typename R>
 __global__ void __launch_bounds__(128) k_p2m_fix_tab(P2MArgs a, StarTab t)
 {
+    constexpr int Q = 4, UM = UMAX_SVD;
     const int cnt = min(*a.defer_count, a.defer_cap);
+    const int q = threadIdx.x & (Q - 1), e0 = q, e1 = min(q + 1, 3);
     P2MArgs f = a;
     f.defer_cap = 0;
     const int nc = a.n - 1;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / Q; i < cnt; i += gridDim.x * blockDim.x / Q) {
         const long long node = a.defer_list[i];
         const int I = (int)(node % a.n), J = (int)(node / a.n);
         const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
@@ -825,26 +886,45 @@ __global__ void __launch_bounds__(128) k_p2m_fix_tab(P2MArgs a, StarTab t)
                 sa[e] = tab_star(t, tri[e]);
                 if (sa[e].n < 0) st = sa[e].n == -1 ? -PFEM_ERR_CAPACITY : sa[e].n;
             }
-        NodePos<P, R> np;
-        np.init(Iu, Ju, nc);
         R acc[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) acc[c] = R(0);
         if (st == 0) {
+            NodePos<P, R> np;
+            np.init(Iu, Ju, nc);
             R lam[3];
             barycentric(f, np, tri, lam);
-            auto emit = [&](int sl, R wgt) {
-                R v[8];
-                load_vals<V, R>((const V *)f.vals, f.perm, sl, f.C, v);
+            int us[UM];
+            R uw[UM];
+            int nu;
+            unsigned vm[3];
+            int vi[3];
+            if (node_u_sets<UM>(tri, sa, us, nu, vm, vi) != 0) {
+                st = -PFEM_ERR_CAPACITY;
+            } else {
+                for (int k = 0; k < nu; ++k) uw[k] = R(0);
+                if (q == 0)
+#pragma unroll
+                    for (int e = 0; e < 3; ++e) uw[vi[e]] += lam[e];
+                // nothing is added to uw by a system that Cholesky cannot factor
+                if (node_u_solve<P, R, double, REFINE_NONE, false, UM>(f, np, us, uw, vm, vi, lam, e0, e1) != 0)
+                    node_u_solve<P, R, double, REFINE_NONE, true, UM>(f, np, us, uw, vm, vi, lam, e0, e1);
+                __syncwarp(0xfu << (threadIdx.x & 28));
+                for (int k = 0; k < nu; ++k) {
+                    const R wk = group_sum<Q>(uw[k]);
+                    if ((k & (Q - 1)) != q) continue;
+                    R v[8];
+                    load_vals<V, R>((const V *)f.vals, f.perm, us[k], f.C, v);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        if (c < f.C) acc[c] = fma(wk, v[c], acc[c]);
+                }
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
-                    if (c < f.C) acc[c] = fma(wgt, v[c], acc[c]);
-            };
-            st = CHOL ? node_quadratic<P, R, double, REFINE_NONE, false>(f, np, tri, sa, lam, emit)
-                      : -PFEM_DEFER;
-            if (st == -PFEM_DEFER)      // nothing was emitted
-                st = node_quadratic<P, R, double, REFINE_NONE, true>(f, np, tri, sa, lam, emit);
+                    if (c < f.C) acc[c] = group_sum<Q>(acc[c]);
+            }
         }
+        if (q != 0) continue;
         if (st != 0) {
             record_error(f.status, -st, node);
 #pragma unroll
@@ -862,17 +942,24 @@ __global__ void __launch_bounds__(128) k_p2m_fix_tab(P2MArgs a, StarTab t)
 // of the mesh's 2-norm; the two results differ by 1e-9 of it).  The float-float refinement that
 // PFEM_SOLVE_F32_REFINED_FF names (48 bits, about 200 FP32 instructions a point and edge) took
 // 0.84 ms in two kernels; it takes this path too, whose residual is the more exact.
-// Resident blocks per SM: 8 (64 registers).
-#ifndef PFEM_TAB_MIN_BLOCKS
-#define PFEM_TAB_MIN_BLOCKS 8
-#endif
-template <typename S> constexpr int tab_min_blocks() { return sizeof(S) == 8 ? 4 : PFEM_TAB_MIN_BLOCKS; }
+// Resident 128-thread blocks per SM: 9 with one lane a node (1025^2 / 2048^2 round trip: 7, 8, 9, 10
+// blocks 1220, 1210, 1195, 1201 us), and for the solution refined to FP64, with its longer live
+// ranges, 6 (513^2 / 1024^2: 4, 5, 6 blocks 739, 713, 700 us); 8 and 4 with four lanes a node, where
+// there are not enough nodes to fill the SMs.
+template <int REFINE, int Q = 1> constexpr int tab_min_blocks()
+{
+    return REFINE == REFINE_FIX64 ? (Q > 1 ? 4 : 6) : (Q > 1 ? 8 : 9);
+}
 
 // Node (I, J) of the problem of a (mesh output a.out; queue entries and error details at node
-// a.noff + J * a.n + I of the batch).
-template <typename P, typename V, typename R, typename S, int REFINE>
+// a.noff + J * a.n + I of the batch), by Q = 1 lane, or by Q = 4 lanes that all locate it, solve an
+// edge each (the fourth none) and take the components c = q, q + 4 of the apply.  Both give the same
+// result bit for bit: the edges' contributions and the particles are added up in the same order.
+template <typename P, typename V, typename R, typename S, int REFINE, int Q = 1>
 __device__ __forceinline__ void tab_node(const P2MArgs &a, const StarTab &t, int I, int J)
 {
+    const int q = Q > 1 ? (int)threadIdx.x & (Q - 1) : 0;
+    const int e0 = Q > 1 ? q : 0, e1 = Q > 1 ? min(q + 1, 3) : 3;
     const int nc = a.n - 1;
     const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
     const long long node = (long long)J * a.n + I;
@@ -886,9 +973,23 @@ __device__ __forceinline__ void tab_node(const P2MArgs &a, const StarTab &t, int
             sa[e] = tab_star(t, tri[e]);
             if (sa[e].n < 0) st = sa[e].n == -1 ? -PFEM_FAR : sa[e].n;
         }
-    R acc[8];
+    R acc[8];                   // all components (Q = 1), or q, q + 4
 #pragma unroll
     for (int c = 0; c < 8; ++c) acc[c] = R(0);
+    auto apply = [&](int s, R w) {
+        if constexpr (Q == 1) {
+            R v[8];
+            load_vals<V, R>((const V *)a.vals, a.perm, s, a.C, v);
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c < a.C) acc[c] = fma(w, v[c], acc[c]);
+        } else {
+            const V *p = (const V *)a.vals + (a.perm ? (long long)__ldg(a.perm + s) : (long long)s) * a.C;
+#pragma unroll
+            for (int k = 0; k < 8 / Q; ++k)
+                if (q + Q * k < a.C) acc[k] = fma(w, load_val<V, R>(p + q + Q * k), acc[k]);
+        }
+    };
     if (st == 0) {
         NodePos<P, R> np;
         np.init(Iu, Ju, nc);
@@ -900,38 +1001,69 @@ __device__ __forceinline__ void tab_node(const P2MArgs &a, const StarTab &t, int
         int vi[3];
         if (node_u_sets<UMAX>(tri, sa, us, nu, vm, vi, min(a.ucap, UMAX)) != 0) {
             st = a.defer_cap > 0 ? -PFEM_DEFER : -PFEM_ERR_CAPACITY;
+        } else if constexpr (REFINE == REFINE_FIX64) {
+            longlong2 o[UMAX];
+            long long w[UMAX];
+            node_offsets64<P>(a.pos, Iu, Ju, nc, us, nu, o);
+            for (int i = 0; i < nu; ++i) w[i] = 0;
+            const double l64[3] = {(double)lam[0], (double)lam[1], (double)lam[2]};
+            st = group_min<Q>(node_solve64(o, vm, vi, l64, e0, e1, w, -PFEM_DEFER));
+            if (st == 0) {
+                for (int i = 0; i < nu; ++i)
+                    apply(us[i], (R)(__ll2double_rn(group_sum<Q>(w[i])) * W64_UNIT));
+#pragma unroll
+                for (int e = 0; e < 3; ++e) apply(tri[e], lam[e]);
+            }
         } else {
             R uw[UMAX];
             for (int i = 0; i < nu; ++i) uw[i] = R(0);
+            if constexpr (Q == 1) {
 #pragma unroll
-            for (int e = 0; e < 3; ++e) uw[vi[e]] += lam[e];
-            st = node_u_solve<P, R, S, REFINE, false, UMAX>(a, np, us, uw, vm, vi, lam);
-            if (st == 0)
-                for (int i = 0; i < nu; ++i) {
-                    R v[8];
-                    load_vals<V, R>((const V *)a.vals, a.perm, us[i], a.C, v);
+                for (int e = 0; e < 3; ++e) uw[vi[e]] += lam[e];
+                st = node_u_solve<P, R, S, REFINE, false, UMAX>(a, np, us, uw, vm, vi, lam);
+                if (st == 0)
+                    for (int i = 0; i < nu; ++i) apply(us[i], uw[i]);
+            } else {
+                st = group_min<Q>(node_u_solve<P, R, S, REFINE, false, UMAX, true>(a, np, us, uw, vm, vi,
+                                                                                   lam, e0, e1));
+                const R coef[3] = {R(2) * lam[0] * lam[1], R(2) * lam[1] * lam[2], R(2) * lam[2] * lam[0]};
+                if (st == 0)
+                    for (int i = 0; i < nu; ++i) {
+                        R w = i == vi[0] ? lam[0] : i == vi[1] ? lam[1] : i == vi[2] ? lam[2] : R(0);
 #pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        if (c < a.C) acc[c] = fma(uw[i], v[c], acc[c]);
-                }
+                        for (int e = 0; e < 3; ++e)
+                            w = fma(coef[e], __shfl_sync(group_mask<Q>(), uw[i], e, Q), w);
+                        apply(us[i], w);
+                    }
+            }
         }
     }
     if (st != 0) {
-        st = defer_or_error(a, st, a.noff + node);
-        if (st < 0) record_error(a.status, -st, a.noff + node);
+        if (q == 0) {
+            st = defer_or_error(a, st, a.noff + node);
+            if (st < 0) record_error(a.status, -st, a.noff + node);
+        }
 #pragma unroll
         for (int c = 0; c < 8; ++c) acc[c] = (R)nan_of<R>();
     }
-    store_vals<V, R>((V *)a.out, node, a.C, acc);
+    if constexpr (Q == 1) {
+        store_vals<V, R>((V *)a.out, node, a.C, acc);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8 / Q; ++k)
+            if (q + Q * k < a.C) store_val<V, R>((V *)a.out + node * a.C + q + Q * k, acc[k]);
+    }
 }
 
-template <typename P, typename V, typename R, typename S, int REFINE>
-__global__ void __launch_bounds__(128, tab_min_blocks<S>()) k_p2m_tab(P2MArgs a, StarTab t)
+template <typename P, typename V, typename R, typename S, int REFINE, int Q>
+__global__ void __launch_bounds__(128, tab_min_blocks<REFINE, Q>()) k_p2m_tab(P2MArgs a, StarTab t)
 {
-    const int I = blockIdx.x * 16 + (threadIdx.x & 15);
-    const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
+    // 16 x 8 nodes a block, or 8 x 4 with four lanes a node
+    const int x = threadIdx.x / Q;
+    const int I = blockIdx.x * (Q > 1 ? 8 : 16) + (Q > 1 ? x & 7 : x & 15);
+    const int J = blockIdx.y * (Q > 1 ? 4 : 8) + (Q > 1 ? x >> 3 : x >> 4);
     if (I >= a.n || J >= a.n) return;
-    tab_node<P, V, R, S, REFINE>(a, t, I, J);
+    tab_node<P, V, R, S, REFINE, Q>(a, t, I, J);
 }
 
 }  // namespace pfem

@@ -121,3 +121,32 @@ def test_stars_of_uneven_sets(P, which):
         assert mine[mine.index(min(mine)):] + mine[:mine.index(min(mine))] == \
             ref[ref.index(min(ref)):] + ref[:ref.index(min(ref))], s
         assert (nbrs[s, counts[s]:] == -1).all()
+
+
+@pytest.mark.parametrize("which", sorted(PROBLEMS) + ["quad_end", "quad_past"])
+def test_fp64_solves(P, which):
+    """The FP32 factor with the solution refined in 64-bit fixed point: FP64 values within the FP64
+    bound of the oracle and FP32 values within the FP32 bound, on both sides of the line between
+    four lanes and one lane a node, with positions from other periods of the torus."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    nodes = {"quad_end": 160 * sms, "quad_past": 160 * sms + 1}.get(which)
+    if nodes:
+        n = int(np.sqrt(nodes)) + (which == "quad_past")
+        pr = G.scaled_config("tg", n, 2 * (n - 1))
+    else:
+        pr = PROBLEMS[which]()
+    ref = O.p2m(pr.n, pr.pos, pr.vals, shape=1, nthreads=8)
+    for shift in ((0.0, 0.0), (-3.0, 5.0)):
+        pos = pr.pos + np.array(shift)
+        want = ref if shift[0] == 0.0 else O.p2m(pr.n, pos, pr.vals, shape=1, nthreads=8)
+        proj = P.Projector(pr.n, pr.N, C=pr.C, pos_dtype=torch.float64)
+        proj.build(torch.tensor(pos, device="cuda"))
+        mesh = proj.p2m(torch.tensor(pr.vals, device="cuda"))
+        proj.check(which)
+        assert relerr(mesh.cpu().numpy(), want) <= TOL64, shift
+    pos = torch.tensor(pr.pos, dtype=torch.float32, device="cuda")
+    proj = P.Projector(pr.n, pr.N, C=pr.C, pos_dtype=torch.float32)
+    proj.build(pos)
+    mesh = proj.p2m(torch.tensor(pr.vals, dtype=torch.float32, device="cuda"), solve=P.PFEM_SOLVE_F64)
+    proj.check(which)
+    assert relerr(mesh.cpu().numpy(), O.p2m(pr.n, pos.double().cpu().numpy(), pr.vals, shape=1, nthreads=8)) <= TOL32
