@@ -222,7 +222,8 @@ pfem_status pfem_delaunay_stars(pfem_ctx *ctx, int32_t nb, int64_t N, const uint
  * K <= PFEM_KW_MAX; a node with more distinct particles records PFEM_ERR_CAPACITY.
  * Used by the checkpointed backward and by pfem_project_p2m with given weights.
  * Quadratic shape functions: the workspace beyond its first 512 bytes holds a queue of the
- * nodes the fast solve cannot take (see pfem_project_p2m). */
+ * nodes the fast solve cannot take and, where it has room, the star table (see
+ * pfem_project_p2m). */
 pfem_status pfem_shape_quadratic(pfem_ctx *ctx, int32_t n, int32_t nb, int64_t N, const void *pos_sorted,
                                  pfem_dtype pos_t, const uint32_t *q_sorted,
                                  const int32_t *cell_start, pfem_shape shape, pfem_solve solve,

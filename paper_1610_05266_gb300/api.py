@@ -283,8 +283,10 @@ class Projector:
             torch.empty(max(N, 1), dtype=torch.int32, device=dev),
             torch.empty((max(N, 1), 2), dtype=pos_dtype, device=dev),
             torch.empty((max(N, 1), 2), dtype=torch.int32, device=dev),
-            torch.zeros((ws_bytes + 15) // 16 * 2, dtype=torch.float64, device=dev),
+            # only the status block needs to start as zeros
+            torch.empty((ws_bytes + 15) // 16 * 2, dtype=torch.float64, device=dev),
         )
+        self.reset_status()
 
     @property
     def ws(self) -> torch.Tensor:
@@ -357,9 +359,8 @@ class Projector:
         mode = PFEM_BACKWARD_CHECKPOINT if weights is not None else PFEM_BACKWARD_RECOMPUTE
         nbytes = pfem_backward_workspace_size(self.n, self.N, K)
         if getattr(self, "_bws", None) is None or self._bws.numel() * 8 < nbytes:
-            self._bws = torch.zeros((nbytes + 7) // 8, dtype=torch.float64, device=self.device)
-        else:
-            pfem_reset_status(self._bws, stream)
+            self._bws = torch.empty((nbytes + 7) // 8, dtype=torch.float64, device=self.device)
+        pfem_reset_status(self._bws, stream)
         gv = torch.empty_like(vals)
         gp = torch.empty((self.N, 2), dtype=vals.dtype, device=self.device) if want_pos else None
         pfem_project_backward(self.n, self.nb, self.N, c.pos_sorted, c.q_sorted, c.cell_start,

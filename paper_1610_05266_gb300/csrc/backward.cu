@@ -13,9 +13,17 @@
 // the derivative at a fixed frame is the derivative of A.
 //
 // Determinism without atomics on values: phase 1 writes each node's entries (slot, w, dpos)
-// into [n*n, K] arrays; phase 2 builds a transposed index by a stable counting sort keyed by
-// particle slot (entries per particle ordered by entry id) and gathers per particle.
+// into arrays of K entries a node; phase 2 builds a transposed index by a stable counting sort
+// keyed by particle slot (entries per particle ordered by entry id) and gathers per particle.
+//
+// The entries of phase 1 are laid out entry by entry (entry k of node i at k * nodes + i), only as
+// many as the node has, so that a warp's nodes write whole lines; weight and position adjoint of
+// an entry lie together, since the gather reads them together.  Phase 1 also counts the entries
+// of each particle as it writes them.  (Node by node, padded to K = 32 entries and counted by a
+// pass of its own, the solve kernel's scattered 4-byte stores bound it: 1040 us at 1025^2 nodes /
+// 2048^2 particles, C = 1, FP32, and 376 us for the transposed gather.)
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 #include "p2m.cuh"
@@ -26,10 +34,46 @@ struct BwdArgs {
     P2MArgs f;                  // forward geometry/values (f.out unused)
     const void *grad_mesh;      // [n*n, C]
     int K;                      // entries per node
-    int *e_slot;                // [n*n*K]
-    void *e_w;                  // [n*n*K] R
-    void *e_dpos;               // [n*n*K*2] R (may be null: value gradient only)
+    long long nodes;            // n*n
+    int *e_cnt;                 // [nodes] entries of the node
+    int *e_slot;                // [K][nodes]
+    int *e_rank;                // [K][nodes] arrival rank of the entry at its particle
+    void *e_val;                // [K][nodes] Entry<R>, or the weights alone (R) without positions
+    int *count;                 // [N] entries of the particle
 };
+
+// Weight and position adjoint of an entry: one 16-byte access in FP32.
+template <typename R> struct Entry;
+template <> struct __align__(16) Entry<float> {
+    float w, dx, dy, pad;
+};
+template <> struct Entry<double> {
+    double w, dx, dy;
+};
+// An entry's id in the transposed index: its node and its number.
+constexpr int ENTRY_BITS = 5;
+
+// Write the entries of a node (nu <= K).
+template <typename R, typename T, bool POS>
+__device__ __forceinline__ void write_entries(const BwdArgs &b, long long node, int nu, const int *us,
+                                              const T *uw, const T *udx, const T *udy)
+{
+    b.e_cnt[node] = nu;
+    for (int k = 0; k < nu; ++k) {
+        const long long e = k * b.nodes + node;
+        b.e_slot[e] = us[k];
+        b.e_rank[e] = atomicAdd(b.count + us[k], 1);
+        if constexpr (POS) {
+            Entry<R> v;
+            v.w = (R)uw[k];
+            v.dx = (R)udx[k];
+            v.dy = (R)udy[k];
+            ((Entry<R> *)b.e_val)[e] = v;
+        } else {
+            ((R *)b.e_val)[e] = (R)uw[k];
+        }
+    }
+}
 
 constexpr int KBWD = 32;   // distinct particles per node kept by the recompute kernel
 
@@ -164,17 +208,161 @@ __device__ __forceinline__ int bwd_u_solve(const BwdArgs &b, const NodePos<P, R>
     return st;
 }
 
-template <typename P, typename V, typename R, typename S, int SHAPE, bool POS>
-__device__ __forceinline__ void bwd_node(const BwdArgs &b, int I, int J)
+// bwd_u_solve for quadratic shape functions in FP64 without FP64 systems: y and z of each edge from the
+// FP32 factor, refined in 64-bit fixed point (fix64.cuh); what is left in FP64 is about 20
+// instructions a stencil point.  beta enters as 57-bit integers relative to the node's largest.
+template <typename P, typename V, typename R, bool POS>
+__device__ __forceinline__ int bwd_u_solve64(const BwdArgs &b, int Iu, int Ju, const R g[8], const int tri[3],
+                                             const int *us, int nu, const unsigned vm[3], const int vi[3],
+                                             R *uw, R *udx, R *udy)
 {
     const P2MArgs &a = b.f;
     const int nc = a.n - 1;
+    longlong2 o[UMAX];
+    const int L = node_offsets64<P>(a.pos, Iu, Ju, nc, us, nu, o);
+    long long bi[POS ? UMAX : 1];
+    double lbar[3] = {0.0, 0.0, 0.0}, bunit = 0.0;
+    if (POS) {
+        double bm = 0.0;
+        bool bad = false;
+        auto beta = [&](int i) {
+            R v[8];
+            load_vals<V, R>((const V *)a.vals, a.perm, us[i], a.C, v);
+            R t = R(0);
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c < a.C) t = fma(g[c], v[c], t);
+            return (double)t;
+        };
+        for (int i = 0; i < nu; ++i) {
+            const double t = beta(i);
+            bad |= !(fabs(t) < 1e290);           // infinities and NaN: left to the fix pass in FP64
+            bm = fmax(bm, fabs(t));
+            bi[i] = __double_as_longlong(t);
+#pragma unroll
+            for (int e = 0; e < 3; ++e)
+                if (i == vi[e]) lbar[e] = t;
+        }
+        if (bad) return -PFEM_DEFER;
+        // 2^(be - 1022) > bm: beta = bi 2^(be - 1078); without an upstream field beta = 0
+        const int be = max((__double2hiint(bm) >> 20) & 0x7ff, 200);
+        const double bs = __hiloint2double((1022 + 56 - be + 1023) << 20, 0);
+        bunit = __hiloint2double((be - 1022 + 1023) << 20, 0);       // of the scaled beta, 2^56
+        for (int i = 0; i < nu; ++i) bi[i] = __double2ll_rn(__longlong_as_double(bi[i]) * bs);
+    }
+    NodePos<P, R> np;
+    np.init(Iu, Ju, nc);
+    double d[3][2];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        R x, y;
+        np.off(a.pos, tri[e], x, y);
+        d[e][0] = (double)x;
+        d[e][1] = (double)y;
+    }
+    const double Na = d[1][0] * d[2][1] - d[1][1] * d[2][0];
+    const double Nb = d[2][0] * d[0][1] - d[2][1] * d[0][0];
+    const double Nc = d[0][0] * d[1][1] - d[0][1] * d[1][0];
+    const double A2 = Na + Nb + Nc;
+    const double lam[3] = {Na / A2, Nb / A2, Nc / A2};
+    // quadratic part first: it queues nodes
+#pragma unroll 1
+    for (int e = 0; e < 3; ++e) {
+        const int f = e == 2 ? 0 : e + 1;
+        EdgeSystem<UMAX> sys(o, vm[e] | vm[f], o[vi[e]], o[vi[f]]);
+        long long Y[6], Z[6], u[6] = {0, 0, 0, 0, 0, 0};
+        int sy, sz = 0;
+        if (!sys.factor() || !sys.solve_coefficients(Y, sy)) return -PFEM_DEFER;
+        const double yu = __hiloint2double((1023 - sy) << 20, 0), ce = 2.0 * lam[e] * lam[f];
+        EdgeFix64 Ey, Ez;
+        Ey.set(Y);
+        if constexpr (!POS) {
+            for (unsigned m = sys.mask; m; m &= m - 1) {
+                const int i = __ffs(m) - 1;
+                Split64 X, T;
+                sys.coords(i, X, T);
+                uw[i] += R(ce * (__ll2double_rn(Ey.value(X, T)) * yu));
+            }
+        } else {
+        for (unsigned m = sys.mask; m; m &= m - 1) {
+            const int i = __ffs(m) - 1;
+            Split64 X, T;
+            sys.coords(i, X, T);
+            const Split64 bt = split64(bi[i]);
+            const long long bx = mul64(X, bt), by = mul64(T, bt);
+            const Split64 xs = split64(bx), ys = split64(by);
+            u[0] += bi[i];
+            u[1] += bx;
+            u[2] += by;
+            u[3] += mul64(X, xs);
+            u[4] += mul64(T, xs);
+            u[5] += mul64(T, ys);
+        }
+        if (!sys.solve_adjoint(u, Z, sz)) return -PFEM_DEFER;
+        Ez.set(Z);
+        const double zu = __hiloint2double((1023 - sz) << 20, 0);
+        double y[6], z[6], Be = 0.0;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            y[q] = __ll2double_rn(Y[q]) * yu;
+            z[q] = __ll2double_rn(Z[q]) * zu;
+            Be = fma(__ll2double_rn(u[q]) * W64_UNIT, y[q], Be);
+        }
+        lbar[e] += 2.0 * lam[f] * Be * bunit;
+        lbar[f] += 2.0 * lam[e] * Be * bunit;
+        // X' = position * 2^(L + k + 1)
+        const double cp = ce * bunit * __hiloint2double((1023 + L + sys.k + 1) << 20, 0);
+        for (unsigned m = sys.mask; m; m &= m - 1) {
+            const int i = __ffs(m) - 1;
+            Split64 X, T;
+            sys.coords(i, X, T);
+            const double A = __ll2double_rn(Ey.value(X, T)) * yu, Zi = __ll2double_rn(Ez.value(X, T)) * zu;
+            uw[i] += R(ce * A);
+            const longlong2 p = o[i];
+            const double x = __ll2double_rn((2 * p.x - sys.mx) << sys.k) * 5.421010862427522e-20;   // 2^-64
+            const double t = __ll2double_rn((2 * p.y - sys.my) << sys.k) * 5.421010862427522e-20;
+            const double q = cp * (__ll2double_rn(bi[i]) * W64_UNIT - Zi), Aq = cp * A;
+            const double x2 = 2.0 * x, t2 = 2.0 * t;
+            udx[i] += R(q * fma(x2, y[3], fma(t, y[4], y[1])) - Aq * fma(x2, z[3], fma(t, z[4], z[1])));
+            udy[i] += R(q * fma(t2, y[5], fma(x, y[4], y[2])) - Aq * fma(t2, z[5], fma(x, z[4], z[2])));
+        }
+        // b' = -(1/2) (E'x^2, E'x E'y, E'y^2), E' = X' of the first end less that of the second
+        const double Ex = __ll2double_rn(sys.dx << sys.k) * 1.0842021724855044e-19;    // 2^-63: 2 X' of the first
+        const double Et = __ll2double_rn(sys.dy << sys.k) * 1.0842021724855044e-19;
+        const double exb = -cp * (Ex * z[3] + 0.5 * Et * z[4]);
+        const double eyb = -cp * (0.5 * Ex * z[4] + Et * z[5]);
+        udx[vi[e]] += R(exb);
+        udy[vi[e]] += R(eyb);
+        udx[vi[f]] -= R(exb);
+        udy[vi[f]] -= R(eyb);
+        }
+    }
+    for (int e = 0; e < 3; ++e) uw[vi[e]] += R(lam[e]);
+    if (POS) {
+        // lambda_k = N_k / A2 with N_a = d_b x d_c, N_b = d_c x d_a, N_c = d_a x d_b
+        const double Lam = lbar[0] * lam[0] + lbar[1] * lam[1] + lbar[2] * lam[2];
+        const double n0 = (lbar[0] - Lam) / A2, n1 = (lbar[1] - Lam) / A2, n2 = (lbar[2] - Lam) / A2;
+        udx[vi[0]] += R(n2 * d[1][1] - n1 * d[2][1]);
+        udy[vi[0]] += R(n1 * d[2][0] - n2 * d[1][0]);
+        udx[vi[1]] += R(n0 * d[2][1] - n2 * d[0][1]);
+        udy[vi[1]] += R(n2 * d[0][0] - n0 * d[2][0]);
+        udx[vi[2]] += R(n1 * d[0][1] - n0 * d[1][1]);
+        udy[vi[2]] += R(n0 * d[1][0] - n1 * d[0][0]);
+    }
+    return 0;
+}
+
+// Linear shape functions: the triangle's vertices are the entries.
+template <typename P, typename V, typename R, bool POS>
+__global__ void __launch_bounds__(128, PFEM_P2M_MIN_BLOCKS) k_bwd_linear(BwdArgs b)
+{
+    const P2MArgs &a = b.f;
+    const int I = blockIdx.x * 16 + (threadIdx.x & 15);
+    const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
+    if (I >= a.n || J >= a.n) return;
+    const int nc = a.n - 1;
     const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
     const long long node = (long long)J * a.n + I;
-    int *oslot = b.e_slot + node * b.K;
-    R *ow = (R *)b.e_w + node * b.K;
-    R *od = POS ? (R *)b.e_dpos + node * b.K * 2 : nullptr;
-
     R g[8];
     bool any = false;
 #pragma unroll
@@ -182,90 +370,36 @@ __device__ __forceinline__ void bwd_node(const BwdArgs &b, int I, int J)
         g[c] = c < a.C ? load_val<V, R>((const V *)b.grad_mesh + node * a.C + c) : R(0);
         any |= g[c] != R(0);
     }
-    // the node's distinct particles U: slot, weight, beta = gbar . alpha, position adjoint
-    int us[UMAX];
-    R uw[UMAX], ub[UMAX], udx[UMAX], udy[UMAX];
+    int us[3];
+    R uw[3] = {R(0), R(0), R(0)}, ub[3], udx[3] = {R(0), R(0), R(0)}, udy[3] = {R(0), R(0), R(0)};
     int nu = 0;
-    int st = 0;
     if (any) {
-        const uint2 qn = make_uint2(node_fx(Iu, nc), node_fx(Ju, nc));
-        int tri[3];
-        int stars[3][KMAX];
-        int ns[3] = {0, 0, 0};
-        st = locate(a.B, qn, a.R0, tri, stars[0], ns[0]);
-        if (SHAPE == PFEM_SHAPE_QUADRATIC && st == 0)
-            for (int e = 0; e < 3 && st == 0; ++e)
-                if (ns[e] == 0) {
-                    const int c = star_of(a.B, tri[e], a.R0, stars[e]);
-                    if (c < 0) st = c;
-                    else ns[e] = c;
-                }
+        int star[KMAX], ns;
+        int st = locate(a.B, make_uint2(node_fx(Iu, nc), node_fx(Ju, nc)), a.R0, us, star, ns);
         if (st == 0) {
             NodePos<P, R> np;
             np.init(Iu, Ju, nc);
-            bool over = false;
-            auto add = [&](int s) -> int {
-                for (int i = 0; i < nu; ++i)
-                    if (us[i] == s) return i;
-                if (nu == UMAX || nu == b.K) { over = true; return 0; }
-                us[nu] = s;
-                uw[nu] = udx[nu] = udy[nu] = R(0);
-                return nu++;
-            };
-            int vi[3];
-            unsigned vm[3] = {0u, 0u, 0u};
-#pragma unroll
-            for (int e = 0; e < 3; ++e) vi[e] = add(tri[e]);
-            if (SHAPE == PFEM_SHAPE_QUADRATIC)
-#pragma unroll
-                for (int e = 0; e < 3; ++e) {
-                    unsigned m = 1u << vi[e];
-                    for (int i = 0; i < ns[e]; ++i) m |= 1u << add(stars[e][i]);
-                    vm[e] = m;
-                }
-            if (over) st = -PFEM_DEFER;
-            if (st == 0)
-                st = bwd_u_solve<P, V, R, S, SHAPE, POS>(b, np, g, tri, us, nu, vm, vi, uw, ub,
-                                                         udx, udy);
-        }
-        if (st != 0) {
+            const int vi[3] = {0, 1, 2};
+            const unsigned vm[3] = {0u, 0u, 0u};
+            bwd_u_solve<P, V, R, R, PFEM_SHAPE_LINEAR, POS>(b, np, g, us, us, 3, vm, vi, uw, ub, udx, udy);
+            nu = 3;
+        } else {
             st = defer_or_error(a, st, node);
             if (st < 0) record_error(a.status, -st, node);
-            nu = 0;
         }
     }
-    for (int k = 0; k < b.K; ++k) {
-        const bool v = k < nu;
-        oslot[k] = v ? us[k] : -1;
-        ow[k] = v ? uw[k] : R(0);
-        if (POS) {
-            od[2 * k] = v ? udx[k] : R(0);
-            od[2 * k + 1] = v ? udy[k] : R(0);
-        }
-    }
+    write_entries<R, R, POS>(b, node, nu, us, uw, udx, udy);
 }
 
-template <typename P, typename V, typename R, typename S, int SHAPE, bool POS>
-__global__ void __launch_bounds__(128, PFEM_P2M_MIN_BLOCKS) k_bwd_node(BwdArgs b)
-{
-    const int I = blockIdx.x * 16 + (threadIdx.x & 15);
-    const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
-    if (I >= b.f.n || J >= b.f.n) return;
-    bwd_node<P, V, R, S, SHAPE, POS>(b, I, J);
-}
-
-// The adjoint with FP32 solves as two kernels, as in the forward: k_p2m_geom writes each
-// node's record (particle set, stencil masks), this kernel solves the adjoint of the three edge
-// systems with its own register budget and writes the node's entries.
+// The quadratic adjoint as two kernels: k_p2m_geom writes each node's record (particle set, stencil
+// masks), this kernel solves the adjoint of the three edge systems with its own register budget
+// and writes the node's entries.
 template <typename P, typename V, typename R, typename S, bool POS>
 __global__ void __launch_bounds__(128, 4) k_bwd_solve(BwdArgs b, NodeRecs r)
 {
     const P2MArgs &a = b.f;
     const long long node = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (node >= r.nodes) return;
-    int *oslot = b.e_slot + node * b.K;
-    R *ow = (R *)b.e_w + node * b.K;
-    R *od = POS ? (R *)b.e_dpos + node * b.K * 2 : nullptr;
     R g[8];
     bool any = false;
 #pragma unroll
@@ -274,7 +408,7 @@ __global__ void __launch_bounds__(128, 4) k_bwd_solve(BwdArgs b, NodeRecs r)
         any |= g[c] != R(0);
     }
     int us[UMAX];
-    R uw[UMAX], ub[UMAX], udx[UMAX], udy[UMAX];
+    R uw[UMAX], udx[UMAX], udy[UMAX];
     int nu = 0;
     const int meta = r.meta[node];
     if (any && meta >= 0) {
@@ -297,10 +431,17 @@ __global__ void __launch_bounds__(128, 4) k_bwd_solve(BwdArgs b, NodeRecs r)
             }
             const int nc = a.n - 1;
             const int I = (int)(node % a.n), J = (int)(node / a.n);
-            NodePos<P, R> np;
-            np.init(I == nc ? 0 : I, J == nc ? 0 : J, nc);
-            int st = bwd_u_solve<P, V, R, S, PFEM_SHAPE_QUADRATIC, POS>(
-                b, np, g, tri, us, nu, vm, vi, uw, ub, udx, udy);
+            int st;
+            if constexpr (sizeof(S) == 8) {
+                st = bwd_u_solve64<P, V, R, POS>(b, I == nc ? 0 : I, J == nc ? 0 : J, g, tri, us, nu, vm, vi,
+                                                 uw, udx, udy);
+            } else {
+                NodePos<P, R> np;
+                np.init(I == nc ? 0 : I, J == nc ? 0 : J, nc);
+                R ub[UMAX];
+                st = bwd_u_solve<P, V, R, S, PFEM_SHAPE_QUADRATIC, POS>(b, np, g, tri, us, nu, vm, vi, uw, ub,
+                                                                       udx, udy);
+            }
             if (st != 0) {
                 st = defer_or_error(a, st, node);
                 if (st < 0) record_error(a.status, -st, node);
@@ -308,15 +449,7 @@ __global__ void __launch_bounds__(128, 4) k_bwd_solve(BwdArgs b, NodeRecs r)
             }
         }
     }
-    for (int k = 0; k < b.K; ++k) {
-        const bool v = k < nu;
-        oslot[k] = v ? us[k] : -1;
-        ow[k] = v ? uw[k] : R(0);
-        if (POS) {
-            od[2 * k] = v ? udx[k] : R(0);
-            od[2 * k + 1] = v ? udy[k] : R(0);
-        }
-    }
+    write_entries<R, R, POS>(b, node, nu, us, uw, udx, udy);
 }
 
 // ---------------------------------------------------------------- fix pass
@@ -405,7 +538,9 @@ __device__ __forceinline__ void offset64(const void *pos, int s, double xn, doub
     dy = wrap1((double)py - yn);
 }
 
-template <typename P, typename V, typename R, int SHAPE, bool POS>
+// With CHOL (FP64 systems) a node first takes the FP64 Cholesky form of the adjoint, down to FP64's
+// pivot tolerance: it is queued where the FP32 factor cannot carry the fixed-point refinement.
+template <typename P, typename V, typename R, int SHAPE, bool POS, bool CHOL>
 __global__ void __launch_bounds__(64) k_bwd_fix(BwdArgs b)
 {
     const P2MArgs &a = b.f;
@@ -415,9 +550,6 @@ __global__ void __launch_bounds__(64) k_bwd_fix(BwdArgs b)
         const int I = (int)(node % a.n), J = (int)(node / a.n);
         const int nc = a.n - 1;
         const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
-        int *oslot = b.e_slot + node * b.K;
-        R *ow = (R *)b.e_w + node * b.K;
-        R *od = POS ? (R *)b.e_dpos + node * b.K * 2 : nullptr;
         double g[8];
         for (int c = 0; c < 8; ++c)
             g[c] = c < a.C ? (double)load_val<V, R>((const V *)b.grad_mesh + node * a.C + c) : 0.0;
@@ -455,6 +587,19 @@ __global__ void __launch_bounds__(64) k_bwd_fix(BwdArgs b)
                     vm[e] = m;
                 }
             if (over) st = -PFEM_ERR_CAPACITY;
+        }
+        if constexpr (CHOL) {
+            if (st == 0 && nu <= UMAX) {
+                NodePos<P, R> np;
+                np.init(Iu, Ju, nc);
+                R g1[8], w1[UMAX], b1[UMAX], x1[UMAX], y1[UMAX];
+                for (int c = 0; c < 8; ++c) g1[c] = (R)g[c];
+                for (int k = 0; k < nu; ++k) w1[k] = x1[k] = y1[k] = R(0);
+                if (bwd_u_solve<P, V, R, double, SHAPE, POS>(b, np, g1, tri, us, nu, vm, vi, w1, b1, x1, y1) == 0) {
+                    write_entries<R, R, POS>(b, node, nu, us, w1, x1, y1);
+                    continue;
+                }
+            }
         }
         if (st == 0) {
             // offsets from the node in FP64 (FP32 positions promoted, as the forward fix pass does)
@@ -557,19 +702,13 @@ __global__ void __launch_bounds__(64) k_bwd_fix(BwdArgs b)
             record_error(a.status, -st, node);
             nu = 0;
         }
-        for (int k = 0; k < b.K; ++k) {
-            const bool v = k < nu;
-            oslot[k] = v ? us[k] : -1;
-            ow[k] = v ? (R)uw[k] : R(0);
-            if (POS) {
-                od[2 * k] = v ? (R)udx[k] : R(0);
-                od[2 * k + 1] = v ? (R)udy[k] : R(0);
-            }
-        }
+        write_entries<R, double, POS>(b, node, nu, us, uw, udx, udy);
     }
 }
 
 // ---------------------------------------------------------------- transposed gather
+// Two sources of entries: given weights [nodes, K] (-1: unused; entry id = node * K + k), counted by
+// k_tr_count, and the entries that the node kernels wrote and counted (id = node << ENTRY_BITS | k).
 
 __global__ void k_tr_count(long long E, const int *__restrict__ slot, int *__restrict__ count,
                            int *__restrict__ rank)
@@ -591,28 +730,41 @@ __global__ void k_tr_scatter(long long E, const int *__restrict__ slot, const in
     }
 }
 
-__global__ void k_tr_sort(long long N, const int *__restrict__ start, int *order)
+__global__ void k_tr_scatter_nodes(long long nodes, const int *__restrict__ cnt, const int *__restrict__ slot,
+                                   const int *__restrict__ rank, const int *__restrict__ start,
+                                   int *__restrict__ order)
 {
-    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < N;
-         s += (long long)gridDim.x * blockDim.x) {
-        const int a = start[s], b = start[s + 1];
-        for (int i = a + 1; i < b; ++i) {
-            const int v = order[i];
-            int j = i - 1;
-            while (j >= a && order[j] > v) {
-                order[j + 1] = order[j];
-                --j;
-            }
-            order[j + 1] = v;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nodes;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int nu = cnt[i];
+        for (int k = 0; k < nu; ++k) {
+            const long long e = k * nodes + i;
+            order[__ldg(start + slot[e]) + rank[e]] = (int)(i << ENTRY_BITS | k);
         }
     }
 }
 
-// grad_vals[particle] = sum_e w_e gbar_node(e); grad_pos[particle] = sum_e dpos_e
-template <typename V, typename R, typename W>
-__global__ void k_tr_gather(long long N, int K, int C, const int *__restrict__ start,
-                            const int *__restrict__ order, const W *__restrict__ ew,
-                            const R *__restrict__ edpos, const V *__restrict__ grad_mesh,
+// The ids of one particle's entries in increasing order (arrival order before): f(id) for each.
+// Up to 16 are sorted in the thread, more in place.
+template <typename F> __device__ __forceinline__ void in_order(int *order, int n, F &&f)
+{
+    constexpr int LOCAL = 16;
+    int ids[LOCAL];
+    int *v = n <= LOCAL ? ids : order;
+    for (int i = 0; i < n; ++i) {
+        const int x = order[i];
+        int j = i - 1;
+        for (; j >= 0 && v[j] > x; --j) v[j + 1] = v[j];
+        v[j + 1] = x;
+    }
+    for (int i = 0; i < n; ++i) f(v[i]);
+}
+
+// grad_vals[particle] = sum_e w_e gbar_node(e); grad_pos[particle] = sum_e dpos_e.  NODES: the node
+// kernels' entries (val: Entry<R> with POS, else R), otherwise given weights (val: R).
+template <typename V, typename R, bool NODES, bool POS>
+__global__ void k_tr_gather(long long N, int K, long long nodes, int C, const int *__restrict__ start,
+                            int *order, const void *__restrict__ val, const V *__restrict__ grad_mesh,
                             const int *__restrict__ perm, V *__restrict__ grad_vals,
                             V *__restrict__ grad_pos)
 {
@@ -623,22 +775,27 @@ __global__ void k_tr_gather(long long N, int K, int C, const int *__restrict__ s
         for (int c = 0; c < 8; ++c) gv[c] = R(0);
         R gx = R(0), gy = R(0);
         const int a = __ldg(start + s), b = __ldg(start + s + 1);
-        for (int i = a; i < b; ++i) {
-            const int e = __ldg(order + i);
-            const long long node = e / K;
-            const R w = (R)__ldg(ew + e);
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < C) gv[c] = fma(w, load_val<V, R>(grad_mesh + node * C + c), gv[c]);
-            if (edpos) {
-                gx += __ldg(edpos + 2LL * e);
-                gy += __ldg(edpos + 2LL * e + 1);
+        in_order(order + a, b - a, [&](int id) {
+            const long long node = NODES ? id >> ENTRY_BITS : id / K;
+            const long long e = NODES ? (long long)(id & ((1 << ENTRY_BITS) - 1)) * nodes + node : id;
+            R w;
+            if constexpr (POS) {
+                const Entry<R> v = ((const Entry<R> *)val)[e];
+                w = v.w;
+                gx += v.dx;
+                gy += v.dy;
+            } else {
+                w = __ldg((const R *)val + e);
             }
-        }
+            if (grad_vals)
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (c < C) gv[c] = fma(w, load_val<V, R>(grad_mesh + node * C + c), gv[c]);
+        });
         const long long o = perm ? (long long)__ldg(perm + s) : s;
         if (grad_vals)
             for (int c = 0; c < C; ++c) store_val<V, R>(grad_vals + o * C + c, gv[c]);
-        if (grad_pos && edpos) {
+        if (POS) {
             store_val<V, R>(grad_pos + 2 * o, gx);
             store_val<V, R>(grad_pos + 2 * o + 1, gy);
         }
@@ -662,8 +819,7 @@ BwdLayout bwd_layout(int n, long long N, int Kw)
     const long long E = (long long)n * n * K;
     size_t off = 256;
     L.e_slot = off;  off = al(off + 4 * (size_t)E);
-    L.e_w = off;     off = al(off + 8 * (size_t)E);
-    L.e_dpos = off;  off = al(off + 16 * (size_t)E);
+    L.e_val = off;   off = al(off + 24 * (size_t)E);
     L.count = off;   off = al(off + 4 * (size_t)(N + 1));
     L.start = off;   off = al(off + 4 * (size_t)(N + 1));
     L.rank = off;    off = al(off + 4 * (size_t)E);
@@ -677,30 +833,46 @@ BwdLayout bwd_layout(int n, long long N, int Kw)
     return L;
 }
 
-// Phase 2 over entries (slot, w, dpos) laid out [n*n, K].
-template <typename V, typename R, typename W>
-static cudaError_t transposed_gather(int n, long long N, int K, int C, const int *e_slot,
-                                     const W *e_w, const R *e_dpos, const void *grad_mesh,
-                                     const int *perm, void *grad_vals, void *grad_pos,
-                                     const BwdLayout &L, char *ws, cudaStream_t s)
+// Phase 2: the transposed index of the entries, whose counts per particle are in L.count, and the
+// gather.
+template <typename V, typename R>
+static cudaError_t gather_nodes(const BwdArgs &b, long long N, int C, const int *perm, void *grad_vals,
+                                void *grad_pos, const BwdLayout &L, char *ws, cudaStream_t s)
 {
-    const long long E = (long long)n * n * K;
-    int *count = (int *)(ws + L.count);
-    int *start = (int *)(ws + L.start);
-    int *rank = (int *)(ws + L.rank);
-    int *order = (int *)(ws + L.order);
-    cudaError_t e = cudaMemsetAsync(count, 0, 4 * (size_t)(N + 1), s);
+    int *start = (int *)(ws + L.start), *order = (int *)(ws + L.order);
+    cudaError_t e = scan_exclusive(b.count, start, N + 1, (int *)(ws + L.scan), s);
     if (e != cudaSuccess) return e;
-    k_tr_count<<<grid1(E, 256), 256, 0, s>>>(E, e_slot, count, rank);
+    k_tr_scatter_nodes<<<grid1(b.nodes, 128), 128, 0, s>>>(b.nodes, b.e_cnt, b.e_slot, b.e_rank, start, order);
+    auto go = [&](auto pos) {
+        k_tr_gather<V, R, true, decltype(pos)::value><<<grid1(N, 128), 128, 0, s>>>(
+            N, b.K, b.nodes, C, start, order, b.e_val, (const V *)b.grad_mesh, perm, (V *)grad_vals,
+            (V *)grad_pos);
+    };
+    if (grad_pos) go(std::true_type());
+    else go(std::false_type());
+    count_launch(2);
+    return cudaGetLastError();
+}
+
+// The same from given weights [nodes, K]: the value gradient.
+template <typename V, typename R>
+static cudaError_t gather_weights(const BwdArgs &b, long long N, int K, int C, const int *w_idx, const R *w,
+                                  const int *perm, void *grad_vals, const BwdLayout &L, char *ws,
+                                  cudaStream_t s)
+{
+    const long long E = b.nodes * K;
+    int *start = (int *)(ws + L.start), *order = (int *)(ws + L.order);
+    cudaError_t e = cudaMemsetAsync(b.count, 0, 4 * (size_t)(N + 1), s);
+    if (e != cudaSuccess) return e;
+    k_tr_count<<<grid1(E, 256), 256, 0, s>>>(E, w_idx, b.count, b.e_rank);
     count_launch();
-    e = scan_exclusive(count, start, N + 1, (int *)(ws + L.scan), s);
+    e = scan_exclusive(b.count, start, N + 1, (int *)(ws + L.scan), s);
     if (e != cudaSuccess) return e;
-    k_tr_scatter<<<grid1(E, 256), 256, 0, s>>>(E, e_slot, rank, start, order);
-    k_tr_sort<<<grid1(N, 128), 128, 0, s>>>(N, start, order);
-    k_tr_gather<V, R, W><<<grid1(N, 128), 128, 0, s>>>(N, K, C, start, order, e_w, e_dpos,
-                                                       (const V *)grad_mesh, perm, (V *)grad_vals,
-                                                       (V *)grad_pos);
-    count_launch(3);
+    k_tr_scatter<<<grid1(E, 256), 256, 0, s>>>(E, w_idx, b.e_rank, start, order);
+    k_tr_gather<V, R, false, false><<<grid1(N, 128), 128, 0, s>>>(N, K, b.nodes, C, start, order, w,
+                                                                  (const V *)b.grad_mesh, perm,
+                                                                  (V *)grad_vals, (V *)nullptr);
+    count_launch(2);
     return cudaGetLastError();
 }
 
@@ -733,58 +905,55 @@ static cudaError_t bwd_t(const GeoArgs &g, const int *perm, int C, const void *v
     b.f.status = (DevStatus *)ws;
     b.grad_mesh = grad_mesh;
     b.K = K;
+    b.nodes = (long long)g.n * g.n;
     b.e_slot = (int *)(ws + L.e_slot);
-    b.e_w = ws + L.e_w;
-    b.e_dpos = ws + L.e_dpos;
+    b.e_rank = (int *)(ws + L.rank);
+    b.e_val = ws + L.e_val;
+    b.count = (int *)(ws + L.count);
     const dim3 grid((g.n + 15) / 16, (g.n + 7) / 8);
-    // per-node adjoint entries: the geometry and solve kernels for FP32 quadratic solves, else
-    // the single fused kernel
+    // the nodes' records (quadratic shape functions); a node's entry count takes the place of its
+    // record's head, which its thread has read by then
     NodeRecs recs;
-    node_recs_layout(ws + L.rec, (long long)g.n * g.n, &recs);
+    node_recs_layout(ws + L.rec, b.nodes, &recs);
+    b.e_cnt = recs.meta;
     // the star table's queue counter sits in the status block, after the status word
     const StarTab tab = star_tab_layout(ws + L.tab, g.N, (int *)(ws + 64));
-    const bool split = SHAPE == PFEM_SHAPE_QUADRATIC && sizeof(S) == sizeof(float);
     // the fix-pass queue: its counter in the status block, one entry per node
     b.f.defer_count = (int *)(ws + 68);
     b.f.defer_list = (long long *)(ws + L.queue);
-    b.f.defer_cap = (int)std::min((long long)g.n * g.n, (long long)0x7fffffff);
-    auto node_pass = [&](bool pos) {
+    b.f.defer_cap = (int)std::min(b.nodes, (long long)0x7fffffff);
+    auto node_pass = [&](auto pos) {
+        constexpr bool POS = decltype(pos)::value;
         cudaMemsetAsync(b.f.defer_count, 0, sizeof(int), s);
-        if (split) {
-            launch_star_table(b.f.B, g.R0, g.rmax_far, tab, b.f.status, s);
+        cudaMemsetAsync(b.count, 0, 4 * (size_t)(g.N + 1), s);
+        if constexpr (SHAPE == PFEM_SHAPE_QUADRATIC) {
+            // a star that no node needs may fail unnoticed with FP64 systems, whose adjoint has always
+            // looked at the needed ones only: a scratch status word
+            DevStatus *st = sizeof(S) == 8 ? (DevStatus *)(ws + 128) : b.f.status;
+            launch_star_table(b.f.B, g.R0, g.rmax_far, tab, st, s);
             k_p2m_geom<P, V, R><<<grid, 128, 0, s>>>(b.f, tab, recs);
-            const unsigned blocks = (unsigned)((recs.nodes + 127) / 128);
-            if (pos) k_bwd_solve<P, V, R, S, true><<<blocks, 128, 0, s>>>(b, recs);
-            else k_bwd_solve<P, V, R, S, false><<<blocks, 128, 0, s>>>(b, recs);
+            k_bwd_solve<P, V, R, S, POS><<<(unsigned)((b.nodes + 127) / 128), 128, 0, s>>>(b, recs);
             count_launch(2);
         } else {
-            if (pos) k_bwd_node<P, V, R, S, SHAPE, true><<<grid, 128, 0, s>>>(b);
-            else k_bwd_node<P, V, R, S, SHAPE, false><<<grid, 128, 0, s>>>(b);
+            k_bwd_linear<P, V, R, POS><<<grid, 128, 0, s>>>(b);
             count_launch();
         }
         // the queued nodes: widest search radius, FP64 SVD adjoint
         BwdArgs bf = b;
         bf.f.B.rmax = std::max(g.rmax, g.rmax_far);
-        if (pos) k_bwd_fix<P, V, R, SHAPE, true><<<num_sms() * 2, 64, 0, s>>>(bf);
-        else k_bwd_fix<P, V, R, SHAPE, false><<<num_sms() * 2, 64, 0, s>>>(bf);
+        k_bwd_fix<P, V, R, SHAPE, POS, SHAPE == PFEM_SHAPE_QUADRATIC && sizeof(S) == 8><<<num_sms() * 2, 64, 0, s>>>(bf);
         count_launch();
     };
     if (checkpoint) {
         // value gradient straight from the stored weights
-        cudaError_t e = transposed_gather<V, R, R>(g.n, g.N, Kw, C, w_idx, (const R *)w,
-                                                   (const R *)nullptr, grad_mesh, perm, grad_vals,
-                                                   nullptr, L, ws, s);
+        cudaError_t e = gather_weights<V, R>(b, g.N, Kw, C, w_idx, (const R *)w, perm, grad_vals, L, ws, s);
         if (e != cudaSuccess || !grad_pos) return e;
-        node_pass(true);
-        return transposed_gather<V, R, R>(g.n, g.N, K, C, b.e_slot, (const R *)b.e_w,
-                                          (const R *)b.e_dpos, grad_mesh, perm, nullptr, grad_pos,
-                                          L, ws, s);
+        node_pass(std::true_type());
+        return gather_nodes<V, R>(b, g.N, C, perm, nullptr, grad_pos, L, ws, s);
     }
-    if (!grad_pos) b.e_dpos = nullptr;
-    node_pass(grad_pos != nullptr);
-    return transposed_gather<V, R, R>(g.n, g.N, K, C, b.e_slot, (const R *)b.e_w,
-                                      grad_pos ? (const R *)b.e_dpos : nullptr, grad_mesh, perm,
-                                      grad_vals, grad_pos, L, ws, s);
+    if (grad_pos) node_pass(std::true_type());
+    else node_pass(std::false_type());
+    return gather_nodes<V, R>(b, g.N, C, perm, grad_vals, grad_pos, L, ws, s);
 }
 
 cudaError_t launch_p2m_backward(const GeoArgs &g, const int *perm, int C, const void *vals,

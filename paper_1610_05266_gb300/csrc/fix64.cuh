@@ -106,10 +106,10 @@ struct EdgeFix64 {
     }
 };
 
-// Offsets of a node's particles from it in fixed point, scaled up by a common power of two so that
-// every |offset| < 2^60: o[0..nu) in Q64.
+// Offsets of a node's particles from it in fixed point, scaled up by a common power of two 2^L so
+// that every |offset| < 2^60: o[0..nu) in Q64.  Returns L.
 template <typename P, int UM>
-__device__ __forceinline__ void node_offsets64(const void *pos, int Iu, int Ju, int nc, const int *us,
+__device__ __forceinline__ int node_offsets64(const void *pos, int Iu, int Ju, int nc, const int *us,
                                                int nu, longlong2 (&o)[UM])
 {
     const long long nx = node_fx64(Iu, nc), ny = node_fx64(Ju, nc);
@@ -126,7 +126,151 @@ __device__ __forceinline__ void node_offsets64(const void *pos, int Iu, int Ju, 
         if (L >= 0) o[i] = make_longlong2(o[i].x << L, o[i].y << L);
         else o[i] = make_longlong2(o[i].x >> -L, o[i].y >> -L);
     }
+    return L;
 }
+
+// One edge's system over the particles of `mask`: its FP32 factor, the units of the fixed point and the
+// refinement of a solution.  Coordinates are about the edge's midpoint, doubled: x = X 2^-63 in FP32, X'
+// = X 2^(k - 64) in fixed point, so X' = x 2^(k - 1).
+template <int UM> struct EdgeSystem {
+    const longlong2 (&o)[UM];
+    unsigned mask;
+    long long mx, my, dx, dy;           // midpoint doubled; half the edge = X of its first end
+    int k;
+    float ex, ey;                       // the edge in FP32 units
+    float c1;                           // 2^(1 - k)
+    Moment<float> M;
+
+    static __device__ __forceinline__ float pow2(int e) { return __int_as_float((e + 127) << 23); }
+
+    __device__ __forceinline__ EdgeSystem(const longlong2 (&off)[UM], unsigned m, longlong2 on, longlong2 os)
+        : o(off), mask(m), mx(on.x + os.x), my(on.y + os.y), dx(on.x - os.x), dy(on.y - os.y)
+    {
+    }
+
+    // Assemble and factor; false when the system is below the FP32 fast-solve tolerance.
+    __device__ __forceinline__ bool factor()
+    {
+        M.zero();
+        int hm = 0;
+        for (unsigned m = mask; m; m &= m - 1) {
+            const longlong2 p = o[__ffs(m) - 1];
+            const int hx = (int)((2 * p.x - mx) >> 32), hy = (int)((2 * p.y - my) >> 32);
+            hm = max(hm, max(hx ^ (hx >> 31), hy ^ (hy >> 31)));
+            M.add((float)hx * 4.656612873077393e-10f, (float)hy * 4.656612873077393e-10f);
+        }
+        ex = (float)dx * 2.168404344971009e-19f;
+        ey = (float)dy * 2.168404344971009e-19f;
+        const float l2 = fmaf(ex, ex, ey * ey);
+        // the tolerance of the system scaled by the edge length: pivots of degree d carry l^2d
+        const float i2 = 1.f / l2, i4 = i2 * i2;
+        const float tol = FastTol<float>::v *
+                          (M.m[tri_ix(0, 0)] + (M.m[tri_ix(1, 1)] + M.m[tri_ix(2, 2)]) * i2 +
+                           (M.m[tri_ix(3, 3)] + M.m[tri_ix(4, 4)] + M.m[tri_ix(5, 5)]) * i4);
+        const float t1 = tol * l2, t2 = t1 * l2;
+        const float tols[6] = {tol, t1, t1, t2, t2, t2};
+        // k: the left shift that brings the largest coordinate up to a half in Q64
+        k = __clz(hm + 1) - 1;
+        c1 = pow2(1 - k);
+        return M.factor_tol(tols) && k <= 20;
+    }
+
+    // factor of degree deg(q) from FP32 to fixed-point units of a solution
+    __device__ __forceinline__ float unit(int q) const { return q == 0 ? 1.f : q < 3 ? c1 : c1 * c1; }
+
+    __device__ __forceinline__ void coords(int i, Split64 &X, Split64 &Z) const
+    {
+        const longlong2 p = o[i];
+        X = split64((2 * p.x - mx) << k);
+        Z = split64((2 * p.y - my) << k);
+    }
+
+    // The unit 2^-s of a solution y (FP32 units) with right-hand side b (fixed-point units): |y'|, |b'| <=
+    // 2^(60 - s), at least 2^-most; false when it would be above 2^-20.  ym: the largest of them.
+    __device__ __forceinline__ bool range(const float y[6], const float b[6], int most, int &s, float &ym) const
+    {
+        ym = 0.f;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) ym = fmaxf(ym, fmaxf(fabsf(y[q] * unit(q)), fabsf(b[q])));
+        s = min(186 - (int)(__float_as_uint(ym) >> 23), most);
+        return s >= 20;
+    }
+
+    // Y = y in units 2^-s, refined until M' Y = B to the last bits.
+    __device__ __forceinline__ bool refine(const float y[6], int s, float ym, const long long B[6],
+                                           long long Y[6]) const
+    {
+        const float us = pow2(-s), sc = pow2(s - 60);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) Y[q] = __float2ll_rn(y[q] * unit(q) * sc * 1152921504606846976.0f);
+        EdgeFix64 E;
+        float last = ym;                 // the correction before
+        for (int it = 0; it < 12; ++it) {
+            E.set(Y);
+            long long r[6];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) r[q] = B[q];
+            for (unsigned m = mask; m; m &= m - 1) {
+                Split64 X, Z;
+                coords(__ffs(m) - 1, X, Z);
+                E.residual(X, Z, r);
+            }
+            float rf[6], d[6], dm = 0.f;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) rf[q] = __ll2float_rn(r[q]) * us * unit(q);
+            M.solve(rf, d);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                d[q] *= unit(q);
+                dm = fmaxf(dm, fabsf(d[q]));
+                Y[q] += __float2ll_rn(d[q] * sc * 1152921504606846976.0f);
+            }
+            // 2^-43: the next correction would be smaller by this one's ratio to the last; or the
+            // floor that the rounding of the residual sets, if it is below 2^-36
+            if (dm <= 1.1368683772161603e-13f * ym || (dm > 0.5f * last && dm <= 1.4551915228366852e-11f * ym))
+                return true;
+            last = dm;
+        }
+        return false;
+    }
+
+    // y of the coefficients: b = -(1/2) (ex^2, ex ey, ey^2) in the quadratic rows.
+    __device__ __forceinline__ bool solve_coefficients(long long Y[6], int &s) const
+    {
+        const float b[6] = {0.f, 0.f, 0.f, -0.5f * ex * ex, -0.5f * ex * ey, -0.5f * ey * ey};
+        float y[6];
+        M.solve(b, y);
+        const float ic2 = 1.f / (c1 * c1);
+        const float bf[6] = {0.f, 0.f, 0.f, b[3] * ic2, b[4] * ic2, b[5] * ic2};
+        float ym;
+        if (!range(y, bf, 62, s, ym)) return false;
+        const long long xn = dx << k, yn = dy << k;              // X' of the first end; b' = -2 (X'^2, X'Y', Y'^2)
+        const long long half = 1ll << (62 - s);
+        const long long B[6] = {0, 0, 0, -((__mul64hi(xn, xn) + half) >> (63 - s)),
+                                -((__mul64hi(xn, yn) + half) >> (63 - s)),
+                                -((__mul64hi(yn, yn) + half) >> (63 - s))};
+        return refine(y, s, ym, B, Y);
+    }
+
+    // z with M z = u, u' in units 2^-56 (|u'| < 2^7): the adjoint's right-hand side.
+    __device__ __forceinline__ bool solve_adjoint(const long long u[6], long long Z[6], int &s) const
+    {
+        float uf[6], ux[6], z[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            uf[q] = __ll2float_rn(u[q]) * 1.3877787807814457e-17f;
+            ux[q] = uf[q] * unit(q);
+        }
+        M.solve(ux, z);
+        float zm;
+        if (!range(z, uf, 110, s, zm)) return false;
+        long long B[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q)
+            B[q] = s >= 56 ? u[q] << (s - 56) : (u[q] + (1ll << (55 - s))) >> (56 - s);
+        return refine(z, s, zm, B, Z);
+    }
+};
 
 // Weights of the quadratic part in fixed point: w[i] += 2 lambda_nu lambda_sg A_{i e} 2^56 over the
 // edges e0 <= e < e1.  Returns 0, or -PFEM_DEFER for a system below the FP32 fast-solve
@@ -138,102 +282,23 @@ __device__ __forceinline__ int node_solve64(const longlong2 (&o)[UM], const unsi
                                             const int vi[3], const double lam[3], int e0, int e1,
                                             long long *w, int defer)
 {
-    auto pow2 = [](int e) { return __int_as_float((e + 127) << 23); };
 #pragma unroll 1
     for (int e = e0; e < e1; ++e) {
         const int f = e == 2 ? 0 : e + 1;
-        const unsigned mask = vm[e] | vm[f];
-        const longlong2 on = o[vi[e]], os = o[vi[f]];
-        const long long mx = on.x + os.x, my = on.y + os.y;
-        // FP32 system in units of 2^63: coordinates about the edge's midpoint, doubled
-        Moment<float> M;
-        M.zero();
-        int hm = 0;
-        for (unsigned m = mask; m; m &= m - 1) {
-            const longlong2 p = o[__ffs(m) - 1];
-            const int hx = (int)((2 * p.x - mx) >> 32), hy = (int)((2 * p.y - my) >> 32);
-            hm = max(hm, max(hx ^ (hx >> 31), hy ^ (hy >> 31)));
-            M.add((float)hx * 4.656612873077393e-10f, (float)hy * 4.656612873077393e-10f);
-        }
-        const long long dx = on.x - os.x, dy = on.y - os.y;      // half the edge, as X of nu
-        const float ex = (float)dx * 2.168404344971009e-19f, ey = (float)dy * 2.168404344971009e-19f;
-        const float l2 = fmaf(ex, ex, ey * ey);
-        // the tolerance of the system scaled by the edge length: pivots of degree d carry l^2d
-        const float i2 = 1.f / l2, i4 = i2 * i2;
-        const float tol = FastTol<float>::v *
-                          (M.m[tri_ix(0, 0)] + (M.m[tri_ix(1, 1)] + M.m[tri_ix(2, 2)]) * i2 +
-                           (M.m[tri_ix(3, 3)] + M.m[tri_ix(4, 4)] + M.m[tri_ix(5, 5)]) * i4);
-        const float t1 = tol * l2, t2 = t1 * l2;
-        const float tols[6] = {tol, t1, t1, t2, t2, t2};
-        if (!M.factor_tol(tols)) return defer;
-        const float b[6] = {0.f, 0.f, 0.f, -0.5f * ex * ex, -0.5f * ex * ey, -0.5f * ey * ey};
-        float y[6];
-        M.solve(b, y);
-        // to Q64: X' = x 2^(k - 1) with k the left shift that brings the largest coordinate up to
-        // a half; c[d]: the factor of degree d from the FP32 to the fixed-point units of y
-        const int k = __clz(hm + 1) - 1;
-        if (k > 20) return defer;
-        const float c1 = pow2(1 - k), c2 = c1 * c1;
-        const float c[6] = {1.f, c1, c1, c2, c2, c2};
-        const float ic1 = pow2(k - 1), ic2 = ic1 * ic1;
-        float ym = 0.f;
-#pragma unroll
-        for (int q = 0; q < 6; ++q) ym = fmaxf(ym, fmaxf(fabsf(y[q] * c[q]), fabsf(b[q] * ic2)));
-        const int bm = max((int)(__float_as_uint(ym) >> 23), 124);     // ym < 2^(bm - 126)
-        if (bm > 166) return defer;
-        const int s = 186 - bm;
-        const float us = pow2(-s), sc = pow2(s - 30);
-        long long Y[6], r[6], B[6];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) Y[q] = __float2ll_rn(y[q] * c[q] * sc * 1073741824.0f);
-        const long long xn = dx << k, yn = dy << k;              // X' of nu; b' = -2 (X'^2, X'Y', Y'^2)
-        B[0] = B[1] = B[2] = 0;
-        const long long half = 1ll << (62 - s);
-        B[3] = -((__mul64hi(xn, xn) + half) >> (63 - s));
-        B[4] = -((__mul64hi(xn, yn) + half) >> (63 - s));
-        B[5] = -((__mul64hi(yn, yn) + half) >> (63 - s));
-        auto coords = [&](int i, Split64 &X, Split64 &Z) {
-            const longlong2 p = o[i];
-            X = split64((2 * p.x - mx) << k);
-            Z = split64((2 * p.y - my) << k);
-        };
+        EdgeSystem<UM> sys(o, vm[e] | vm[f], o[vi[e]], o[vi[f]]);
+        long long Y[6];
+        int s;
+        if (!sys.factor() || !sys.solve_coefficients(Y, s)) return defer;
         EdgeFix64 E;
-        bool done = false;
-        float last = ym;                 // the correction before
-        for (int it = 0; it < 12 && !done; ++it) {
-            E.set(Y);
-#pragma unroll
-            for (int q = 0; q < 6; ++q) r[q] = B[q];
-            for (unsigned m = mask; m; m &= m - 1) {
-                Split64 X, Z;
-                coords(__ffs(m) - 1, X, Z);
-                E.residual(X, Z, r);
-            }
-            float rf[6], d[6], dm = 0.f;
-#pragma unroll
-            for (int q = 0; q < 6; ++q) rf[q] = __ll2float_rn(r[q]) * us * c[q];
-            M.solve(rf, d);
-#pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                d[q] *= c[q];
-                dm = fmaxf(dm, fabsf(d[q]));
-                Y[q] += __float2ll_rn(d[q] * sc * 1073741824.0f);
-            }
-            // 2^-43: the next correction would be smaller by this one's ratio to the last; or the
-            // floor that the rounding of the residual sets, if it is below 2^-36
-            done = dm <= 1.1368683772161603e-13f * ym || (dm > 0.5f * last && dm <= 1.4551915228366852e-11f * ym);
-            last = dm;
-        }
-        if (!done) return defer;
         E.set(Y);
         const double coef = 2.0 * lam[e] * lam[f];
         const Split64 cf = split64(__double2ll_rn(coef * 2305843009213693952.0));   // 2^61
         const int sh = W64_SHIFT + 3 - s;                        // product: coef A 2^(s - 3)
         int tm = 0;
-        for (unsigned m = mask; m; m &= m - 1) {
+        for (unsigned m = sys.mask; m; m &= m - 1) {
             const int i = __ffs(m) - 1;
             Split64 X, Z;
-            coords(i, X, Z);
+            sys.coords(i, X, Z);
             const long long t = E.value(X, Z);
             const int h = (int)(t >> 32);
             tm = max(tm, h ^ (h >> 31));
@@ -241,7 +306,7 @@ __device__ __forceinline__ int node_solve64(const longlong2 (&o)[UM], const unsi
             w[i] += sh >= 0 ? ct << sh : ct >> -sh;
         }
         // |A| <= (tm + 1) 2^(32 - s): keep the weights well inside their range
-        if (((float)tm + 1.f) * pow2(32 - s) * fabsf((float)coef) > 30.f) return defer;
+        if (((float)tm + 1.f) * EdgeSystem<UM>::pow2(32 - s) * fabsf((float)coef) > 30.f) return defer;
     }
     return 0;
 }

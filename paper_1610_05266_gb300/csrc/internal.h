@@ -118,7 +118,7 @@ cudaError_t launch_update_cells(int nb, long long N, const void *pos, pfem_dtype
 
 struct BwdLayout {
     int K;   // entries per node written by the recompute kernel
-    size_t e_slot, e_w, e_dpos, count, start, rank, order, scan, rec, tab, queue, total;   // rec: node records, tab: star table, queue: fix-pass nodes
+    size_t e_slot, e_val, count, start, rank, order, scan, rec, tab, queue, total;   // rec: node records, tab: star table, queue: fix-pass nodes
 };
 BwdLayout bwd_layout(int n, long long N, int K);
 

@@ -107,7 +107,18 @@ static cudaError_t go(const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
         e = cudaMemsetAsync(a.defer_count, 0, sizeof(int), s);
         if (e != cudaSuccess) return e;
     }
-    if (SHAPE == PFEM_SHAPE_QUADRATIC && !W && tab) {
+    if (SHAPE == PFEM_SHAPE_QUADRATIC && W && tab) {
+        if constexpr (SHAPE == PFEM_SHAPE_QUADRATIC && W) {
+            // a star that no node needs may fail unnoticed, as where each node searches its own: a
+            // scratch status word
+            e = launch_star_table(a.B, R0, rmax_far, *tab, (DevStatus *)((char *)a.status + 128), s);
+            if (e != cudaSuccess) return e;
+            const bool vec = a.K % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.w_idx) | reinterpret_cast<uintptr_t>(a.w)) & 31) == 0;
+            k_shape_tab<P, R, sizeof(S) == 8 ? REFINE_FIX64 : REF><<<node_grid(a.n), 128, 0, s>>>(a, *tab, vec);
+            count_launch();
+            e = cudaGetLastError();
+        }
+    } else if (SHAPE == PFEM_SHAPE_QUADRATIC && !W && tab) {
         e = launch_star_table(a.B, R0, rmax_far, *tab, a.status, s);
         if (e != cudaSuccess) return e;
         stage_event(g, 1, s);
@@ -187,34 +198,53 @@ cudaError_t launch_shape(const GeoArgs &g, pfem_shape shape, pfem_solve solve, i
     a.w_idx = w_idx;
     a.w = w;
     const bool q = shape == PFEM_SHAPE_QUADRATIC;
+    StarTab tab;
+    const StarTab *t = q && set_table(tab, st, ws_bytes, (long long)g.n * g.n, g.N) ? &tab : nullptr;
     if (w_t == PFEM_F64) {
         if (!q) return go<double, double, double, double, REFINE_NONE, 0, true>(g, a, s);
-        return go<double, double, double, double, REFINE_NONE, 1, true>(g, a, s);
+        return go<double, double, double, double, REFINE_NONE, 1, true>(g, a, s, t);
     }
     if (!q) return go<float, float, float, float, REFINE_NONE, 0, true>(g, a, s);
-    return go_solve<float, float, 1, true>(solve, g, a, s, nullptr);
+    return go_solve<float, float, 1, true>(solve, g, a, s, t);
 }
 
 // alpha_i = sum_k w[i,k] alpha[w_idx[i,k]] (explicit-weight P2M)
 template <typename V, typename R>
 __global__ void __launch_bounds__(256) k_apply(long long nodes, int K, const int *__restrict__ w_idx,
                                                const R *__restrict__ w, const int *__restrict__ perm,
-                                               int C, const V *__restrict__ vals, V *__restrict__ out)
+                                               int C, const V *__restrict__ vals, V *__restrict__ out,
+                                               bool vec)
 {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nodes;
          i += (long long)gridDim.x * blockDim.x) {
         R acc[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) acc[c] = R(0);
-        for (int k = 0; k < K; ++k) {
-            const int s = __ldg(w_idx + i * K + k);
-            if (s < 0) break;
-            const R wk = __ldg(w + i * K + k);
-            R v[8];
-            load_vals<V, R>(vals, perm, s, C, v);
+        for (int k = 0; k < K; k += 4) {
+            // four entries at a time (their loads in flight together), one 16-byte load of the slots
+            // where the rows allow it
+            int s[4];
+            if (vec) {
+                const int4 q = __ldg(reinterpret_cast<const int4 *>(w_idx + i * K + k));
+                s[0] = q.x; s[1] = q.y; s[2] = q.z; s[3] = q.w;
+            } else {
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < C) acc[c] = fma(wk, v[c], acc[c]);
+                for (int j = 0; j < 4; ++j) s[j] = k + j < K ? __ldg(w_idx + i * K + k + j) : -1;
+            }
+            // the row ends at its first -1
+#pragma unroll
+            for (int j = 1; j < 4; ++j) s[j] = s[j - 1] < 0 ? -1 : s[j];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (s[j] < 0) continue;
+                const R wk = __ldg(w + i * K + k + j);
+                R v[8];
+                load_vals<V, R>(vals, perm, s[j], C, v);
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (c < C) acc[c] = fma(wk, v[c], acc[c]);
+            }
+            if (s[3] < 0) break;
         }
         store_vals<V, R>(out, i, C, acc);
     }
@@ -227,16 +257,17 @@ cudaError_t launch_apply(int n, const int *perm, int C, const void *vals, pfem_d
     const long long nodes = (long long)n * n;
     long long blocks = (nodes + 255) / 256;
     if (blocks > num_sms() * 16LL) blocks = num_sms() * 16LL;
+    const bool vec = K % 4 == 0 && (reinterpret_cast<uintptr_t>(w_idx) & 15) == 0;
     if (val_t == PFEM_F64 && w_t == PFEM_F64)
         k_apply<double, double><<<(unsigned)blocks, 256, 0, s>>>(
-            nodes, K, w_idx, (const double *)w, perm, C, (const double *)vals, (double *)out);
+            nodes, K, w_idx, (const double *)w, perm, C, (const double *)vals, (double *)out, vec);
     else if (val_t == PFEM_F32 && w_t == PFEM_F32)
         k_apply<float, float><<<(unsigned)blocks, 256, 0, s>>>(
-            nodes, K, w_idx, (const float *)w, perm, C, (const float *)vals, (float *)out);
+            nodes, K, w_idx, (const float *)w, perm, C, (const float *)vals, (float *)out, vec);
     else if (val_t == PFEM_BF16 && w_t == PFEM_F32)
         k_apply<__nv_bfloat16, float><<<(unsigned)blocks, 256, 0, s>>>(
             nodes, K, w_idx, (const float *)w, perm, C, (const __nv_bfloat16 *)vals,
-            (__nv_bfloat16 *)out);
+            (__nv_bfloat16 *)out, vec);
     else
         return cudaErrorInvalidValue;
     count_launch();

@@ -9,6 +9,8 @@
 // and alpha_i = sum_mu w_{i mu} alpha_mu for every field component in one pass.
 #pragma once
 
+#include <type_traits>
+
 #include "fix64.cuh"
 #include "geom.cuh"
 #include "moments.cuh"
@@ -1064,6 +1066,86 @@ __global__ void __launch_bounds__(128, tab_min_blocks<REFINE, Q>()) k_p2m_tab(P2
     const int J = blockIdx.y * (Q > 1 ? 4 : 8) + (Q > 1 ? x >> 3 : x >> 4);
     if (I >= a.n || J >= a.n) return;
     tab_node<P, V, R, S, REFINE, Q>(a, t, I, J);
+}
+
+// Explicit weights of every node with the star table: as k_p2m_tab, writing the node's row of (slot,
+// weight) pairs, -1 and 0 past them.  vec: rows that 16-byte stores can write.
+template <typename P, typename R, int REFINE>
+__global__ void __launch_bounds__(128, tab_min_blocks<REFINE>()) k_shape_tab(P2MArgs a, StarTab t, bool vec)
+{
+    const int I = blockIdx.x * 16 + (threadIdx.x & 15);
+    const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
+    if (I >= a.n || J >= a.n) return;
+    const int nc = a.n - 1;
+    const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
+    const long long node = (long long)J * a.n + I;
+    int tri[3];
+    int st = locate_tab(a.B, t, make_uint2(node_fx(Iu, nc), node_fx(Ju, nc)), a.R0, tri);
+    TabStar sa[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+        if (st == 0) {
+            sa[e] = tab_star(t, tri[e]);
+            if (sa[e].n < 0) st = sa[e].n == -1 ? -PFEM_FAR : sa[e].n;
+        }
+    int us[UMAX];
+    R uw[UMAX];
+    int nu = 0;
+    if (st == 0) {
+        NodePos<P, R> np;
+        np.init(Iu, Ju, nc);
+        R lam[3];
+        barycentric(a, np, tri, lam);
+        unsigned vm[3];
+        int vi[3];
+        if (node_u_sets<UMAX>(tri, sa, us, nu, vm, vi, min(a.ucap, UMAX)) != 0) {
+            st = -PFEM_DEFER;
+        } else if constexpr (REFINE == REFINE_FIX64) {
+            longlong2 o[UMAX];
+            long long w[UMAX];
+            node_offsets64<P>(a.pos, Iu, Ju, nc, us, nu, o);
+            for (int i = 0; i < nu; ++i) w[i] = 0;
+            const double l64[3] = {(double)lam[0], (double)lam[1], (double)lam[2]};
+            st = node_solve64(o, vm, vi, l64, 0, 3, w, -PFEM_DEFER);
+            for (int i = 0; i < nu; ++i) uw[i] = (R)(__ll2double_rn(w[i]) * W64_UNIT);
+#pragma unroll
+            for (int e = 0; e < 3; ++e) uw[vi[e]] += lam[e];
+        } else {
+            for (int i = 0; i < nu; ++i) uw[i] = R(0);
+#pragma unroll
+            for (int e = 0; e < 3; ++e) uw[vi[e]] += lam[e];
+            st = node_u_solve<P, R, float, REFINE, false, UMAX>(a, np, us, uw, vm, vi, lam);
+        }
+        if (st == 0 && nu > a.K) st = -PFEM_ERR_CAPACITY;
+    }
+    if (st != 0) {
+        st = defer_or_error(a, st, node);
+        if (st < 0) record_error(a.status, -st, node);
+        nu = 0;
+    }
+    int *oi = a.w_idx + node * a.K;
+    R *ow = (R *)a.w + node * a.K;
+    if (vec) {
+        using V4 = std::conditional_t<sizeof(R) == 4, float4, double4>;
+        for (int k = 0; k < a.K; k += 4) {
+            int s[4];
+            R w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                s[i] = k + i < nu ? us[k + i] : -1;
+                w[i] = k + i < nu ? uw[k + i] : R(0);
+            }
+            *reinterpret_cast<int4 *>(oi + k) = make_int4(s[0], s[1], s[2], s[3]);
+            V4 v;
+            v.x = w[0]; v.y = w[1]; v.z = w[2]; v.w = w[3];
+            *reinterpret_cast<V4 *>(ow + k) = v;
+        }
+    } else {
+        for (int k = 0; k < a.K; ++k) {
+            oi[k] = k < nu ? us[k] : -1;
+            ow[k] = k < nu ? uw[k] : R(0);
+        }
+    }
 }
 
 }  // namespace pfem
