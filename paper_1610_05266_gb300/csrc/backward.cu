@@ -354,8 +354,10 @@ __device__ __forceinline__ int bwd_u_solve64(const BwdArgs &b, int Iu, int Ju, c
 
 // Linear shape functions: the triangle's vertices are the entries.
 template <typename P, typename V, typename R, bool POS>
-__global__ void __launch_bounds__(128, PFEM_P2M_MIN_BLOCKS) k_bwd_linear(BwdArgs b)
+__global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_bwd_linear(BwdArgs b)
 {
+    __shared__ float2 sxy[STAR_ROWS * STAR_TPB];
+    __shared__ int ss[STAR_ROWS * STAR_TPB];
     const P2MArgs &a = b.f;
     const int I = blockIdx.x * 16 + (threadIdx.x & 15);
     const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
@@ -374,8 +376,8 @@ __global__ void __launch_bounds__(128, PFEM_P2M_MIN_BLOCKS) k_bwd_linear(BwdArgs
     R uw[3] = {R(0), R(0), R(0)}, ub[3], udx[3] = {R(0), R(0), R(0)}, udy[3] = {R(0), R(0), R(0)};
     int nu = 0;
     if (any) {
-        int star[KMAX], ns;
-        int st = locate(a.B, make_uint2(node_fx(Iu, nc), node_fx(Ju, nc)), a.R0, us, star, ns);
+        int st = locate_hull(a.B, make_uint2(node_fx(Iu, nc), node_fx(Ju, nc)), a.R0,
+                             HullList{sxy + threadIdx.x, ss + threadIdx.x}, us);
         if (st == 0) {
             NodePos<P, R> np;
             np.init(Iu, Ju, nc);
@@ -892,6 +894,7 @@ static cudaError_t bwd_t(const GeoArgs &g, const int *perm, int C, const void *v
     b.f.B.dmax = g.dmax;
     b.f.B.kcap = g.kcap;
     b.f.B.walk_cap = g.walk_cap;
+    b.f.B.last4 = g.N >= 4 ? (int)(g.N - 4) : -1;
     b.f.ucap = g.ucap;
     b.f.R0 = g.R0;
     b.f.pos = g.pos_sorted;

@@ -83,7 +83,8 @@ __device__ __forceinline__ int find_problem(int P, long long x, F &&off)
 }
 
 // Bins and search radii of problem d within the batch's concatenated arrays.
-__device__ __forceinline__ void problem_args(P2MArgs &a, const P2MArgs &base, const BDesc &d)
+__device__ __forceinline__ void problem_args(P2MArgs &a, const P2MArgs &base, const BDesc &d,
+                                             long long total)
 {
     a = base;
     a.n = d.n;
@@ -93,6 +94,8 @@ __device__ __forceinline__ void problem_args(P2MArgs &a, const P2MArgs &base, co
     a.B.dmax = d.dmax;
     a.R0 = d.R0;
     a.noff = d.noff;
+    // slots are batch-wide, and a batch has at least three particles a problem
+    a.B.last4 = (int)(total - 4);
 }
 
 template <typename V>
@@ -149,7 +152,7 @@ __device__ __forceinline__ bool totals_ok(const BPlanDev *pl, long long nodes, c
     return ok;
 }
 
-// Per-node fused P2M (linear shape functions, or no room for the table) in a persistent loop.
+// Per-node fused P2M in a persistent loop: quadratic shape functions without room for the table.
 template <typename P, typename V, typename R, typename S, int REFINE, int SHAPE>
 __global__ void __launch_bounds__(256, PFEM_P2M_MIN_BLOCKS / 2) k_p2m_batch(const BPlanDev *pl, int shape_idx, P2MArgs base,
                             unsigned long long *counter)
@@ -172,9 +175,44 @@ __global__ void __launch_bounds__(256, PFEM_P2M_MIN_BLOCKS / 2) k_p2m_batch(cons
         const int J = (int)(t / tiles_x) * TY + (threadIdx.x >> 4);
         if (I >= d.n || J >= d.n) continue;
         P2MArgs a;
-        problem_args(a, base, d);
+        problem_args(a, base, d, pl->total_particles);
         problem_out<V>(a, base, d);
         p2m_node<P, V, R, S, REFINE, SHAPE, false>(a, I, J);
+    }
+}
+
+// Linear shape functions of every problem in a persistent loop.  Blocks of up to 256 threads share
+// the lists of two 128-thread columns.
+template <typename P, typename V, typename R>
+__global__ void __launch_bounds__(256) k_p2m_batch_linear(const BPlanDev *pl, int shape_idx, P2MArgs base,
+                                                          unsigned long long *counter)
+{
+    extern __shared__ __align__(16) unsigned char lists[];
+    __shared__ long long item;
+    const int half = threadIdx.x / STAR_TPB, lane = threadIdx.x % STAR_TPB;
+    constexpr int BYTES = STAR_ROWS * STAR_TPB * (int)(sizeof(float2) + sizeof(int));
+    float2 *xy = reinterpret_cast<float2 *>(lists + half * BYTES);
+    const HullList L{xy + lane, reinterpret_cast<int *>(xy + STAR_ROWS * STAR_TPB) + lane};
+    const int TY = blockDim.x / 16;
+    const long long total = pl->n_items[shape_idx];
+    const long long *tp = plan_tiles(pl, shape_idx);
+    for (int guard = 0; guard < (1 << 30); ++guard) {
+        __syncthreads();
+        if (threadIdx.x == 0) item = (long long)atomicAdd(counter, 1ull);
+        __syncthreads();
+        const long long it = item;
+        if (it >= total) break;
+        const int p = find_item(tp, pl->P, it);
+        const BDesc d = plan_desc(pl)[p];
+        const long long t = it - tp[p];
+        const int tiles_x = (d.n + 15) / 16;
+        const int I = (int)(t % tiles_x) * 16 + (threadIdx.x & 15);
+        const int J = (int)(t / tiles_x) * TY + (threadIdx.x >> 4);
+        if (I >= d.n || J >= d.n) continue;
+        P2MArgs a;
+        problem_args(a, base, d, pl->total_particles);
+        problem_out<V>(a, base, d);
+        linear_node<P, V, R, false>(a, L, I, J);
     }
 }
 
@@ -193,7 +231,7 @@ __global__ void __launch_bounds__(BSTAR, PFEM_STAR_MIN_BLOCKS) k_star_list_batch
         const long long i = (b - sp[p]) * BSTAR + threadIdx.x;
         if (i >= d.N) continue;
         P2MArgs a;
-        problem_args(a, base, d);
+        problem_args(a, base, d, pl->total_particles);
         const HullList L{sxy + threadIdx.x, ss + threadIdx.x};
         star_list_slot(a.B, a.R0, t, d.poff + i, L, a.status);
     }
@@ -214,7 +252,7 @@ __global__ void __launch_bounds__(RETRY_TPB, PFEM_RETRY_BLOCKS) k_star_retry_bat
         const int p = find_problem(pl->P, v, [&](int k) { return D[k].poff; });
         const BDesc d = D[p];
         P2MArgs a;
-        problem_args(a, base, d);
+        problem_args(a, base, d, pl->total_particles);
         a.B.rmax = max(d.rmax, d.nb / 4 - 1);
         star_retry_slot(a.B, a.R0, t, v, L, a.status);
     }
@@ -246,7 +284,7 @@ __global__ void __launch_bounds__(256, tab_min_blocks<REFINE>() / 2) k_p2m_batch
         const int J = (int)(t / tiles_x) * TY + (threadIdx.x >> 4);
         if (I >= d.n || J >= d.n) continue;
         P2MArgs a;
-        problem_args(a, base, d);
+        problem_args(a, base, d, pl->total_particles);
         problem_out<V>(a, base, d);
         tab_node<P, V, R, S, REFINE>(a, tab, I, J);
     }
@@ -264,7 +302,7 @@ __global__ void __launch_bounds__(128) k_p2m_fix_batch(const BPlanDev *pl, P2MAr
         const int p = find_problem(pl->P, g, [&](int k) { return D[k].noff; });
         const BDesc d = D[p];
         P2MArgs a;
-        problem_args(a, base, d);
+        problem_args(a, base, d, pl->total_particles);
         problem_out<V>(a, base, d);
         a.defer_cap = 0;
         a.B.rmax = max(d.rmax, d.nb / 4 - 1);
@@ -428,10 +466,17 @@ static cudaError_t p2m_batch_t(const void *plan, const P2MArgs &base, int shape_
             pl, shape_idx, base, counter, w.tab, w.nodes);
         count_launch(3);
     } else {
-        constexpr bool F64 = sizeof(S) == 8 && SHAPE == PFEM_SHAPE_QUADRATIC;
-        k_p2m_batch<P, V, R, std::conditional_t<F64, float, S>, F64 ? REFINE_FIX64 : REF, SHAPE>
-            <<<blocks, 16 * TYs[shape_idx], 0, s>>>(
-            pl, shape_idx, base, counter);
+        const int threads = 16 * TYs[shape_idx];
+        if constexpr (SHAPE == PFEM_SHAPE_LINEAR) {
+            const size_t lists = (size_t)((threads + STAR_TPB - 1) / STAR_TPB) * STAR_ROWS * STAR_TPB * (sizeof(float2) + sizeof(int));
+            e = cudaFuncSetAttribute(k_p2m_batch_linear<P, V, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lists);
+            if (e != cudaSuccess) return e;
+            k_p2m_batch_linear<P, V, R><<<blocks, threads, lists, s>>>(pl, shape_idx, base, counter);
+        } else {
+            constexpr bool F64 = sizeof(S) == 8;
+            k_p2m_batch<P, V, R, std::conditional_t<F64, float, S>, F64 ? REFINE_FIX64 : REF, SHAPE>
+                <<<blocks, threads, 0, s>>>(pl, shape_idx, base, counter);
+        }
         count_launch();
     }
     e = cudaGetLastError();

@@ -32,6 +32,7 @@ struct Bins {
     float dmax;                       // candidate distance cutoff of the first attempt (fixed point)
     int kcap = KMAX;                  // largest star kept (<= KMAX); larger: PFEM_ERR_CAPACITY
     int walk_cap = 64;                // visibility-walk steps before PFEM_ERR_TIMEOUT
+    int last4 = -1;                   // N - 4: the last slot that four loads may start at (-1: none)
 };
 
 __device__ __forceinline__ int2 rel(uint2 a, uint2 o)
@@ -564,6 +565,13 @@ __device__ __forceinline__ int fan_walk(const Bins &B, uint2 p, int v0, const SA
     }
     return -PFEM_ERR_TIMEOUT;
 }
+
+// A star as a plain array of slots (the stars a thread searched itself).
+struct ArrStar {
+    const int *p;
+    int n;
+    __device__ __forceinline__ int operator[](int i) const { return p[i]; }
+};
 
 // Locate fixed-point point p in the Delaunay triangulation: tri = counter-clockwise triangle
 // containing p (boundary included).  On success also returns the star of tri[0] in star0

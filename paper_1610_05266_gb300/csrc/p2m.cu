@@ -32,6 +32,7 @@ static P2MArgs make_args(const GeoArgs &g, DevStatus *st)
     a.B.dmax = g.dmax;
     a.B.kcap = g.kcap;
     a.B.walk_cap = g.walk_cap;
+    a.B.last4 = g.N >= 4 ? (int)(g.N - 4) : -1;
     a.R0 = g.R0;
     a.pos = g.pos_sorted;
     a.perm = nullptr;
@@ -57,10 +58,14 @@ static dim3 node_grid(int n) { return dim3((n + 15) / 16, (n + 7) / 8); }
 template <typename P, typename V, typename R, typename S, int REF, int SHAPE, bool W>
 static cudaError_t go_fast(const P2MArgs &a, cudaStream_t s)
 {
-    // FP64 solves take the FP32 factor with the solution refined to FP64 (fix64.cuh)
-    constexpr bool F64 = sizeof(S) == 8 && SHAPE == PFEM_SHAPE_QUADRATIC;
-    k_p2m<P, V, R, std::conditional_t<F64, float, S>, F64 ? REFINE_FIX64 : REF, SHAPE, W>
-        <<<node_grid(a.n), 128, 0, s>>>(a);
+    if constexpr (SHAPE == PFEM_SHAPE_LINEAR) {
+        k_p2m_linear<P, V, R, W><<<node_grid(a.n), 128, 0, s>>>(a);
+    } else {
+        // FP64 solves take the FP32 factor with the solution refined to FP64 (fix64.cuh)
+        constexpr bool F64 = sizeof(S) == 8;
+        k_p2m<P, V, R, std::conditional_t<F64, float, S>, F64 ? REFINE_FIX64 : REF, SHAPE, W>
+            <<<node_grid(a.n), 128, 0, s>>>(a);
+    }
     count_launch();
     return cudaGetLastError();
 }

@@ -356,13 +356,6 @@ __device__ __forceinline__ void store_vals<float, float>(float *out, long long n
         if (c < C) out[node * C + c] = acc[c];
 }
 
-// A star as a plain array of slots (the stars a thread searched itself).
-struct ArrStar {
-    const int *p;
-    int n;
-    __device__ __forceinline__ int operator[](int i) const { return p[i]; }
-};
-
 // Quadratic weights of one node over its distinct particles U = T + stars of T's vertices:
 // offsets are loaded once per particle, each edge's stencil is a bit mask over U, and
 // w_u = lambda_u [u in T] + sum_e 2 lambda_nu lambda_sg A_{u e} accumulates per particle.
@@ -708,6 +701,64 @@ __global__ void __launch_bounds__(128, PFEM_P2M_MIN_BLOCKS) k_p2m(P2MArgs a)
     const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
     if (I >= a.n || J >= a.n) return;
     p2m_node<P, V, R, S, REFINE, SHAPE, WEIGHTS>(a, I, J);
+}
+
+// Linear shape functions: one thread a node.  The node's triangle comes from the star of its nearest
+// particle, by the hull over the thread's list in shared memory as in the star table (gift wrapping
+// over lists in local memory took 169 us for 513^2 nodes over 1254^2 particles, this 107); the table itself
+// would hold the stars of every particle, six a node there.
+template <typename P, typename V, typename R, bool WEIGHTS>
+__device__ __forceinline__ void linear_node(const P2MArgs &a, const HullList &L, int I, int J)
+{
+    const int nc = a.n - 1;
+    const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
+    const long long node = (long long)J * a.n + I;
+    int tri[3];
+    int st = locate_hull(a.B, make_uint2(node_fx(Iu, nc), node_fx(Ju, nc)), a.R0, L, tri);
+    R lam[3] = {R(0), R(0), R(0)}, acc[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc[c] = R(0);
+    if (st == 0) {
+        NodePos<P, R> np;
+        np.init(Iu, Ju, nc);
+        barycentric(a, np, tri, lam);
+        if (!WEIGHTS)
+            for (int e = 0; e < 3; ++e) {
+                R v[8];
+                load_vals<V, R>((const V *)a.vals, a.perm, tri[e], a.C, v);
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (c < a.C) acc[c] = fma(lam[e], v[c], acc[c]);
+            }
+        else if (a.K < 3) st = -PFEM_ERR_CAPACITY;
+    }
+    st = defer_or_error(a, st, a.noff + node);
+    if (st < 0) record_error(a.status, -st, a.noff + node);
+    if (!WEIGHTS) {
+        if (st != 0)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[c] = (R)nan_of<R>();
+        store_vals<V, R>((V *)a.out, node, a.C, acc);
+    } else {
+        int *oi = a.w_idx + node * a.K;
+        R *ow = (R *)a.w + node * a.K;
+        for (int k = 0; k < a.K; ++k) {
+            const bool v = st == 0 && k < 3;
+            oi[k] = v ? tri[k] : -1;
+            ow[k] = v ? lam[k] : R(0);
+        }
+    }
+}
+
+template <typename P, typename V, typename R, bool WEIGHTS>
+__global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_p2m_linear(P2MArgs a)
+{
+    __shared__ float2 sxy[STAR_ROWS * STAR_TPB];
+    __shared__ int ss[STAR_ROWS * STAR_TPB];
+    const int I = blockIdx.x * 16 + (threadIdx.x & 15);
+    const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
+    if (I >= a.n || J >= a.n) return;
+    linear_node<P, V, R, WEIGHTS>(a, HullList{sxy + threadIdx.x, ss + threadIdx.x}, I, J);
 }
 
 // The queued nodes again, overwriting the fast pass's placeholder output: the geometry searched

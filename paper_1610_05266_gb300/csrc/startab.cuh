@@ -244,8 +244,7 @@ static __device__ __noinline__ bool certify_region(const Region &g, float D, Hul
 // and b; and the orientation of three images is the sign of the lifted incircle determinant of
 // (v, a, b, c) -- the predicate of the gift-wrapping search, with the same tie-break.  So the
 // hull's vertices in counter-clockwise order are v's star.  Returns the count, -1 (list overflow
-// or not certified: the caller retries wider) or -PFEM_ERR_*.  last4: the last slot of the set
-// but three.
+// or not certified: the caller retries wider) or -PFEM_ERR_*.  B.last4 >= 0.
 //
 // The kernel is bound by instruction issue, and a warp's 32 stars differ in their data, so the
 // steps are laid out as loops of the same length in every lane with predicated bodies:
@@ -263,7 +262,7 @@ static __device__ __noinline__ bool certify_region(const Region &g, float D, Hul
 //  5. Certify every triangle as the gift-wrapping search does (circumcircle inside the searched
 //     region and within D of v).
 __device__ __forceinline__ int star_hull(const Bins &B, int v, uint2 pv, const Region &g, float D,
-                                         int last4, const HullList &L, int *row)
+                                         const HullList &L, int *row)
 {
     constexpr int S = STAR_TPB, KLC = STAR_KL;
     const float D2 = D * D;
@@ -280,7 +279,7 @@ __device__ __forceinline__ int star_hull(const Bins &B, int v, uint2 pv, const R
     // the region's slot runs, four loads in flight at a time
     for_region_runs(B, g, [&](int a, int e) {
         int s = a;
-        for (; s < e && s <= last4; s += 4) {
+        for (; s < e && s <= B.last4; s += 4) {
             const uint2 *q = B.q + s;
             const uint2 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
             const int left = e - s;
@@ -462,6 +461,21 @@ __device__ __forceinline__ int star_hull(const Bins &B, int v, uint2 pv, const R
     return sp;
 }
 
+// Locate fixed-point point p as locate() does, the star of its nearest particle by the hull over the
+// calling thread's list, and only where that cannot certify it by gift wrapping.
+static __device__ __forceinline__ int locate_hull(const Bins &B, uint2 p, int R0, const HullList &L, int tri[3])
+{
+    const int v0 = nearest_particle(B, p, R0);
+    if (v0 < 0) return v0;
+    const uint2 pv = __ldg(B.q + v0);
+    __align__(16) int star[KMAX];
+    int c = -1;
+    if (B.dmax > 0.f && B.last4 >= 0) c = star_hull(B, v0, pv, make_region(B, pv, R0), B.dmax, L, star);
+    if (c == -1) c = star_region(B, v0, pv, R0, star);
+    if (c < 0) return c;
+    return fan_walk(B, p, v0, ArrStar{star, c}, c, [&](int u, int w) { return apex_of(B, u, w, R0); }, tri);
+}
+
 // The list attempt for slot v (candidates in L): its star into the table, or v queued.
 __device__ __forceinline__ void star_list_slot(const Bins &B, int R0, const StarTab &t, long long v,
                                                const HullList &L, DevStatus *st)
@@ -469,8 +483,8 @@ __device__ __forceinline__ void star_list_slot(const Bins &B, int R0, const Star
     const uint2 pv = __ldg(B.q + v);
     int *out = t.nbr + v * KMAX;
     int c = -1;
-    if (B.dmax > 0.f && t.N >= 4)
-        c = star_hull(B, (int)v, pv, make_region(B, pv, R0), B.dmax, (int)(t.N - 4), L, out);
+    if (B.dmax > 0.f && B.last4 >= 0)
+        c = star_hull(B, (int)v, pv, make_region(B, pv, R0), B.dmax, L, out);
     if (c == -1) {
         t.cnt[v] = tab_pack(t.gen, -1);
         t.queue[atomicAdd(t.qcount, 1)] = (int)v;   // at most N entries: each slot once
