@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "m2p.cuh"
 #include "p2m.cuh"
 
 namespace pfem {
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(128) k_p2m_fix_batch(const BPlanDev *pl, P2MAr
 
 // ---------------------------------------------------------------- M2P
 
-template <typename P, typename V, typename R>
+template <typename P, typename V, typename R, int CT, int U>
 __global__ void __launch_bounds__(256) k_m2p_batch(const BPlanDev *pl, const P *__restrict__ pos,
                                                    int C, const V *__restrict__ mesh,
                                                    V *__restrict__ vals)
@@ -323,30 +324,26 @@ __global__ void __launch_bounds__(256) k_m2p_batch(const BPlanDev *pl, const P *
     for (long long c = blockIdx.x; c < pl->n_chunks; c += gridDim.x) {
         const int p = find_item(cp, pl->P, c);
         const BDesc d = plan_desc(pl)[p];
-        const int n = d.n, nc = n - 1;
-        const V *mp = mesh + d.noff * C;
-        const long long first = (c - cp[p]) * BCHUNK;
-        const long long end = min(d.N, first + BCHUNK);
-        for (long long i = first + threadIdx.x; i < end; i += blockDim.x) {
-            const long long m = d.poff + i;
-            P px, py;
-            load_pos(pos, m, px, py);
-            const int ci = bin_of(fx_of(px), nc), cj = bin_of(fx_of(py), nc);
-            P s = fma(px - floor(px), (P)nc, (P)(-ci)), t = fma(py - floor(py), (P)nc, (P)(-cj));
-            if (s > (P)(0.5 * nc)) s -= (P)nc;
-            if (t > (P)(0.5 * nc)) t -= (P)nc;
-            const long long n00 = (long long)cj * n + ci;
-            long long nb_, nc_;
-            R w0, w1, w2;
-            if (s >= t) { nb_ = n00 + 1; nc_ = n00 + n + 1; w0 = R(P(1) - s); w1 = R(s - t); w2 = R(t); }
-            else        { nb_ = n00 + n + 1; nc_ = n00 + n; w0 = R(P(1) - t); w1 = R(s); w2 = R(t - s); }
-            for (int k = 0; k < C; ++k) {
-                const R v = w0 * load_val<V, R>(mp + n00 * C + k) + w1 * load_val<V, R>(mp + nb_ * C + k) +
-                            w2 * load_val<V, R>(mp + nc_ * C + k);
-                store_val<V, R>(vals + m * C + k, v);
-            }
-        }
+        const long long first = d.poff + (c - cp[p]) * BCHUNK;
+        const long long end = d.poff + min(d.N, (c - cp[p] + 1) * BCHUNK);
+        for (long long m = first + threadIdx.x; m < end; m += 256 * U)
+            m2p_particles<P, V, R, CT, U>(d.n, m, end, pos, C, mesh + d.noff * C, vals);
     }
+}
+
+template <typename P, typename V, typename R>
+static void m2p_batch_t(const void *plan, const void *pos, int C, const void *mesh, void *vals, int blocks,
+                        cudaStream_t s)
+{
+    auto go = [&](auto ct, auto u) {
+        k_m2p_batch<P, V, R, decltype(ct)::value, decltype(u)::value><<<blocks, 256, 0, s>>>(
+            (const BPlanDev *)plan, (const P *)pos, C, (const V *)mesh, (V *)vals);
+    };
+    // as for one problem (a problem's mesh may start on any multiple of C values: no 16-byte accesses)
+    if (C == 1) go(std::integral_constant<int, 1>(), std::integral_constant<int, 4>());
+    else if (C == 2) go(std::integral_constant<int, 2>(), std::integral_constant<int, 4>());
+    else if (C == 3) go(std::integral_constant<int, 3>(), std::integral_constant<int, 2>());
+    else go(std::integral_constant<int, 0>(), std::integral_constant<int, 1>());
 }
 
 // ---------------------------------------------------------------- host side
@@ -553,11 +550,10 @@ cudaError_t launch_batch_m2p(const void *plan, const void *pos, pfem_dtype pos_t
                              const void *mesh, void *vals, pfem_dtype val_t, int blocks,
                              cudaStream_t s)
 {
-    const BPlanDev *pl = (const BPlanDev *)plan;
     if (val_t == PFEM_F64 && pos_t == PFEM_F64)
-        k_m2p_batch<double, double, double><<<blocks, 256, 0, s>>>(pl, (const double *)pos, C, (const double *)mesh, (double *)vals);
+        m2p_batch_t<double, double, double>(plan, pos, C, mesh, vals, blocks, s);
     else if (val_t == PFEM_F32 && pos_t == PFEM_F32)
-        k_m2p_batch<float, float, float><<<blocks, 256, 0, s>>>(pl, (const float *)pos, C, (const float *)mesh, (float *)vals);
+        m2p_batch_t<float, float, float>(plan, pos, C, mesh, vals, blocks, s);
     else
         return cudaErrorInvalidValue;
     count_launch();

@@ -48,6 +48,9 @@ __device__ __forceinline__ long long fx64(float x)
     return (long long)((b >> 31) ? 0ull - q : q);
 }
 
+__device__ __forceinline__ bool is_finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool is_finite_bits(float x) { return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u; }
+
 // I / nc in Q64, rounded to nearest (0 <= I < nc < 2^31).
 __device__ __forceinline__ long long node_fx64(int I, int nc)
 {

@@ -1,81 +1,50 @@
 // m2p.cu -- mesh-to-particle interpolation (Sec. 2.2 eq. m2p) with linear FE shape functions
-// on the fixed structured mesh: one thread per particle, in the caller's particle order.
+// on the fixed structured mesh, in the caller's particle order.
 //
 // The particle's cell (i, j) comes from its fixed-point coordinates (the same rule that bins
 // the particles); local coordinates s = x/H - i, t = y/H - j select the triangle of the cell
-// split along (i,j)->(i+1,j+1):
-//   s >= t: weights (1-s, s-t, t) on nodes (i,j), (i+1,j), (i+1,j+1)
-//   s <  t: weights (1-t, s, t-s) on nodes (i,j), (i+1,j+1), (i,j+1)
+// split along (i,j)->(i+1,j+1).  With hi = max(s, t), lo = min(s, t) the weights are 1 - hi on node
+// (i,j), lo on (i+1,j+1) and hi - lo on (i+1,j) where s >= t, on (i,j+1) where s < t.
 // Because the image row and column are stored, i+1 and j+1 never wrap.  The kernel is a
 // bandwidth-bound gather: positions and outputs stream once; the mesh is read through L2.
 #include <cmath>
 #include <type_traits>
 
 #include "internal.h"
+#include "m2p.cuh"
 
 namespace pfem {
 
-template <typename R> __device__ __forceinline__ R local_coord(R x, int i, int nc)
-{
-    const R xw = x - floor(x);                          // exact
-    R s = fma(xw, (R)nc, (R)(-i));
-    if (s > (R)(0.5 * nc)) s -= (R)nc;                  // fixed point rounded up to 2^32 -> cell 0
-    return s;
-}
-
-template <typename P, typename V, typename R, int CT>
+// Particles a thread, 256 apart: their loads are in flight together.  8192^2 particles of one BF16
+// component 632 -> 314 us with four (their bytes take 104 us), 1254^2 of three FP32 ones 18 -> 13
+// us with two; four FP32 components, whose three 16-byte gathers keep enough in flight, 23 us with
+// one and 29 with two.  FP64 positions in fixed point (m2p.cuh): 1024^2 of three 63 -> 26 us.
+template <typename P, typename V, typename R, int CT, int U>
 __global__ void __launch_bounds__(256) k_m2p(int n, long long N, const P *__restrict__ pos,
                                              int Crt, const V *__restrict__ mesh,
                                              V *__restrict__ vals)
 {
-    const int C = CT > 0 ? CT : Crt;
-    const int nc = n - 1;
-    for (long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x; m < N;
-         m += (long long)gridDim.x * blockDim.x) {
-        P px, py;
-        load_pos(pos, m, px, py);
-        const int i = bin_of(fx_of(px), nc), j = bin_of(fx_of(py), nc);
-        const P s = local_coord<P>(px, i, nc), t = local_coord<P>(py, j, nc);
-        const long long n00 = (long long)j * n + i;
-        long long nb_, nc_;
-        R w0, w1, w2;
-        if (s >= t) { nb_ = n00 + 1; nc_ = n00 + n + 1; w0 = R(P(1) - s); w1 = R(s - t); w2 = R(t); }
-        else        { nb_ = n00 + n + 1; nc_ = n00 + n; w0 = R(P(1) - t); w1 = R(s); w2 = R(t - s); }
-        if constexpr (CT == 4 && sizeof(V) == 4 && sizeof(R) == 4) {
-            const float4 a = __ldg(reinterpret_cast<const float4 *>(mesh) + n00);
-            const float4 b = __ldg(reinterpret_cast<const float4 *>(mesh) + nb_);
-            const float4 c = __ldg(reinterpret_cast<const float4 *>(mesh) + nc_);
-            float4 o;
-            o.x = fmaf(w0, a.x, fmaf(w1, b.x, w2 * c.x));
-            o.y = fmaf(w0, a.y, fmaf(w1, b.y, w2 * c.y));
-            o.z = fmaf(w0, a.z, fmaf(w1, b.z, w2 * c.z));
-            o.w = fmaf(w0, a.w, fmaf(w1, b.w, w2 * c.w));
-            __stcs(reinterpret_cast<float4 *>(vals) + m, o);
-        } else {
-            for (int c = 0; c < C; ++c) {
-                const R v = w0 * load_val<V, R>(mesh + n00 * C + c) +
-                            w1 * load_val<V, R>(mesh + nb_ * C + c) +
-                            w2 * load_val<V, R>(mesh + nc_ * C + c);
-                store_val<V, R>(vals + m * C + c, v);
-            }
-        }
-    }
+    const long long m0 = blockIdx.x * (256LL * U) + threadIdx.x;
+    m2p_particles<P, V, R, CT, U>(n, m0, N, pos, Crt, mesh, vals);
 }
 
 template <typename P, typename V, typename R>
 static cudaError_t m2p_t(int n, long long N, const void *pos, int C, const void *mesh, void *vals,
                          cudaStream_t s)
 {
-    long long blocks = (N + 255) / 256;
-    if (blocks > num_sms() * 16LL) blocks = num_sms() * 16LL;
-    if (blocks < 1) blocks = 1;
     const bool aligned = ((reinterpret_cast<uintptr_t>(mesh) | reinterpret_cast<uintptr_t>(vals)) & 15) == 0;
-    if (C == 4 && aligned)
-        k_m2p<P, V, R, 4><<<(unsigned)blocks, 256, 0, s>>>(n, N, (const P *)pos, C,
-                                                          (const V *)mesh, (V *)vals);
-    else
-        k_m2p<P, V, R, 0><<<(unsigned)blocks, 256, 0, s>>>(n, N, (const P *)pos, C,
-                                                          (const V *)mesh, (V *)vals);
+    auto go = [&](auto ct, auto u) {
+        constexpr int CT = decltype(ct)::value, U = decltype(u)::value;
+        k_m2p<P, V, R, CT, U><<<(unsigned)((N + 256 * U - 1) / (256 * U)), 256, 0, s>>>(
+            n, N, (const P *)pos, C, (const V *)mesh, (V *)vals);
+    };
+    // the components in registers up to four; four FP32 ones as one 16-byte access when the arrays
+    // allow it
+    if (C == 1) go(std::integral_constant<int, 1>(), std::integral_constant<int, 4>());
+    else if (C == 2) go(std::integral_constant<int, 2>(), std::integral_constant<int, 4>());
+    else if (C == 3) go(std::integral_constant<int, 3>(), std::integral_constant<int, 2>());
+    else if (C == 4 && (aligned || sizeof(V) != 4)) go(std::integral_constant<int, 4>(), std::integral_constant<int, 1>());
+    else go(std::integral_constant<int, 0>(), std::integral_constant<int, 1>());
     count_launch();
     return cudaGetLastError();
 }
@@ -132,23 +101,15 @@ __global__ void __launch_bounds__(128) k_m2p_bwd_mesh(int n, int nb, const P *__
                     const int m = __ldg(perm + s);
                     P px, py;
                     load_pos(pos, m, px, py);
-                    const int i = bin_of(fx_of(px), nc), j = bin_of(fx_of(py), nc);
+                    int i, j;
+                    cell_index(px, py, nc, i, j);
                     if (i != ci || j != cj) continue;
-                    const P ss = local_coord<P>(px, i, nc), tt = local_coord<P>(py, j, nc);
-                    const long long n00 = (long long)j * n + i;
-                    R w = R(0);
-                    if (ss >= tt) {
-                        if (node == n00) w = R(P(1) - ss);
-                        else if (node == n00 + 1) w = R(ss - tt);
-                        else if (node == n00 + n + 1) w = R(tt);
-                    } else {
-                        if (node == n00) w = R(P(1) - tt);
-                        else if (node == n00 + n + 1) w = R(ss);
-                        else if (node == n00 + n) w = R(tt - ss);
-                    }
+                    const MeshCell<R> c = mesh_cell<P, R>(px, py, n);
+                    const R w = node == c.n00 ? c.w0 : node == c.n00 + c.mid ? c.w1 : node == c.n00 + n + 1 ? c.w2 : R(0);
                     if (w == R(0)) continue;
-                    for (int c = 0; c < C; ++c)
-                        acc[c] = fma(w, load_val<V, R>(gv + (long long)m * C + c), acc[c]);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        if (k < C) acc[k] = fma(w, load_val<V, R>(gv + (long long)m * C + k), acc[k]);
                 }
             }
         }
@@ -167,8 +128,8 @@ __global__ void __launch_bounds__(256) k_m2p_bwd_pos(int n, long long N, const P
          m += (long long)gridDim.x * blockDim.x) {
         P px, py;
         load_pos(pos, m, px, py);
-        const int i = bin_of(fx_of(px), nc), j = bin_of(fx_of(py), nc);
-        const P s = local_coord<P>(px, i, nc), t = local_coord<P>(py, j, nc);
+        int i, j;
+        const bool below = cell_index(px, py, nc, i, j);
         const long long n00 = (long long)j * n + i, n10 = n00 + 1, n11 = n00 + n + 1, n01 = n00 + n;
         R gx = R(0), gy = R(0);
         for (int c = 0; c < C; ++c) {
@@ -176,7 +137,7 @@ __global__ void __launch_bounds__(256) k_m2p_bwd_pos(int n, long long N, const P
             const R f00 = load_val<V, R>(mesh + n00 * C + c), f10 = load_val<V, R>(mesh + n10 * C + c);
             const R f11 = load_val<V, R>(mesh + n11 * C + c), f01 = load_val<V, R>(mesh + n01 * C + c);
             R ds, dt;
-            if (s >= t) { ds = f10 - f00; dt = f11 - f10; }
+            if (below) { ds = f10 - f00; dt = f11 - f10; }
             else        { ds = f11 - f01; dt = f01 - f00; }
             gx = fma(g, ds, gx);
             gy = fma(g, dt, gy);
@@ -228,7 +189,6 @@ cudaError_t launch_m2p_backward(int n, int nb, long long N, const void *pos, pfe
 // edges into one table: the coefficient of each stencil node in each edge.  Then
 //   w_k = lambda_k [k vertex] + sum_e 2 lambda_P(e) lambda_Q(e) A_{k,e}.
 // Node values are read at the unique nodes (I mod (n-1), J mod (n-1)).
-
 //
 // The triangle above the diagonal is the one below it with x and y exchanged, so the kernel
 // works in coordinates (hi, lo) = (max, min) of the particle's cell coordinates, with vertices
@@ -356,11 +316,10 @@ __global__ void __launch_bounds__(256) k_m2p_q(int n, long long N, const P *__re
          m += (long long)gridDim.x * blockDim.x) {
         P px, py;
         load_pos(pos, m, px, py);
-        const int i = bin_of(fx_of(px), nc), j = bin_of(fx_of(py), nc);
-        const P s = local_coord<P>(px, i, nc), t = local_coord<P>(py, j, nc);
-        const bool below = s >= t;
-        const P hi = below ? s : t, lo = below ? t : s;
-        const R lam[3] = {R(P(1) - hi), R(hi - lo), R(lo)};
+        const MeshCell<R> cell = mesh_cell<P, R>(px, py, n);
+        const int i = cell.i, j = cell.j;
+        const bool below = cell.mid == 1;
+        const R lam[3] = {cell.w0, cell.w1, cell.w2};
         const R ce[3] = {R(2) * lam[0] * lam[1], R(2) * lam[1] * lam[2], R(2) * lam[2] * lam[0]};
         R w[MQ_NODES];
 #pragma unroll
