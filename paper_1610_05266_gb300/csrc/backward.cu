@@ -220,6 +220,7 @@ __device__ __forceinline__ int bwd_u_solve64(const BwdArgs &b, int Iu, int Ju, c
     const int nc = a.n - 1;
     longlong2 o[UMAX];
     const int L = node_offsets64<P>(a.pos, Iu, Ju, nc, us, nu, o);
+    if (L == NOT_FINITE) return -PFEM_DEFER;
     long long bi[POS ? UMAX : 1];
     double lbar[3] = {0.0, 0.0, 0.0}, bunit = 0.0;
     if (POS) {
@@ -356,8 +357,7 @@ __device__ __forceinline__ int bwd_u_solve64(const BwdArgs &b, int Iu, int Ju, c
 template <typename P, typename V, typename R, bool POS>
 __global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_bwd_linear(BwdArgs b)
 {
-    __shared__ float2 sxy[STAR_ROWS * STAR_TPB];
-    __shared__ int ss[STAR_ROWS * STAR_TPB];
+    __shared__ __align__(16) unsigned char lists[HullList::BYTES];
     const P2MArgs &a = b.f;
     const int I = blockIdx.x * 16 + (threadIdx.x & 15);
     const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_bwd_linear(B
     int nu = 0;
     if (any) {
         int st = locate_hull(a.B, make_uint2(node_fx(Iu, nc), node_fx(Ju, nc)), a.R0,
-                             HullList{sxy + threadIdx.x, ss + threadIdx.x}, us);
+                             HullList::at(lists, threadIdx.x), us);
         if (st == 0) {
             NodePos<P, R> np;
             np.init(Iu, Ju, nc);

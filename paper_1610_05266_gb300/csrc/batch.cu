@@ -190,10 +190,7 @@ __global__ void __launch_bounds__(256) k_p2m_batch_linear(const BPlanDev *pl, in
 {
     extern __shared__ __align__(16) unsigned char lists[];
     __shared__ long long item;
-    const int half = threadIdx.x / STAR_TPB, lane = threadIdx.x % STAR_TPB;
-    constexpr int BYTES = STAR_ROWS * STAR_TPB * (int)(sizeof(float2) + sizeof(int));
-    float2 *xy = reinterpret_cast<float2 *>(lists + half * BYTES);
-    const HullList L{xy + lane, reinterpret_cast<int *>(xy + STAR_ROWS * STAR_TPB) + lane};
+    const HullList L = HullList::at(lists + threadIdx.x / STAR_TPB * HullList::BYTES, threadIdx.x % STAR_TPB);
     const int TY = blockDim.x / 16;
     const long long total = pl->n_items[shape_idx];
     const long long *tp = plan_tiles(pl, shape_idx);
@@ -222,8 +219,7 @@ __global__ void __launch_bounds__(BSTAR, PFEM_STAR_MIN_BLOCKS) k_star_list_batch
                                                                                  P2MArgs base, StarTab t)
 {
     static_assert(BSTAR == STAR_TPB, "HullList's columns");
-    __shared__ float2 sxy[STAR_ROWS * BSTAR];
-    __shared__ int ss[STAR_ROWS * BSTAR];
+    __shared__ __align__(16) unsigned char lists[HullList::BYTES];
     if (!totals_ok(pl, -1, t, base.status)) return;
     const long long *sp = plan_star_tiles(pl);
     for (long long b = blockIdx.x; b < pl->n_star_tiles; b += gridDim.x) {
@@ -233,30 +229,27 @@ __global__ void __launch_bounds__(BSTAR, PFEM_STAR_MIN_BLOCKS) k_star_list_batch
         if (i >= d.N) continue;
         P2MArgs a;
         problem_args(a, base, d, pl->total_particles);
-        const HullList L{sxy + threadIdx.x, ss + threadIdx.x};
-        star_list_slot(a.B, a.R0, t, d.poff + i, L, a.status);
+        star_list_slot(a.B, a.R0, t, d.poff + i, HullList::at(lists, threadIdx.x), a.status);
     }
 }
 
-// The queued particles of the table, a warp each, with its problem's bins and the widest radius.
-__global__ void __launch_bounds__(RETRY_TPB, PFEM_RETRY_BLOCKS) k_star_retry_batch(const BPlanDev *pl,
-                                                                                   P2MArgs base, StarTab t)
+// The queued particles of the table, each with its problem's bins and the widest radius.
+__global__ void __launch_bounds__(RETRY_TPB, RETRY_BLOCKS) k_star_retry_batch(const BPlanDev *pl,
+                                                                              P2MArgs base, StarTab t)
 {
+    __shared__ __align__(16) unsigned char lists[HullListLong::BYTES];
     __shared__ int2 sd[RETRY_TPB / 32 * WSTAR_CAP];
     __shared__ int ss[RETRY_TPB / 32 * WSTAR_CAP];
     const int w = threadIdx.x >> 5;
-    const WarpList L{sd + w * WSTAR_CAP, ss + w * WSTAR_CAP};
-    const int n = min(*t.qcount, (int)min(t.N, (long long)0x7fffffff));
     const BDesc *D = plan_desc(pl);
-    for (int i = blockIdx.x * (RETRY_TPB / 32) + w; i < n; i += gridDim.x * (RETRY_TPB / 32)) {
-        const int v = t.queue[i];
-        const int p = find_problem(pl->P, v, [&](int k) { return D[k].poff; });
-        const BDesc d = D[p];
+    star_retry(t, lists, WarpList{sd + w * WSTAR_CAP, ss + w * WSTAR_CAP}, base.status, [&](int v, int &R0) {
+        const BDesc d = D[find_problem(pl->P, v, [&](int k) { return D[k].poff; })];
         P2MArgs a;
         problem_args(a, base, d, pl->total_particles);
         a.B.rmax = max(d.rmax, d.nb / 4 - 1);
-        star_retry_slot(a.B, a.R0, t, v, L, a.status);
-    }
+        R0 = a.R0;
+        return a.B;
+    });
 }
 
 // The table path's fast pass of every problem in one persistent kernel (as k_p2m_tab: location
@@ -267,6 +260,7 @@ __global__ void __launch_bounds__(256, tab_min_blocks<REFINE>() / 2) k_p2m_batch
     long long nodes)
 {
     __shared__ long long item;
+    extern __shared__ int su[];             // tab_rows words a thread
     if (!totals_ok(pl, nodes, tab, base.status)) return;
     const int TY = blockDim.x / 16;
     const long long total = pl->n_items[shape_idx];
@@ -287,7 +281,7 @@ __global__ void __launch_bounds__(256, tab_min_blocks<REFINE>() / 2) k_p2m_batch
         P2MArgs a;
         problem_args(a, base, d, pl->total_particles);
         problem_out<V>(a, base, d);
-        tab_node<P, V, R, S, REFINE>(a, tab, I, J);
+        tab_node<P, V, R, S, REFINE>(a, tab, I, J, su + threadIdx.x, blockDim.x);
     }
 }
 
@@ -457,15 +451,16 @@ static cudaError_t p2m_batch_t(const void *plan, const P2MArgs &base, int shape_
         // a block per tile of 128 particles (the problems' ragged last tiles are taken by the
         // blocks that are done first)
         k_star_list_batch<<<(unsigned)((w.tab.N + BSTAR - 1) / BSTAR), BSTAR, 0, s>>>(pl, base, w.tab);
-        k_star_retry_batch<<<num_sms() * PFEM_RETRY_BLOCKS, RETRY_TPB, 0, s>>>(pl, base, w.tab);
+        k_star_retry_batch<<<num_sms() * RETRY_BLOCKS, RETRY_TPB, 0, s>>>(pl, base, w.tab);
         constexpr int TREF = sizeof(S) == 8 ? REFINE_FIX64 : REF;    // as for one problem
-        k_p2m_batch_tab<P, V, R, float, TREF><<<blocks, 16 * TYs[shape_idx], 0, s>>>(
+        const size_t su = (size_t)16 * TYs[shape_idx] * tab_rows<TREF>() * sizeof(int);
+        k_p2m_batch_tab<P, V, R, float, TREF><<<blocks, 16 * TYs[shape_idx], su, s>>>(
             pl, shape_idx, base, counter, w.tab, w.nodes);
         count_launch(3);
     } else {
         const int threads = 16 * TYs[shape_idx];
         if constexpr (SHAPE == PFEM_SHAPE_LINEAR) {
-            const size_t lists = (size_t)((threads + STAR_TPB - 1) / STAR_TPB) * STAR_ROWS * STAR_TPB * (sizeof(float2) + sizeof(int));
+            const size_t lists = (size_t)((threads + STAR_TPB - 1) / STAR_TPB) * HullList::BYTES;
             e = cudaFuncSetAttribute(k_p2m_batch_linear<P, V, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lists);
             if (e != cudaSuccess) return e;
             k_p2m_batch_linear<P, V, R><<<blocks, threads, lists, s>>>(pl, shape_idx, base, counter);

@@ -110,16 +110,20 @@ struct EdgeFix64 {
 };
 
 // Offsets of a node's particles from it in fixed point, scaled up by a common power of two 2^L so
-// that every |offset| < 2^60: o[0..nu) in Q64.  Returns L.
-template <typename P, int UM>
-__device__ __forceinline__ int node_offsets64(const void *pos, int Iu, int Ju, int nc, const int *us,
+// that every |offset| < 2^60: o[0..nu) in Q64.  Returns L, or NOT_FINITE when a position is not.
+constexpr int NOT_FINITE = -1000;
+template <typename P, int UM, typename Slots>
+__device__ __forceinline__ int node_offsets64(const void *pos, int Iu, int Ju, int nc, Slots &&us,
                                                int nu, longlong2 (&o)[UM])
 {
     const long long nx = node_fx64(Iu, nc), ny = node_fx64(Ju, nc);
     unsigned long long m = 0;
+    bool bad = false;
     for (int i = 0; i < nu; ++i) {
         P px, py;
         load_pos((const P *)pos, us[i], px, py);
+        bad |= !is_finite_bits(px) || !is_finite_bits(py);     // no second way out of the loop: the warp
+                                                              // would not come together after it
         const long long x = fx64(px) - nx, y = fx64(py) - ny;
         m |= (unsigned long long)(x ^ (x >> 63)) | (unsigned long long)(y ^ (y >> 63));
         o[i] = make_longlong2(x, y);
@@ -129,7 +133,7 @@ __device__ __forceinline__ int node_offsets64(const void *pos, int Iu, int Ju, i
         if (L >= 0) o[i] = make_longlong2(o[i].x << L, o[i].y << L);
         else o[i] = make_longlong2(o[i].x >> -L, o[i].y >> -L);
     }
-    return L;
+    return bad ? NOT_FINITE : L;
 }
 
 // One edge's system over the particles of `mask`: its FP32 factor, the units of the fixed point and the

@@ -30,8 +30,9 @@ template <typename S> struct Moment {
     __device__ __forceinline__ void add(S x, S y)
     {
         const S p[6] = {S(1), x, y, x * x, x * y, y * y};
+        m[0] += S(1);
 #pragma unroll
-        for (int r = 0; r < 6; ++r)
+        for (int r = 1; r < 6; ++r)
 #pragma unroll
             for (int c = 0; c <= r; ++c) m[tri_ix(r, c)] = fma(p[r], p[c], m[tri_ix(r, c)]);
     }

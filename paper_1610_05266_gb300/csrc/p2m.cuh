@@ -429,19 +429,11 @@ __device__ __forceinline__ int node_u_sets(const int tri[3], const SA *st, int *
 // The edge systems e0 <= e < e1 of a node over its particle set: uw[u] += 2 lambda_nu lambda_sg
 // A_{u e}, or with RAW (one edge) uw[u] = A_{u e}.
 // Returns 0, or -PFEM_DEFER when a moment matrix is below the fast-solve tolerance.
-template <typename P, typename R, typename S, int REFINE, bool SVD, int UM, bool RAW = false>
-__device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R> &np,
-                                            const int *us, R *uw, const unsigned vm[3],
-                                            const int vi[3], const R lam[3], int e0 = 0, int e1 = 3)
+// offset(i, x, y): the offset of particle i from the node.
+template <typename R, typename S, int REFINE, bool SVD, int UM, bool RAW, typename W, typename Offset>
+__device__ __forceinline__ int node_edges(W &&uw, const unsigned vm[3], const int vi[3], const R lam[3],
+                                          int e0, int e1, Offset &&offset)
 {
-    // Offsets are re-read from the positions, which neighbouring nodes share in L1, instead of
-    // being copied into thread-private memory.
-    auto offset = [&](int i, S &x, S &y) {
-        R dx, dy;
-        np.off(a.pos, us[i], dx, dy);
-        x = S(dx);
-        y = S(dy);
-    };
     // The three edges in a loop that is not unrolled: one copy of the edge code keeps the
     // kernels' instruction footprint and register spills down (fused kernel with the refined
     // solve: 1.047 -> 1.010 ms at 1025^2 nodes / 2048^2 particles; spills 164 -> 40 bytes).
@@ -458,7 +450,7 @@ __device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R
         offset(vi[f], rsx, rsy);
         const S mx = (rnx + rsx) * S(0.5), my = (rny + rsy) * S(0.5);
         const S ex = rnx - rsx, ey = rny - rsy;
-        const S inv = S(1) / sqrt(ex * ex + ey * ey);
+        const S inv = S(1) / sqrt(fma(ex, ex, ey * ey));
         if constexpr (SVD) {
             double pt[UM][6];
             int ids[UM];
@@ -477,7 +469,7 @@ __device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R
             double A[UM];
             minnorm_lsq(k, pt, b, A);
             const double coef = 2.0 * (double)lam[e] * (double)lam[f];
-            for (int j = 0; j < k; ++j) uw[ids[j]] += (R)(coef * A[j]);
+            for (int j = 0; j < k; ++j) uw(ids[j]) += (R)(coef * A[j]);
             continue;
         }
         Moment<S> M;
@@ -509,7 +501,7 @@ __device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R
             fr.result(rs);
             M.solve(rs, dy);
 #pragma unroll
-            for (int k = 0; k < 6; ++k) y[k] += dy[k];
+            for (int k = 0; k < 6; ++k) y[k] = __fadd_rn(y[k], dy[k]);
         }
         const R coef = R(2) * lam[e] * lam[f];
         for (unsigned m = mask; m; m &= m - 1) {
@@ -517,11 +509,25 @@ __device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R
             S ox, oy;
             offset(i, ox, oy);
             const S x = (ox - mx) * inv, yv = (oy - my) * inv;
-            const S A = y[0] + x * y[1] + yv * y[2] + x * x * y[3] + x * yv * y[4] + yv * yv * y[5];
-            uw[i] = RAW ? R(A) : fma(coef, R(A), uw[i]);
+            const S A = fma(yv * yv, y[5], fma(x * yv, y[4], fma(x * x, y[3], fma(yv, y[2], fma(x, y[1], y[0])))));
+            uw(i) = RAW ? R(A) : fma(coef, R(A), uw(i));
         }
     }
     return 0;
+}
+
+// node_edges with offsets re-read from the positions, which neighbouring nodes share in L1.
+template <typename P, typename R, typename S, int REFINE, bool SVD, int UM>
+__device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R> &np,
+                                            const int *us, R *uw, const unsigned vm[3],
+                                            const int vi[3], const R lam[3], int e0 = 0, int e1 = 3)
+{
+    return node_edges<R, S, REFINE, SVD, UM, false>([&](int i) -> R & { return uw[i]; }, vm, vi, lam, e0, e1, [&](int i, S &x, S &y) {
+        R dx, dy;
+        np.off(a.pos, us[i], dx, dy);
+        x = S(dx);
+        y = S(dy);
+    });
 }
 
 template <typename P, typename R, typename S, int REFINE, bool SVD = false, typename SA,
@@ -557,7 +563,7 @@ __device__ __forceinline__ int node_quadratic64(const P2MArgs &a, int Iu, int Ju
     if (node_u_sets<UMAX>(tri, st, us, nu, vm, vi, min(a.ucap, UMAX)) != 0) return -PFEM_DEFER;
     longlong2 o[UMAX];
     long long w[UMAX];
-    node_offsets64<P>(a.pos, Iu, Ju, a.n - 1, us, nu, o);
+    if (node_offsets64<P>(a.pos, Iu, Ju, a.n - 1, us, nu, o) == NOT_FINITE) return -PFEM_DEFER;
     for (int i = 0; i < nu; ++i) w[i] = 0;
     const double l64[3] = {(double)lam[0], (double)lam[1], (double)lam[2]};
     const int r = node_solve64(o, vm, vi, l64, 0, 3, w, -PFEM_DEFER);
@@ -568,7 +574,9 @@ __device__ __forceinline__ int node_quadratic64(const P2MArgs &a, int Iu, int Ju
     return 0;
 }
 
-// Barycentric coordinates of the node (the origin of np's offsets) in triangle tri.
+// Barycentric coordinates of the node (the origin of np's offsets) in triangle tri.  Here and in the
+// edge systems every fused multiply-add is written out: the compiler would choose them differently
+// in the kernels that share this arithmetic, whose results agree bit for bit.
 template <typename P, typename R>
 __device__ __forceinline__ void barycentric(const P2MArgs &a, const NodePos<P, R> &np,
                                             const int tri[3], R lam[3])
@@ -576,10 +584,10 @@ __device__ __forceinline__ void barycentric(const P2MArgs &a, const NodePos<P, R
     R d[3][2];
 #pragma unroll
     for (int e = 0; e < 3; ++e) np.off(a.pos, tri[e], d[e][0], d[e][1]);
-    const R area2 = (d[1][0] - d[0][0]) * (d[2][1] - d[0][1]) - (d[1][1] - d[0][1]) * (d[2][0] - d[0][0]);
-    lam[0] = (d[1][0] * d[2][1] - d[1][1] * d[2][0]) / area2;
-    lam[1] = (d[2][0] * d[0][1] - d[2][1] * d[0][0]) / area2;
-    lam[2] = (d[0][0] * d[1][1] - d[0][1] * d[1][0]) / area2;
+    const R area2 = fma(d[1][0] - d[0][0], d[2][1] - d[0][1], -((d[1][1] - d[0][1]) * (d[2][0] - d[0][0])));
+    lam[0] = fma(d[1][0], d[2][1], -(d[1][1] * d[2][0])) / area2;
+    lam[1] = fma(d[2][0], d[0][1], -(d[2][1] * d[0][0])) / area2;
+    lam[2] = fma(d[0][0], d[1][1], -(d[0][1] * d[1][0])) / area2;
 }
 
 template <typename V> __device__ __forceinline__ V nan_of();
@@ -753,12 +761,11 @@ __device__ __forceinline__ void linear_node(const P2MArgs &a, const HullList &L,
 template <typename P, typename V, typename R, bool WEIGHTS>
 __global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_p2m_linear(P2MArgs a)
 {
-    __shared__ float2 sxy[STAR_ROWS * STAR_TPB];
-    __shared__ int ss[STAR_ROWS * STAR_TPB];
+    __shared__ __align__(16) unsigned char lists[HullList::BYTES];
     const int I = blockIdx.x * 16 + (threadIdx.x & 15);
     const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
     if (I >= a.n || J >= a.n) return;
-    linear_node<P, V, R, WEIGHTS>(a, HullList{sxy + threadIdx.x, ss + threadIdx.x}, I, J);
+    linear_node<P, V, R, WEIGHTS>(a, HullList::at(lists, threadIdx.x), I, J);
 }
 
 // The queued nodes again, overwriting the fast pass's placeholder output: the geometry searched
@@ -814,18 +821,99 @@ inline size_t node_recs_layout(char *base, long long nodes, NodeRecs *r, bool wi
     return total;
 }
 
+// The node's particle set and stencil masks as node_u_sets gives them (same order), from stars of up
+// to 8 particles held in registers: n the stars' sizes, su the thread's column of shared memory
+// (stride between entries) that receives the slots.  Returns the set's size; the slots are complete
+// up to SET_MAX.  Jittered lattices fit everywhere.
+//
+// The node kernel is bound by latency: what a thread kept in local memory (the growing set, which
+// node_u_sets searches entry by entry, and the weights) came to half a megabyte a resident SM's
+// threads, and its loads waited on L2.  node_u_sets took 178 us of the kernel's 660 us at 1025^2
+// nodes / 2048^2 particles; here every step is the same in every lane, the stars' rows come in two
+// loads each, and slots and weights lie in shared memory: 560 us.  (The offsets in shared memory as
+// well, or everything in registers with the loops over all 16 entries unrolled, cost blocks per SM:
+// 600 and 770 us.)
+constexpr int SET_MAX = 16;
+// Rows of a thread's column: the slots (two spare) and the weights.
+constexpr int SET_W = SET_MAX + 2, SET_ROWS = SET_W + SET_MAX;
+
+// An array whose entries lie `stride` apart.
+template <typename T> struct Strided {
+    T *p;
+    int stride;
+    __device__ __forceinline__ T &operator[](int i) const { return p[i * stride]; }
+};
+
+__device__ __forceinline__ int node_sets8(const StarTab &t, const int tri[3], const int n[3], int *su,
+                                          int stride, unsigned vm[3])
+{
+    int s[3][8];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        const int4 *row = reinterpret_cast<const int4 *>(t.nbr + (long long)tri[e] * KMAX);
+        const int4 lo = __ldg(row), hi = __ldg(row + 1);
+        s[e][0] = lo.x; s[e][1] = lo.y; s[e][2] = lo.z; s[e][3] = lo.w;
+        s[e][4] = hi.x; s[e][5] = hi.y; s[e][6] = hi.z; s[e][7] = hi.w;
+        su[e * stride] = tri[e];
+    }
+    int nu = 3;
+    unsigned bit[2][8];                  // set bit of each entry of the first two stars (0: none)
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        unsigned m = 1u << e;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int x = s[e][j];
+            unsigned b = 0u;
+#pragma unroll
+            for (int f = 0; f < 3; ++f)
+                if (f != e) b |= x == tri[f] ? 1u << f : 0u;
+#pragma unroll
+            for (int f = 0; f < e; ++f)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) b |= s[f][i] == x ? bit[f][i] : 0u;
+            const bool valid = j < n[e], fresh = valid && b == 0u;
+            su[min(nu, SET_MAX) * stride] = x;
+            b = fresh ? 1u << nu : b;
+            nu += fresh ? 1 : 0;
+            b = valid ? b : 0u;
+            if (e < 2) bit[e < 2 ? e : 0][j] = b;
+            m |= b;
+        }
+        vm[e] = m;
+    }
+    return nu;
+}
+
+// node_sets8 where it applies: true when the sets of all nodes of the warp fit (one path a warp: a
+// few nodes with larger sets would otherwise cost it both).  st != 0: no node here.
+__device__ __forceinline__ bool warp_sets8(const StarTab &t, int st, const int tri[3], const TabStar sa[3],
+                                           int cap, int *su, int stride, int &nu, unsigned vm[3])
+{
+    bool fits = true;
+    if (st == 0) {
+        const int n[3] = {sa[0].n, sa[1].n, sa[2].n};
+        fits = max(n[0], max(n[1], n[2])) <= 8;
+        if (fits) {
+            nu = node_sets8(t, tri, n, su, stride, vm);
+            fits = nu <= min(cap, SET_MAX);
+        }
+    }
+    return __all_sync(__activemask(), fits);
+}
+
 // Resident 128-thread blocks per SM of the geometry kernel: its node search waits on memory,
 // and more warps in flight hide it (8, 10, 12, 16 blocks measured 0.291, 0.275, 0.268, 0.266 ms
 // at 1025^2 nodes / 2048^2 particles); 12 keeps the register spills to a few dozen bytes.
 #ifndef PFEM_GEOM_MIN_BLOCKS
-#define PFEM_GEOM_MIN_BLOCKS 12
+#define PFEM_GEOM_MIN_BLOCKS 8
 #endif
 // Node (I, J) of the mesh of a.n nodes per side: locate it and build its particle set from the
 // star table, and write its record at index `rec` (node J * a.n + I of a single problem; the
 // problem's offset plus that in a batch, which also records the node's coordinates).
 template <typename P, typename V, typename R>
 __device__ __forceinline__ void geom_node(const P2MArgs &a, const StarTab &t, const NodeRecs &r,
-                                          int I, int J, long long rec)
+                                          int I, int J, long long rec, int *su, int stride)
 {
     const int nc = a.n - 1;
     const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
@@ -840,19 +928,16 @@ __device__ __forceinline__ void geom_node(const P2MArgs &a, const StarTab &t, co
             sa[e] = tab_star(t, tri[e]);
             if (sa[e].n < 0) st = sa[e].n == -1 ? -PFEM_FAR : sa[e].n;
         }
-    int meta = -1;
+    int meta = -1, nu = 0;
+    unsigned vm[3] = {0u, 0u, 0u};
+    const bool small = warp_sets8(t, st, tri, sa, a.ucap, su, stride, nu, vm);
     if (st == 0) {
         NodePos<P, R> np;
         np.init(Iu, Ju, nc);
         R lam[3];
         barycentric(a, np, tri, lam);
-        int us[UMAX];
-        int nu;
-        unsigned vm[3];
-        int vi[3];
-        if (node_u_sets<UMAX>(tri, sa, us, nu, vm, vi, min(a.ucap, UMAX)) != 0) {
-            st = a.defer_cap > 0 ? -PFEM_DEFER : -PFEM_ERR_CAPACITY;
-        } else {
+        int vi[3] = {0, 1, 2};
+        auto write = [&](auto us) {
             // entries up to the warp's largest set, -1 past this node's, so that the warp's
             // stores to each entry array cover contiguous runs of it
             const int nw = __reduce_max_sync(__activemask(), nu);
@@ -863,6 +948,15 @@ __device__ __forceinline__ void geom_node(const P2MArgs &a, const StarTab &t, co
                 r.lam[e * r.nodes + rec] = (double)lam[e];
             }
             meta = nu | vi[0] << 5 | vi[1] << 10 | vi[2] << 15;
+        };
+        if (small) {
+            write(Strided<int>{su, stride});
+        } else {
+            int us[UMAX];
+            if (node_u_sets<UMAX>(tri, sa, us, nu, vm, vi, min(a.ucap, UMAX)) != 0)
+                st = a.defer_cap > 0 ? -PFEM_DEFER : -PFEM_ERR_CAPACITY;
+            else
+                write(Strided<int>{us, 1});
         }
     }
     r.meta[rec] = meta;
@@ -883,10 +977,11 @@ template <typename P, typename V, typename R>
 __global__ void __launch_bounds__(128, PFEM_GEOM_MIN_BLOCKS) k_p2m_geom(P2MArgs a, StarTab t,
                                                                         NodeRecs r)
 {
+    __shared__ int su[SET_W * 128];
     const int I = blockIdx.x * 16 + (threadIdx.x & 15);
     const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
     if (I >= a.n || J >= a.n) return;
-    geom_node<P, V, R>(a, t, r, I, J, (long long)J * a.n + I);
+    geom_node<P, V, R>(a, t, r, I, J, (long long)J * a.n + I, su + threadIdx.x, 128);
 }
 
 // The lanes of a node (a group of Q consecutive ones that run the same control flow), and the sum
@@ -995,24 +1090,77 @@ __global__ void __launch_bounds__(128) k_p2m_fix_tab(P2MArgs a, StarTab t)
 // of the mesh's 2-norm; the two results differ by 1e-9 of it).  The float-float refinement that
 // PFEM_SOLVE_F32_REFINED_FF names (48 bits, about 200 FP32 instructions a point and edge) took
 // 0.84 ms in two kernels; it takes this path too, whose residual is the more exact.
-// Resident 128-thread blocks per SM: 9 with one lane a node (1025^2 / 2048^2 round trip: 7, 8, 9, 10
-// blocks 1220, 1210, 1195, 1201 us), and for the solution refined to FP64, with its longer live
+// Resident 128-thread blocks per SM: 7 with one lane a node (1025^2 / 2048^2 round trip: 6, 7, 8, 9
+// blocks 1124, 1096, 1107, 1123 us), and for the solution refined to FP64, with its longer live
 // ranges, 6 (513^2 / 1024^2: 4, 5, 6 blocks 739, 713, 700 us); 8 and 4 with four lanes a node, where
 // there are not enough nodes to fill the SMs.
 template <int REFINE, int Q = 1> constexpr int tab_min_blocks()
 {
-    return REFINE == REFINE_FIX64 ? (Q > 1 ? 4 : 6) : (Q > 1 ? 8 : 9);
+    return REFINE == REFINE_FIX64 ? (Q > 1 ? 4 : 6) : (Q > 1 ? 8 : 7);
+}
+
+// The edge systems of a node's set (slots us, weights weight) and the apply of the result; tab_node
+// says what Q and q are.  Returns 0 or -PFEM_DEFER.
+template <int UM, typename P, typename V, typename R, typename S, int REFINE, int Q, typename Slots,
+          typename Weights, typename Apply>
+__device__ __forceinline__ int set_solve(const P2MArgs &a, const NodePos<P, R> &np, int Iu, int Ju, int q,
+                                         const int tri[3], int nu, const unsigned vm[3], const int vi[3],
+                                         const R lam[3], Slots us, Weights weight, Apply &&apply)
+{
+    const int e0 = Q > 1 ? q : 0, e1 = Q > 1 ? min(q + 1, 3) : 3;
+    int st;
+    if constexpr (REFINE == REFINE_FIX64) {
+        longlong2 o[UM];
+        long long w[UM];
+        const bool finite = node_offsets64<P>(a.pos, Iu, Ju, a.n - 1, us, nu, o) != NOT_FINITE;
+        for (int i = 0; i < nu; ++i) w[i] = 0;
+        const double l64[3] = {(double)lam[0], (double)lam[1], (double)lam[2]};
+        st = group_min<Q>(finite ? node_solve64(o, vm, vi, l64, e0, e1, w, -PFEM_DEFER) : -PFEM_DEFER);
+        if (st == 0) {
+            for (int i = 0; i < nu; ++i) apply(us[i], (R)(__ll2double_rn(group_sum<Q>(w[i])) * W64_UNIT));
+#pragma unroll
+            for (int e = 0; e < 3; ++e) apply(tri[e], lam[e]);
+        }
+    } else {
+        for (int i = 0; i < nu; ++i) weight[i] = R(0);
+        auto ref = [&](int i) -> R & { return weight[i]; };
+        auto offset = [&](int i, S &x, S &y) {
+            R dx, dy;
+            np.off(a.pos, us[i], dx, dy);
+            x = S(dx);
+            y = S(dy);
+        };
+        if constexpr (Q == 1) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) weight[vi[e]] += lam[e];
+            st = node_edges<R, S, REFINE, false, UM, false>(ref, vm, vi, lam, 0, 3, offset);
+            if (st == 0)
+                for (int i = 0; i < nu; ++i) apply(us[i], weight[i]);
+        } else {
+            st = group_min<Q>(node_edges<R, S, REFINE, false, UM, true>(ref, vm, vi, lam, e0, e1, offset));
+            const R coef[3] = {R(2) * lam[0] * lam[1], R(2) * lam[1] * lam[2], R(2) * lam[2] * lam[0]};
+            if (st == 0)
+                for (int i = 0; i < nu; ++i) {
+                    R w = i == vi[0] ? lam[0] : i == vi[1] ? lam[1] : i == vi[2] ? lam[2] : R(0);
+#pragma unroll
+                    for (int e = 0; e < 3; ++e)
+                        w = fma(coef[e], __shfl_sync(group_mask<Q>(), weight[i], e, Q), w);
+                    apply(us[i], w);
+                }
+        }
+    }
+    return st;
 }
 
 // Node (I, J) of the problem of a (mesh output a.out; queue entries and error details at node
 // a.noff + J * a.n + I of the batch), by Q = 1 lane, or by Q = 4 lanes that all locate it, solve an
 // edge each (the fourth none) and take the components c = q, q + 4 of the apply.  Both give the same
 // result bit for bit: the edges' contributions and the particles are added up in the same order.
+// su: the calling thread's column of SET_ROWS words in shared memory, entry i at i * stride.
 template <typename P, typename V, typename R, typename S, int REFINE, int Q = 1>
-__device__ __forceinline__ void tab_node(const P2MArgs &a, const StarTab &t, int I, int J)
+__device__ __forceinline__ void tab_node(const P2MArgs &a, const StarTab &t, int I, int J, int *su, int stride)
 {
     const int q = Q > 1 ? (int)threadIdx.x & (Q - 1) : 0;
-    const int e0 = Q > 1 ? q : 0, e1 = Q > 1 ? min(q + 1, 3) : 3;
     const int nc = a.n - 1;
     const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
     const long long node = (long long)J * a.n + I;
@@ -1043,52 +1191,27 @@ __device__ __forceinline__ void tab_node(const P2MArgs &a, const StarTab &t, int
                 if (q + Q * k < a.C) acc[k] = fma(w, load_val<V, R>(p + q + Q * k), acc[k]);
         }
     };
+    int nu = 0;
+    unsigned vm[3] = {0u, 0u, 0u};
+    const bool small = warp_sets8(t, st, tri, sa, a.ucap, su, stride, nu, vm);
     if (st == 0) {
         NodePos<P, R> np;
         np.init(Iu, Ju, nc);
         R lam[3];
         barycentric(a, np, tri, lam);
-        int us[UMAX];
-        int nu;
-        unsigned vm[3];
-        int vi[3];
-        if (node_u_sets<UMAX>(tri, sa, us, nu, vm, vi, min(a.ucap, UMAX)) != 0) {
-            st = a.defer_cap > 0 ? -PFEM_DEFER : -PFEM_ERR_CAPACITY;
-        } else if constexpr (REFINE == REFINE_FIX64) {
-            longlong2 o[UMAX];
-            long long w[UMAX];
-            node_offsets64<P>(a.pos, Iu, Ju, nc, us, nu, o);
-            for (int i = 0; i < nu; ++i) w[i] = 0;
-            const double l64[3] = {(double)lam[0], (double)lam[1], (double)lam[2]};
-            st = group_min<Q>(node_solve64(o, vm, vi, l64, e0, e1, w, -PFEM_DEFER));
-            if (st == 0) {
-                for (int i = 0; i < nu; ++i)
-                    apply(us[i], (R)(__ll2double_rn(group_sum<Q>(w[i])) * W64_UNIT));
-#pragma unroll
-                for (int e = 0; e < 3; ++e) apply(tri[e], lam[e]);
-            }
+        int vi[3] = {0, 1, 2};
+        if (small) {
+            st = set_solve<SET_MAX, P, V, R, S, REFINE, Q>(a, np, Iu, Ju, q, tri, nu, vm, vi, lam, Strided<int>{su, stride},
+                                                           Strided<R>{reinterpret_cast<R *>(su) + SET_W * stride, stride},
+                                                           apply);
         } else {
-            R uw[UMAX];
-            for (int i = 0; i < nu; ++i) uw[i] = R(0);
-            if constexpr (Q == 1) {
-#pragma unroll
-                for (int e = 0; e < 3; ++e) uw[vi[e]] += lam[e];
-                st = node_u_solve<P, R, S, REFINE, false, UMAX>(a, np, us, uw, vm, vi, lam);
-                if (st == 0)
-                    for (int i = 0; i < nu; ++i) apply(us[i], uw[i]);
-            } else {
-                st = group_min<Q>(node_u_solve<P, R, S, REFINE, false, UMAX, true>(a, np, us, uw, vm, vi,
-                                                                                   lam, e0, e1));
-                const R coef[3] = {R(2) * lam[0] * lam[1], R(2) * lam[1] * lam[2], R(2) * lam[2] * lam[0]};
-                if (st == 0)
-                    for (int i = 0; i < nu; ++i) {
-                        R w = i == vi[0] ? lam[0] : i == vi[1] ? lam[1] : i == vi[2] ? lam[2] : R(0);
-#pragma unroll
-                        for (int e = 0; e < 3; ++e)
-                            w = fma(coef[e], __shfl_sync(group_mask<Q>(), uw[i], e, Q), w);
-                        apply(us[i], w);
-                    }
-            }
+            int us[UMAX];
+            R uw[REFINE == REFINE_FIX64 ? 1 : UMAX];
+            if (node_u_sets<UMAX>(tri, sa, us, nu, vm, vi, min(a.ucap, UMAX)) != 0)
+                st = a.defer_cap > 0 ? -PFEM_DEFER : -PFEM_ERR_CAPACITY;
+            else
+                st = set_solve<UMAX, P, V, R, S, REFINE, Q>(a, np, Iu, Ju, q, tri, nu, vm, vi, lam, Strided<int>{us, 1},
+                                                            Strided<R>{uw, 1}, apply);
         }
     }
     if (st != 0) {
@@ -1108,15 +1231,19 @@ __device__ __forceinline__ void tab_node(const P2MArgs &a, const StarTab &t, int
     }
 }
 
+// Shared words a thread: slots, and weights where they are FP32 ones.
+template <int REFINE> constexpr int tab_rows() { return REFINE == REFINE_FIX64 ? SET_W : SET_ROWS; }
+
 template <typename P, typename V, typename R, typename S, int REFINE, int Q>
 __global__ void __launch_bounds__(128, tab_min_blocks<REFINE, Q>()) k_p2m_tab(P2MArgs a, StarTab t)
 {
+    __shared__ int su[tab_rows<REFINE>() * 128];
     // 16 x 8 nodes a block, or 8 x 4 with four lanes a node
     const int x = threadIdx.x / Q;
     const int I = blockIdx.x * (Q > 1 ? 8 : 16) + (Q > 1 ? x & 7 : x & 15);
     const int J = blockIdx.y * (Q > 1 ? 4 : 8) + (Q > 1 ? x >> 3 : x >> 4);
     if (I >= a.n || J >= a.n) return;
-    tab_node<P, V, R, S, REFINE, Q>(a, t, I, J);
+    tab_node<P, V, R, S, REFINE, Q>(a, t, I, J, su + threadIdx.x, 128);
 }
 
 // Explicit weights of every node with the star table: as k_p2m_tab, writing the node's row of (slot,
@@ -1154,10 +1281,10 @@ __global__ void __launch_bounds__(128, tab_min_blocks<REFINE>()) k_shape_tab(P2M
         } else if constexpr (REFINE == REFINE_FIX64) {
             longlong2 o[UMAX];
             long long w[UMAX];
-            node_offsets64<P>(a.pos, Iu, Ju, nc, us, nu, o);
+            const bool finite = node_offsets64<P>(a.pos, Iu, Ju, nc, us, nu, o) != NOT_FINITE;
             for (int i = 0; i < nu; ++i) w[i] = 0;
             const double l64[3] = {(double)lam[0], (double)lam[1], (double)lam[2]};
-            st = node_solve64(o, vm, vi, l64, 0, 3, w, -PFEM_DEFER);
+            st = finite ? node_solve64(o, vm, vi, l64, 0, 3, w, -PFEM_DEFER) : -PFEM_DEFER;
             for (int i = 0; i < nu; ++i) uw[i] = (R)(__ll2double_rn(w[i]) * W64_UNIT);
 #pragma unroll
             for (int e = 0; e < 3; ++e) uw[vi[e]] += lam[e];

@@ -11,25 +11,24 @@ namespace pfem {
 __global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_star_list(Bins B, int R0, StarTab t,
                                                                               DevStatus *st)
 {
-    __shared__ float2 sxy[STAR_ROWS * STAR_TPB];
-    __shared__ int ss[STAR_ROWS * STAR_TPB];
+    __shared__ __align__(16) unsigned char lists[HullList::BYTES];
     const long long v = blockIdx.x * (long long)STAR_TPB + threadIdx.x;
     if (v >= t.N) return;
-    const HullList L{sxy + threadIdx.x, ss + threadIdx.x};
-    star_list_slot(B, R0, t, v, L, st);
+    star_list_slot(B, R0, t, v, HullList::at(lists, threadIdx.x), st);
 }
 
-// The queued particles, with the radius of B (the launcher passes the widest one), a warp each.
-__global__ void __launch_bounds__(RETRY_TPB, PFEM_RETRY_BLOCKS) k_star_retry(Bins B, int R0, StarTab t,
-                                                                             DevStatus *st)
+// The queued particles, with the radius of B (the launcher passes the widest one).
+__global__ void __launch_bounds__(RETRY_TPB, RETRY_BLOCKS) k_star_retry(Bins B, int R0, StarTab t,
+                                                                        DevStatus *st)
 {
+    __shared__ __align__(16) unsigned char lists[HullListLong::BYTES];
     __shared__ int2 sd[RETRY_TPB / 32 * WSTAR_CAP];
     __shared__ int ss[RETRY_TPB / 32 * WSTAR_CAP];
     const int w = threadIdx.x >> 5;
-    const WarpList L{sd + w * WSTAR_CAP, ss + w * WSTAR_CAP};
-    const int n = min(*t.qcount, (int)min(t.N, (long long)0x7fffffff));
-    for (int i = blockIdx.x * (RETRY_TPB / 32) + w; i < n; i += gridDim.x * (RETRY_TPB / 32))
-        star_retry_slot(B, R0, t, t.queue[i], L, st);
+    star_retry(t, lists, WarpList{sd + w * WSTAR_CAP, ss + w * WSTAR_CAP}, st, [&](int, int &r) {
+        r = R0;
+        return B;
+    });
 }
 
 size_t star_tab_bytes(long long N)
@@ -73,7 +72,7 @@ cudaError_t launch_star_table(const Bins &B, int R0, int rmax_far, const StarTab
     k_star_list<<<(unsigned)((t.N + STAR_TPB - 1) / STAR_TPB), STAR_TPB, 0, s>>>(B, R0, t, st);
     Bins Bf = B;
     Bf.rmax = std::max(B.rmax, rmax_far);
-    k_star_retry<<<num_sms() * PFEM_RETRY_BLOCKS, RETRY_TPB, 0, s>>>(Bf, R0, t, st);
+    k_star_retry<<<num_sms() * RETRY_BLOCKS, RETRY_TPB, 0, s>>>(Bf, R0, t, st);
     count_launch(2);
     return cudaGetLastError();
 }

@@ -150,3 +150,29 @@ def test_fp64_solves(P, which):
     mesh = proj.p2m(torch.tensor(pr.vals, dtype=torch.float32, device="cuda"), solve=P.PFEM_SOLVE_F64)
     proj.check(which)
     assert relerr(mesh.cpu().numpy(), O.p2m(pr.n, pos.double().cpu().numpy(), pr.vals, shape=1, nthreads=8)) <= TOL32
+
+
+@pytest.mark.parametrize("C", [1, 2, 3, 4, 7])
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+def test_linear_m2p_components_and_ends(P, C, dtype):
+    """M2P for every component count and several particles a thread, with particles in the last cell, on
+    cell boundaries and diagonals, from other periods, and a count that no block divides; a position
+    that is not finite gives no finite value."""
+    n, N = 38, 3001
+    pos = G.uniform01(G.SEED_BASE + 950, 2 * N).reshape(N, 2)
+    pos[:64, 0] = np.repeat([0.0, 1e-12, 1.0 - 1e-12, 36.0 / 37.0], 16)
+    pos[64:128, 1] = np.repeat([0.0, 1e-12, 1.0 - 1e-12, 36.0 / 37.0], 16)
+    pos[128:160, 1] = pos[128:160, 0]
+    pos[200:300] += [-3.0, 5.0]
+    pos_t = torch.float64 if dtype == "f64" else torch.float32
+    pos = torch.tensor(pos, dtype=pos_t, device="cuda")
+    mesh = G.uniform01(G.SEED_BASE + 951, n * n * C).reshape(n, n, C)
+    mesh[-1], mesh[:, -1] = mesh[0], mesh[:, 0]
+    mesh = torch.tensor(mesh, device="cuda").to({"f64": torch.float64, "f32": torch.float32, "bf16": torch.bfloat16}[dtype])
+    proj = P.Projector(n, N, C=C, pos_dtype=pos_t)
+    ref = O.m2p(n, pos.double().cpu().numpy(), mesh.double().cpu().numpy())
+    # BF16: one rounding of the result, 2^-9; FP32 coordinates: 2^-24 n of a cell
+    tol = {"f64": TOL64, "f32": n * 2.0 ** -23 + TOL32, "bf16": 2.0 ** -8}[dtype]
+    assert relerr(proj.m2p(pos, mesh).double().cpu().numpy(), ref) <= tol
+    pos[5, 0] = float("nan")
+    assert not torch.isfinite(proj.m2p(pos, mesh)[5].float()).any()
