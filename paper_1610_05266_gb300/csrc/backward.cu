@@ -920,24 +920,24 @@ static cudaError_t bwd_t(const GeoArgs &g, const int *perm, int C, const void *v
     node_recs_layout(ws + L.rec, b.nodes, &recs);
     b.e_cnt = recs.meta;
     // the star table's queue counter sits in the status block, after the status word
-    const StarTab tab = star_tab_layout(ws + L.tab, g.N, (int *)(ws + 64));
+    const StarTab tab = star_tab_layout(ws + L.tab, g.N, (int *)(ws + 64));   // (right before the fix-pass counter)
     // the fix-pass queue: its counter in the status block, one entry per node
     b.f.defer_count = (int *)(ws + 68);
     b.f.defer_list = (long long *)(ws + L.queue);
     b.f.defer_cap = (int)std::min(b.nodes, (long long)0x7fffffff);
     auto node_pass = [&](auto pos) {
         constexpr bool POS = decltype(pos)::value;
-        cudaMemsetAsync(b.f.defer_count, 0, sizeof(int), s);
         cudaMemsetAsync(b.count, 0, 4 * (size_t)(g.N + 1), s);
         if constexpr (SHAPE == PFEM_SHAPE_QUADRATIC) {
             // a star that no node needs may fail unnoticed with FP64 systems, whose adjoint has always
             // looked at the needed ones only: a scratch status word
             DevStatus *st = sizeof(S) == 8 ? (DevStatus *)(ws + 128) : b.f.status;
-            launch_star_table(b.f.B, g.R0, g.rmax_far, tab, st, s);
+            launch_star_table(b.f.B, g.R0, g.rmax_far, tab, st, s, 1);     // and the fix-pass counter
             k_p2m_geom<P, V, R><<<grid, 128, 0, s>>>(b.f, tab, recs);
             k_bwd_solve<P, V, R, S, POS><<<(unsigned)((b.nodes + 127) / 128), 128, 0, s>>>(b, recs);
             count_launch(2);
         } else {
+            cudaMemsetAsync(b.f.defer_count, 0, sizeof(int), s);
             k_bwd_linear<P, V, R, POS><<<grid, 128, 0, s>>>(b);
             count_launch();
         }

@@ -86,8 +86,9 @@ struct Bins;
 size_t star_tab_bytes(long long N);
 unsigned next_tab_gen();
 StarTab star_tab_layout(char *base, long long N, int *qcount);
+// The launcher clears *t.qcount and the `also` ints behind it (a caller's other counters).
 cudaError_t launch_star_table(const Bins &B, int R0, int rmax_far, const StarTab &t,
-                              DevStatus *st, cudaStream_t s);
+                              DevStatus *st, cudaStream_t s, int also = 0);
 
 
 cudaError_t launch_p2m(const GeoArgs &g, const int *perm, int C, const void *vals,

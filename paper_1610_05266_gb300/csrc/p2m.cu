@@ -73,7 +73,7 @@ static cudaError_t go_fast(const P2MArgs &a, cudaStream_t s)
 static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Workspace layout of P2M after the 256-byte status block: the fix-pass queue counter at byte
-// 256 and the star-table queue counter at byte 260, the fix-pass queue from byte 512 (8 bytes
+// 256 and the star-table queue counter right before it, the fix-pass queue from byte 512 (8 bytes
 // per node), then a record's space per node (the adjoint's layout) and the star table.
 static size_t recs_offset(long long nodes) { return al256(512 + 8 * (size_t)nodes); }
 
@@ -91,7 +91,7 @@ static bool set_table(StarTab &t, void *ws, size_t ws_bytes, long long nodes, lo
     char *base = (char *)ws + recs_offset(nodes);
     NodeRecs r;
     const size_t recs = al256(node_recs_layout(nullptr, nodes, &r));
-    t = star_tab_layout(base + recs, N, (int *)((char *)ws + 260));
+    t = star_tab_layout(base + recs, N, (int *)((char *)ws + 252));
     return true;
 }
 
@@ -108,7 +108,8 @@ static cudaError_t go(const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
     const int R0 = g.R0, rmax_far = g.rmax_far;
     cudaError_t e;
     stage_event(g, 0, s);
-    if (a.defer_cap > 0) {
+    // the star table's launcher clears both queue counters, which lie side by side
+    if (a.defer_cap > 0 && !(SHAPE == PFEM_SHAPE_QUADRATIC && tab)) {
         e = cudaMemsetAsync(a.defer_count, 0, sizeof(int), s);
         if (e != cudaSuccess) return e;
     }
@@ -116,7 +117,7 @@ static cudaError_t go(const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
         if constexpr (SHAPE == PFEM_SHAPE_QUADRATIC && W) {
             // a star that no node needs may fail unnoticed, as where each node searches its own: a
             // scratch status word
-            e = launch_star_table(a.B, R0, rmax_far, *tab, (DevStatus *)((char *)a.status + 128), s);
+            e = launch_star_table(a.B, R0, rmax_far, *tab, (DevStatus *)((char *)a.status + 128), s, 1);
             if (e != cudaSuccess) return e;
             const bool vec = a.K % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.w_idx) | reinterpret_cast<uintptr_t>(a.w)) & 31) == 0;
             k_shape_tab<P, R, sizeof(S) == 8 ? REFINE_FIX64 : REF><<<node_grid(a.n), 128, 0, s>>>(a, *tab, vec);
@@ -124,7 +125,7 @@ static cudaError_t go(const GeoArgs &g, const P2MArgs &a, cudaStream_t s,
             e = cudaGetLastError();
         }
     } else if (SHAPE == PFEM_SHAPE_QUADRATIC && !W && tab) {
-        e = launch_star_table(a.B, R0, rmax_far, *tab, a.status, s);
+        e = launch_star_table(a.B, R0, rmax_far, *tab, a.status, s, 1);
         if (e != cudaSuccess) return e;
         stage_event(g, 1, s);
         stage_event(g, 2, s);

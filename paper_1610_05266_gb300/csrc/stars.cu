@@ -64,10 +64,10 @@ StarTab star_tab_layout(char *base, long long N, int *qcount)
 }
 
 cudaError_t launch_star_table(const Bins &B, int R0, int rmax_far, const StarTab &t,
-                              DevStatus *st, cudaStream_t s)
+                              DevStatus *st, cudaStream_t s, int also)
 {
     if (t.N <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(t.qcount, 0, sizeof(int), s);
+    cudaError_t e = cudaMemsetAsync(t.qcount, 0, sizeof(int) * (size_t)(1 + also), s);
     if (e != cudaSuccess) return e;
     k_star_list<<<(unsigned)((t.N + STAR_TPB - 1) / STAR_TPB), STAR_TPB, 0, s>>>(B, R0, t, st);
     Bins Bf = B;
