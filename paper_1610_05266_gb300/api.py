@@ -286,7 +286,7 @@ class Projector:
             # only the status block needs to start as zeros
             torch.empty((ws_bytes + 15) // 16 * 2, dtype=torch.float64, device=dev),
         )
-        self.reset_status()
+        self.cells.ws[:32].zero_()
 
     @property
     def ws(self) -> torch.Tensor:
