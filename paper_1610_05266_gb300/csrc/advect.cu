@@ -21,7 +21,7 @@ template <typename R> __device__ __forceinline__ R cell_coord(R x, int i, int nc
 {
     const R xw = x - floor(x);
     R s = fma(xw, (R)nc, (R)(-i));
-    if (s > (R)(0.5 * nc)) s -= (R)nc;                  // fixed point rounded up to 2^32 -> cell 0
+    if (s > (R)0.5 * (R)nc) s -= (R)nc;                  // fixed point rounded up to 2^32 -> cell 0
     return s;
 }
 

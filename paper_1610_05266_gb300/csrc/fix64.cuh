@@ -17,8 +17,8 @@
 // rounding of the same sums is 2^-53 of their largest terms.  The sums may wrap: the residual
 // itself is small.
 //
-// Measured (round trip, FP64 values): 513^2 nodes / 1024^2 particles 1798 -> 700 us (node kernel
-// 1475 -> 455), 33^2 / 64^2 200 -> 101 us with four lanes a node; the mesh's error against 64-bit
+// Measured (round trip, FP64 values): 513^2 nodes / 1024^2 particles 1798 -> 643 us (node kernel
+// 1475 -> 455), 33^2 / 64^2 200 -> 89 us with four lanes a node; the mesh's error against 64-bit
 // arithmetic 2.6e-16 -> 1.6e-16 of its 2-norm.
 #pragma once
 

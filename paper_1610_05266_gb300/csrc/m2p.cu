@@ -17,8 +17,8 @@ namespace pfem {
 
 // Particles a thread, 256 apart: their loads are in flight together.  8192^2 particles of one BF16
 // component 632 -> 314 us with four (their bytes take 104 us), 1254^2 of three FP32 ones 18 -> 13
-// us with two; four FP32 components, whose three 16-byte gathers keep enough in flight, 23 us with
-// one and 29 with two.  FP64 positions in fixed point (m2p.cuh): 1024^2 of three 63 -> 26 us.
+// us with two; the round trip of four FP32 ones at 1025^2 / 2048^2 1061 us with one and 1057 with two;
+// four FP64 ones keep enough in flight with one.  FP64 positions in fixed point (m2p.cuh): 1024^2 of three 63 -> 26 us.
 template <typename P, typename V, typename R, int CT, int U>
 __global__ void __launch_bounds__(256) k_m2p(int n, long long N, const P *__restrict__ pos,
                                              int Crt, const V *__restrict__ mesh,
@@ -43,7 +43,7 @@ static cudaError_t m2p_t(int n, long long N, const void *pos, int C, const void 
     if (C == 1) go(std::integral_constant<int, 1>(), std::integral_constant<int, 4>());
     else if (C == 2) go(std::integral_constant<int, 2>(), std::integral_constant<int, 4>());
     else if (C == 3) go(std::integral_constant<int, 3>(), std::integral_constant<int, 2>());
-    else if (C == 4 && (aligned || sizeof(V) != 4)) go(std::integral_constant<int, 4>(), std::integral_constant<int, 1>());
+    else if (C == 4 && (aligned || sizeof(V) != 4)) go(std::integral_constant<int, 4>(), std::integral_constant<int, sizeof(R) == 8 ? 1 : 2>());
     else go(std::integral_constant<int, 0>(), std::integral_constant<int, 1>());
     count_launch();
     return cudaGetLastError();

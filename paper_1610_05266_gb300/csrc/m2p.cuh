@@ -15,11 +15,13 @@ template <typename R> struct MeshCell {
     R w0, w1, w2;
 };
 
+// Half of nc is taken in R: an FP32 particle with the three FP64-pipe instructions of (R)(0.5 * nc)
+// held M2P at 41 us for 2048^2 particles of four components (23 without).
 template <typename R> __device__ __forceinline__ R local_coord(R x, int i, int nc)
 {
     const R xw = x - floor(x);                          // exact
     R s = fma(xw, (R)nc, (R)(-i));
-    if (s > (R)(0.5 * nc)) s -= (R)nc;                  // fixed point rounded up to 2^32 -> cell 0
+    if (s > (R)0.5 * (R)nc) s -= (R)nc;                  // fixed point rounded up to 2^32 -> cell 0
     return s;
 }
 

@@ -902,9 +902,9 @@ __device__ __forceinline__ bool warp_sets8(const StarTab &t, int st, const int t
     return __all_sync(__activemask(), fits);
 }
 
-// Resident 128-thread blocks per SM of the geometry kernel: its node search waits on memory,
-// and more warps in flight hide it (8, 10, 12, 16 blocks measured 0.291, 0.275, 0.268, 0.266 ms
-// at 1025^2 nodes / 2048^2 particles); 12 keeps the register spills to a few dozen bytes.
+// Resident 128-thread blocks per SM of the geometry kernel: its node search waits on memory, and
+// its particle sets in shared memory and registers want room (the whole gradient step at 1025^2
+// nodes / 2048^2 particles, C = 1, FP32, with 6, 8, 10, 12 blocks: 2395, 2369, 2372, 2391 us).
 #ifndef PFEM_GEOM_MIN_BLOCKS
 #define PFEM_GEOM_MIN_BLOCKS 8
 #endif
@@ -1085,8 +1085,9 @@ __global__ void __launch_bounds__(128) k_p2m_fix_tab(P2MArgs a, StarTab t)
 // The table path's fast pass in one kernel: each thread locates its node with the star table,
 // builds its particle set and solves its three edge systems, without a node record in between.
 // The refined solve's residual runs on the integer pipes (FixRes); in FP64 it held the FP64 pipe
-// for 0.47 ms of this kernel's 0.99 ms at 1025^2 nodes / 2048^2 particles, C = 4, FP32 (now 0.67
-// ms; 4097^2 / 8192^2: 14.6 -> 9.6 ms).  Errors against 64-bit arithmetic are unchanged (1.1e-7
+// for 0.47 ms of this kernel's 0.99 ms at 1025^2 nodes / 2048^2 particles, C = 4, FP32 (now 0.56
+// ms with the sets in shared memory; 4097^2 / 8192^2: 14.6 -> 8.2 ms).  What bounds it now are the
+// waits for star rows and positions in L2 (24 of 32 lanes active).  Errors against 64-bit arithmetic are unchanged (1.1e-7
 // of the mesh's 2-norm; the two results differ by 1e-9 of it).  The float-float refinement that
 // PFEM_SOLVE_F32_REFINED_FF names (48 bits, about 200 FP32 instructions a point and edge) took
 // 0.84 ms in two kernels; it takes this path too, whose residual is the more exact.
