@@ -3,23 +3,26 @@
 // An SM of GB300 issues two FP64 instructions a clock, so a warp's FP64 instruction takes its
 // scheduler 64 cycles; assembling, factoring and solving the three 6 x 6 systems of a node in FP64
 // took about 2600 of them.  Here each edge system is factored in FP32 and its solution y
-// refined until it is exact to the last bits of a 64-bit fixed-point number: residuals r = b - M y in
-// 64-bit fixed point on the integer pipes, corrections through the FP32 factor.  Each step gains
-// the bits that FP32 has over the system's condition (about 11 on jittered lattices: four
-// steps), at about 100 integer instructions a stencil point.  Positions enter as 64-bit fixed
-// point too: an offset between two of them is exact where FP64 rounds it.
+// refined in 64-bit fixed point: residuals r = b - M y on the integer pipes, corrections through the
+// FP32 factor, each step gaining the bits that FP32 has over the system's condition (on jittered
+// lattices two steps, at about 100 integer instructions a stencil point).  Positions enter as 64-bit
+// fixed point too: an offset between two of them is exact where FP64 rounds it.
 //
 // Scaling, all by powers of two: coordinates X in Q64, |X| < 1/2, from the largest of the
 // stencil; y'_k = y_k g^deg(k) and b' likewise, as integers with unit 2^-s, |y'|, |b'| <= 2^(60 - s); t
-// = p . y, X t, Y t and the sums in the same unit.  |t| <= 2.75 of the largest |y'|.  A product is
-// rounded within 1.5 units; with the largest coordinate at 1/4 to 1/2 and an edge of a fifth of
-// the stencil the unit is 2^-57 or below against coefficients A = p . y of about 0.3: FP64's
-// rounding of the same sums is 2^-53 of their largest terms.  The sums may wrap: the residual
-// itself is small.
+// = p . y in the same unit, |t| <= 2.75 of the largest |y'|.  A product is rounded within 1.5 units.
+// t itself is the coefficient A, which on irregular stencils is far below |y'| (an edge short beside
+// its stencil, particles close together): it is shifted up by its headroom of 2^h before X t, Y t
+// and the sums are formed, so that their rounding, which the inverse of M enlarges, is in units of
+// 2^-(s + h) (the rounding of t is not enlarged: P^T M^-1 P is a projection).  The sums may wrap:
+// the residual itself is small.
 //
-// Measured (round trip, FP64 values): 513^2 nodes / 1024^2 particles 1798 -> 643 us (node kernel
-// 1475 -> 455), 33^2 / 64^2 200 -> 89 us with four lanes a node; the mesh's error against 64-bit
-// arithmetic 2.6e-16 -> 1.6e-16 of its 2-norm.
+// Error of the coefficients against 128-bit arithmetic, the largest of an edge over its largest
+// coefficient; the FP64 Cholesky of the same edges in brackets:
+//   lattice, jitter 0.3, 504,000 edges   median 4e-17 (8e-16), 99.9 % 7e-16 (4e-15), worst 8e-15 (1e-14)
+//   uniform random, 504,000 edges        median 2e-16 (1e-15), 99.9 % 1e-14 (2e-14), worst 2e-13 (8e-13)
+// Before the shift by h, with a stalled refinement accepted at 2^-36 of the largest |y'|, the uniform
+// random set's were 7e-16, 6e-14 and 2e-11.
 #pragma once
 
 #include "moments.cuh"
@@ -93,10 +96,13 @@ struct EdgeFix64 {
         const Split64 v = split64(Y2 + mul64(Z, Y[5]));
         return Y0 + mul64(X, u) + mul64(Z, v);
     }
-    // r -= p (p . y)
-    __device__ __forceinline__ void residual(Split64 X, Split64 Z, long long r[6]) const
+    // r -= p (p . y) 2^h; tm: the largest upper half of |p . y|
+    __device__ __forceinline__ void residual(Split64 X, Split64 Z, int h, long long r[6], int &tm) const
     {
-        const long long t = value(X, Z);
+        long long t = value(X, Z);
+        const int top = (int)(t >> 32);
+        tm = max(tm, top ^ (top >> 31));
+        t <<= h;
         const Split64 ts = split64(t);
         const long long xt = mul64(X, ts), zt = mul64(Z, ts);
         const Split64 xs = split64(xt), zs = split64(zt);
@@ -155,8 +161,8 @@ template <int UM> struct EdgeSystem {
     {
     }
 
-    // Assemble and factor; false when the system is below the FP32 fast-solve tolerance.
-    __device__ __forceinline__ bool factor()
+    // Assemble and factor; false when a pivot is below `least` of the trace.
+    __device__ __forceinline__ bool factor(float least)
     {
         M.zero();
         int hm = 0;
@@ -171,7 +177,7 @@ template <int UM> struct EdgeSystem {
         const float l2 = fmaf(ex, ex, ey * ey);
         // the tolerance of the system scaled by the edge length: pivots of degree d carry l^2d
         const float i2 = 1.f / l2, i4 = i2 * i2;
-        const float tol = FastTol<float>::v *
+        const float tol = least *
                           (M.m[tri_ix(0, 0)] + (M.m[tri_ix(1, 1)] + M.m[tri_ix(2, 2)]) * i2 +
                            (M.m[tri_ix(3, 3)] + M.m[tri_ix(4, 4)] + M.m[tri_ix(5, 5)]) * i4);
         const float t1 = tol * l2, t2 = t1 * l2;
@@ -203,8 +209,16 @@ template <int UM> struct EdgeSystem {
         return s >= 20;
     }
 
-    // Y = y in units 2^-s, refined until M' Y = B to the last bits.
-    __device__ __forceinline__ bool refine(const float y[6], int s, float ym, const long long B[6],
+    // Y = y in units 2^-s, refined until M' Y = B.  ym: the largest of |y|; ref: a value that the
+    // largest |p . y| is not to be taken below.  False when that is not reached.
+    //
+    // A step's correction d shrinks by about its ratio to the one before, so the next one is expected at
+    // d^2 / last.  It is left out when it is below 2^-51 (top / ym), top the largest |p . y|: where y
+    // is large beside its values the ratios are uneven.  A correction that shrinks no more is the floor
+    // that the residual's rounding sets.  It is accepted where the values it changes, whose 2-norm is
+    // the root of d . r (r = M d), stay below 2^-50 of top; else the system is left to FP64, which takes 0.1 % of the
+    // edges of a uniform random set and none of a jittered lattice's.
+    __device__ __forceinline__ bool refine(const float y[6], int s, float ym, float ref, const long long B[6],
                                            long long Y[6]) const
     {
         const float us = pow2(-s), sc = pow2(s - 60);
@@ -212,30 +226,38 @@ template <int UM> struct EdgeSystem {
         for (int q = 0; q < 6; ++q) Y[q] = __float2ll_rn(y[q] * unit(q) * sc * 1152921504606846976.0f);
         EdgeFix64 E;
         float last = ym;                 // the correction before
+        int h = 0;                       // headroom of t in the pass before, less a bit for its change
         for (int it = 0; it < 12; ++it) {
             E.set(Y);
             long long r[6];
+            int tm = 0;
 #pragma unroll
-            for (int q = 0; q < 6; ++q) r[q] = B[q];
+            for (int q = 0; q < 6; ++q) r[q] = B[q] << h;
             for (unsigned m = mask; m; m &= m - 1) {
                 Split64 X, Z;
                 coords(__ffs(m) - 1, X, Z);
-                E.residual(X, Z, r);
+                E.residual(X, Z, h, r, tm);
             }
-            float rf[6], d[6], dm = 0.f;
+            const float uh = us * pow2(-h), top = fmaxf(((float)tm + 1.f) * pow2(32 - s), ref);
+            float rf[6], d[6], dm = 0.f, v2 = 0.f;
 #pragma unroll
-            for (int q = 0; q < 6; ++q) rf[q] = __ll2float_rn(r[q]) * us * unit(q);
+            for (int q = 0; q < 6; ++q) rf[q] = __ll2float_rn(r[q]) * uh * unit(q);
             M.solve(rf, d);
 #pragma unroll
             for (int q = 0; q < 6; ++q) {
+                v2 = fmaf(d[q], rf[q], v2);
                 d[q] *= unit(q);
                 dm = fmaxf(dm, fabsf(d[q]));
                 Y[q] += __float2ll_rn(d[q] * sc * 1152921504606846976.0f);
             }
-            // 2^-43: the next correction would be smaller by this one's ratio to the last; or the
-            // floor that the rounding of the residual sets, if it is below 2^-36
-            if (dm <= 1.1368683772161603e-13f * ym || (dm > 0.5f * last && dm <= 1.4551915228366852e-11f * ym))
-                return true;
+            // (the first pass has no headroom yet; a t that has outgrown it has spoilt the sums)
+            if (it > 0 && tm < 1 << (29 - h)) {
+                if (dm <= 1.1102230246251565e-16f * top ||
+                    dm * dm * ym <= 4.440892098500626e-16f * last * top * top)
+                    return true;
+                if (dm > 0.25f * last) return fabsf(v2) <= 7.888609052210118e-31f * top * top;
+            }
+            h = min(max(__clz((int)((unsigned)tm + 1u)) - 4, 0), 16);
             last = dm;
         }
         return false;
@@ -256,10 +278,11 @@ template <int UM> struct EdgeSystem {
         const long long B[6] = {0, 0, 0, -((__mul64hi(xn, xn) + half) >> (63 - s)),
                                 -((__mul64hi(xn, yn) + half) >> (63 - s)),
                                 -((__mul64hi(yn, yn) + half) >> (63 - s))};
-        return refine(y, s, ym, B, Y);
+        return refine(y, s, ym, 0.f, B, Y);
     }
 
-    // z with M z = u, u' in units 2^-56 (|u'| < 2^7): the adjoint's right-hand side.
+    // z with M z = u, u' in units 2^-56 (|u'| < 2^7): the adjoint's right-hand side, formed of values whose
+    // largest is 1/2 to 1.
     __device__ __forceinline__ bool solve_adjoint(const long long u[6], long long Z[6], int &s) const
     {
         float uf[6], ux[6], z[6];
@@ -275,7 +298,7 @@ template <int UM> struct EdgeSystem {
 #pragma unroll
         for (int q = 0; q < 6; ++q)
             B[q] = s >= 56 ? u[q] << (s - 56) : (u[q] + (1ll << (55 - s))) >> (56 - s);
-        return refine(z, s, zm, B, Z);
+        return refine(z, s, zm, 0.5f, B, Z);
     }
 };
 
@@ -295,7 +318,7 @@ __device__ __forceinline__ int node_solve64(const longlong2 (&o)[UM], const unsi
         EdgeSystem<UM> sys(o, vm[e] | vm[f], o[vi[e]], o[vi[f]]);
         long long Y[6];
         int s;
-        if (!sys.factor() || !sys.solve_coefficients(Y, s)) return defer;
+        if (!sys.factor(FastTol<float>::v) || !sys.solve_coefficients(Y, s)) return defer;
         EdgeFix64 E;
         E.set(Y);
         const double coef = 2.0 * lam[e] * lam[f];

@@ -176,3 +176,43 @@ def test_linear_m2p_components_and_ends(P, C, dtype):
     assert relerr(proj.m2p(pos, mesh).double().cpu().numpy(), ref) <= tol
     pos[5, 0] = float("nan")
     assert not torch.isfinite(proj.m2p(pos, mesh)[5].float()).any()
+
+
+def clustered(n, m, seed):
+    """Half of the particles uniform, half in 64 normal clusters of standard deviation 0.02."""
+    k = m * m // 2
+    u = G.uniform01(G.SEED_BASE + seed, 2 * m * m + 2 * k + 128)
+    a, r, c = u[:2 * (m * m - k)].reshape(-1, 2), u[2 * (m * m - k):-128][:2 * k].reshape(k, 2), u[-128:].reshape(64, 2)
+    d = 0.02 * np.sqrt(-2 * np.log(1 - r[:, :1])) * np.stack([np.cos(2 * np.pi * r[:, 1]), np.sin(2 * np.pi * r[:, 1])], 1)
+    p = c[np.arange(k) % 64] + d
+    pos = np.concatenate([a, p - np.floor(p)])
+    return G.Problem("clustered", n, m, 0.0, 0, pos, G.taylor_green(pos))
+
+
+IRREGULAR = {"uniform": lambda: uniform(513, 1024, 71), "clustered": lambda: clustered(257, 512, 81)}
+
+
+def noise(N, C=8):
+    return 2.0 * G.uniform01(G.SEED_BASE + 960, C * N).reshape(N, C) - 1.0
+
+
+def per_node(got, ref, w):
+    """Largest error of a node over its weights' sum of magnitudes (values within one)."""
+    n = ref.shape[0]
+    return (np.abs(got - ref).max(-1) / np.abs(w).sum(-1).reshape(n, n)).max()
+
+
+@pytest.mark.parametrize("which", sorted(IRREGULAR))
+def test_fp64_weights_on_irregular_sets(P, which):
+    """Explicit FP64 weights on particle sets with short edges beside wide stencils and ill-conditioned
+    systems: at every node, not only where the mesh is largest, the image of white noise within
+    FP64's 1e-12 of the oracle's, over the node's sum of weights."""
+    pr = IRREGULAR[which]()
+    v = noise(pr.N)
+    proj = P.Projector(pr.n, pr.N, C=8, pos_dtype=torch.float64)
+    proj.build(torch.tensor(pr.pos, device="cuda"))
+    w_idx, w = proj.shape_weights()
+    proj.check(which)
+    got = proj.p2m(torch.tensor(v, device="cuda"), weights=(w_idx, w))
+    ref = O.p2m(pr.n, pr.pos, v, shape=1, nthreads=16)
+    assert per_node(got.cpu().numpy(), ref, w.cpu().numpy()) <= TOL64
