@@ -161,8 +161,8 @@ template <int UM> struct EdgeSystem {
     {
     }
 
-    // Assemble and factor; false when a pivot is below `least` of the trace.
-    __device__ __forceinline__ bool factor(float least)
+    // Assemble and factor; false when the system is below the FP32 fast-solve tolerance.
+    __device__ __forceinline__ bool factor()
     {
         M.zero();
         int hm = 0;
@@ -177,7 +177,7 @@ template <int UM> struct EdgeSystem {
         const float l2 = fmaf(ex, ex, ey * ey);
         // the tolerance of the system scaled by the edge length: pivots of degree d carry l^2d
         const float i2 = 1.f / l2, i4 = i2 * i2;
-        const float tol = least *
+        const float tol = FastTol<float>::v *
                           (M.m[tri_ix(0, 0)] + (M.m[tri_ix(1, 1)] + M.m[tri_ix(2, 2)]) * i2 +
                            (M.m[tri_ix(3, 3)] + M.m[tri_ix(4, 4)] + M.m[tri_ix(5, 5)]) * i4);
         const float t1 = tol * l2, t2 = t1 * l2;
@@ -318,7 +318,7 @@ __device__ __forceinline__ int node_solve64(const longlong2 (&o)[UM], const unsi
         EdgeSystem<UM> sys(o, vm[e] | vm[f], o[vi[e]], o[vi[f]]);
         long long Y[6];
         int s;
-        if (!sys.factor(FastTol<float>::v) || !sys.solve_coefficients(Y, s)) return defer;
+        if (!sys.factor() || !sys.solve_coefficients(Y, s)) return defer;
         EdgeFix64 E;
         E.set(Y);
         const double coef = 2.0 * lam[e] * lam[f];

@@ -61,6 +61,12 @@ __device__ __forceinline__ int defer_or_error(const P2MArgs &a, int st, long lon
     return PFEM_DEFERRED;
 }
 
+// A queue that does not hold every node of the mesh (a small workspace, or none) is left to the nodes
+// that FP64's own pivot tolerance sends to the SVD: the more that the FP32 factor of the refined
+// solve cannot carry (fix64.cuh; 0.3 % of a uniform random set's) would fill it.  Those are solved
+// in place by the FP64 Cholesky.
+__device__ __forceinline__ bool short_queue(const P2MArgs &a) { return a.defer_cap < (long long)a.n * a.n; }
+
 // Minimum-norm least-squares solution of P A = b (App. A: the SVD with rank detection), for the
 // 6 x k matrix P whose columns are the stencil's monomial vectors; pt holds P^T (k rows of 6,
 // k <= SVD_ROWS) and is overwritten.  jacobi_svd gives P^T V = W with orthogonal columns
@@ -637,8 +643,7 @@ __device__ __forceinline__ void p2m_node(const P2MArgs &a, int I, int J)
                 const ArrStar sa[3] = {{stars[0], ns[0]}, {stars[1], ns[1]}, {stars[2], ns[2]}};
                 if constexpr (REFINE == REFINE_FIX64) {
                     st = node_quadratic64<P, R>(a, Iu, Ju, tri, sa, lam, emit);
-                    // no fix pass to leave it to: FP64's own pivot tolerance decides (nothing was emitted)
-                    if (st == -PFEM_DEFER && a.defer_cap <= 0)
+                    if (st == -PFEM_DEFER && short_queue(a))          // (nothing was emitted)
                         st = node_quadratic<P, R, double, REFINE_NONE, false>(a, np, tri, sa, lam, emit);
                 } else {
                     st = node_quadratic<P, R, S, REFINE, SVD>(a, np, tri, sa, lam, emit);
@@ -670,8 +675,7 @@ __device__ __forceinline__ void p2m_node(const P2MArgs &a, int I, int J)
                 const ArrStar sa[3] = {{stars[0], ns[0]}, {stars[1], ns[1]}, {stars[2], ns[2]}};
                 if constexpr (REFINE == REFINE_FIX64) {
                     st = node_quadratic64<P, R>(a, Iu, Ju, tri, sa, lam, emit);
-                    // no fix pass to leave it to: FP64's own pivot tolerance decides (nothing was emitted)
-                    if (st == -PFEM_DEFER && a.defer_cap <= 0)
+                    if (st == -PFEM_DEFER && short_queue(a))          // (nothing was emitted)
                         st = node_quadratic<P, R, double, REFINE_NONE, false>(a, np, tri, sa, lam, emit);
                 } else {
                     st = node_quadratic<P, R, S, REFINE, SVD>(a, np, tri, sa, lam, emit);

@@ -216,3 +216,28 @@ def test_fp64_weights_on_irregular_sets(P, which):
     got = proj.p2m(torch.tensor(v, device="cuda"), weights=(w_idx, w))
     ref = O.p2m(pr.n, pr.pos, v, shape=1, nthreads=16)
     assert per_node(got.cpu().numpy(), ref, w.cpu().numpy()) <= TOL64
+
+
+@pytest.mark.parametrize("room", [0, 16])
+def test_fp64_with_a_short_queue(P, room):
+    """Uniform random particles, FP64, in a workspace whose fix-pass queue holds no or 16 nodes: about
+    a hundred nodes' systems are beyond the FP32 factor, and the few that FP64's pivot
+    tolerance queues still fit.  Without a queue exactly those report PFEM_ERR_DEGENERATE."""
+    from paper_1610_05266_gb300 import api
+    pr = uniform(129, 256, 970)
+    proj = P.Projector(pr.n, pr.N, C=pr.C, pos_dtype=torch.float64)
+    proj.build(torch.tensor(pr.pos, device="cuda"))
+    c = proj.cells
+    ws = torch.zeros(64 + room, dtype=torch.float64, device="cuda")
+    mesh = torch.empty((pr.n, pr.n, pr.C), dtype=torch.float64, device="cuda")
+    api.pfem_project_p2m(pr.n, proj.nb, pr.N, c.pos_sorted, c.q_sorted, c.cell_start, c.perm, pr.C,
+                         torch.tensor(pr.vals, device="cuda"), P.PFEM_SHAPE_QUADRATIC, P.PFEM_SOLVE_F64,
+                         None, None, 0, mesh, ws)
+    code, detail = api.pfem_read_status(ws)
+    mesh, ref = mesh.cpu().numpy(), O.p2m(pr.n, pr.pos, pr.vals, shape=1, nthreads=8)
+    lost = ~np.isfinite(mesh).all(-1)
+    if room:
+        assert code == 0 and not lost.any(), (code, detail)
+    else:
+        assert lost.sum() <= 16 and (code == 5) == bool(lost.any())
+    assert np.abs(mesh - ref)[~lost].max() <= TOL64 * np.abs(ref).max()
