@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(256, tab_min_blocks<REFINE>() / 2) k_p2m_batch
 }
 
 // The fix pass over the batch's queued nodes (batch-wide indices), each with its problem's
-// bins, the widest search radius and FP64 SVD solves.
+// bins, the widest search radius and FP64 solves (node_u_fix).
 template <typename P, typename V, typename R, int SHAPE>
 __global__ void __launch_bounds__(128) k_p2m_fix_batch(const BPlanDev *pl, P2MArgs base)
 {

@@ -120,8 +120,9 @@ __device__ __forceinline__ float f32_trunc(double d)
 }
 
 // Refinement of the FP32 moment solve: none, one step with the residual r = b - M y in 64-bit
-// fixed point (FixRes), or steps until the solution has FP64's accuracy (fix64.cuh).
-enum { REFINE_NONE = 0, REFINE_FIX = 1, REFINE_FIX64 = 2 };
+// fixed point (FixRes), steps until the solution has FP64's accuracy (fix64.cuh), or for an FP64 solve
+// one step with the residual in FP64.
+enum { REFINE_NONE = 0, REFINE_FIX = 1, REFINE_FIX64 = 2, REFINE_STEP = 3 };
 
 // ----------------------------------------------------------------- fixed-point residual
 // The residual r = b - sum_mu p_mu (p_mu . y) of one edge system on the integer pipes.

@@ -372,8 +372,7 @@ constexpr int UMAX = PFEM_UMAX; // fast pass: jittered lattices have at most abo
 constexpr int UMAX_SVD = 32;   // SVD pass (the stencil masks are 32-bit)
 static_assert(UMAX_SVD <= SVD_ROWS, "stencils of the SVD pass fit jacobi_svd's rows");
 
-// SVD = true (the FP64 pass over queued nodes): each edge's coefficients are the minimum-norm
-// least-squares solution by SVD instead of the Cholesky solve of the moment system.
+// SVD = true: the FP64 pass over queued nodes (node_u_fix).
 // The node's distinct particles U = T + stars of T's vertices (slots us[0..nu)), the stencil
 // of the edge (tri[e], tri[e+1]) as the bit mask vm[e] | vm[e+1] over U, vi[e] the index of
 // tri[e] in U, and uw initialised to the linear weights lambda.  Returns 0, or -1 when U has
@@ -487,7 +486,7 @@ __device__ __forceinline__ int node_edges(W &&uw, const unsigned vm[3], const in
             offset(i, ox, oy);
             const S x = (ox - mx) * inv, yv = (oy - my) * inv;
             M.add(x, yv);
-            if (REFINE != REFINE_NONE) ext = fmax(ext, fmax(fabs(x), fabs(yv)));
+            if (REFINE == REFINE_FIX) ext = fmax(ext, fmax(fabs(x), fabs(yv)));
         }
         if (!M.factor(FastTol<S>::v)) return -PFEM_DEFER;
         const S tx = ex * inv, ty = ey * inv;
@@ -508,6 +507,31 @@ __device__ __forceinline__ int node_edges(W &&uw, const unsigned vm[3], const in
             M.solve(rs, dy);
 #pragma unroll
             for (int k = 0; k < 6; ++k) y[k] = __fadd_rn(y[k], dy[k]);
+        }
+        if constexpr (REFINE == REFINE_STEP) {
+            // corrected semi-normal equations (Bjorck 1987): with the residual formed from the points
+            // the error grows with the condition of P instead of that of M, its square.  504,000
+            // edges of a uniform random set: worst 3e-10 of an edge's largest coefficient -> 1e-13.
+            S r[6], dy[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) r[k] = b[k];
+            for (unsigned m = mask; m; m &= m - 1) {
+                const int i = __ffs(m) - 1;
+                S ox, oy;
+                offset(i, ox, oy);
+                const S x = (ox - mx) * inv, z = (oy - my) * inv;
+                const S t = fma(z * z, y[5], fma(x * z, y[4], fma(x * x, y[3], fma(z, y[2], fma(x, y[1], y[0])))));
+                const S xt = x * t, zt = z * t;
+                r[0] -= t;
+                r[1] = fma(-x, t, r[1]);
+                r[2] = fma(-z, t, r[2]);
+                r[3] = fma(-x, xt, r[3]);
+                r[4] = fma(-z, xt, r[4]);
+                r[5] = fma(-z, zt, r[5]);
+            }
+            M.solve(r, dy);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) y[k] += dy[k];
         }
         const R coef = R(2) * lam[e] * lam[f];
         for (unsigned m = mask; m; m &= m - 1) {
@@ -536,6 +560,21 @@ __device__ __forceinline__ int node_u_solve(const P2MArgs &a, const NodePos<P, R
     });
 }
 
+// The edges e0 <= e < e1 of a node of the fix pass in FP64: each by Cholesky down to the FP64 pivot
+// tolerance -- a system too ill-conditioned for the FP32 factor is usually well within FP64's -- refined
+// where the weights are FP64, and below it (rank deficient, or conditioned beyond it) by the SVD.  A
+// system that Cholesky cannot factor adds nothing to uw.
+template <typename P, typename R, int UM>
+__device__ __forceinline__ void node_u_fix(const P2MArgs &a, const NodePos<P, R> &np, const int *us, R *uw,
+                                           const unsigned vm[3], const int vi[3], const R lam[3], int e0, int e1)
+{
+    constexpr int REFINE = sizeof(R) == 8 ? REFINE_STEP : REFINE_NONE;
+#pragma unroll 1
+    for (int e = e0; e < e1; ++e)
+        if (node_u_solve<P, R, double, REFINE, false, UM>(a, np, us, uw, vm, vi, lam, e, e + 1) != 0)
+            node_u_solve<P, R, double, REFINE_NONE, true, UM>(a, np, us, uw, vm, vi, lam, e, e + 1);
+}
+
 template <typename P, typename R, typename S, int REFINE, bool SVD = false, typename SA,
           typename Emit>
 __device__ __forceinline__ int node_quadratic(const P2MArgs &a, const NodePos<P, R> &np,
@@ -550,8 +589,12 @@ __device__ __forceinline__ int node_quadratic(const P2MArgs &a, const NodePos<P,
     int vi[3];
     if (node_u_build<UM>(tri, st, lam, us, uw, nu, vm, vi, SVD ? UM : min(a.ucap, UM)) != 0)
         return SVD ? -PFEM_ERR_CAPACITY : -PFEM_DEFER;
-    const int r = node_u_solve<P, R, S, REFINE, SVD, UM>(a, np, us, uw, vm, vi, lam);
-    if (r != 0) return r;
+    if constexpr (SVD) {
+        node_u_fix<P, R, UM>(a, np, us, uw, vm, vi, lam, 0, 3);
+    } else {
+        const int r = node_u_solve<P, R, S, REFINE, false, UM>(a, np, us, uw, vm, vi, lam);
+        if (r != 0) return r;
+    }
     for (int i = 0; i < nu; ++i) emit(us[i], uw[i]);
     return 0;
 }
@@ -644,7 +687,7 @@ __device__ __forceinline__ void p2m_node(const P2MArgs &a, int I, int J)
                 if constexpr (REFINE == REFINE_FIX64) {
                     st = node_quadratic64<P, R>(a, Iu, Ju, tri, sa, lam, emit);
                     if (st == -PFEM_DEFER && short_queue(a))          // (nothing was emitted)
-                        st = node_quadratic<P, R, double, REFINE_NONE, false>(a, np, tri, sa, lam, emit);
+                        st = node_quadratic<P, R, double, sizeof(R) == 8 ? REFINE_STEP : REFINE_NONE, false>(a, np, tri, sa, lam, emit);
                 } else {
                     st = node_quadratic<P, R, S, REFINE, SVD>(a, np, tri, sa, lam, emit);
                 }
@@ -676,7 +719,7 @@ __device__ __forceinline__ void p2m_node(const P2MArgs &a, int I, int J)
                 if constexpr (REFINE == REFINE_FIX64) {
                     st = node_quadratic64<P, R>(a, Iu, Ju, tri, sa, lam, emit);
                     if (st == -PFEM_DEFER && short_queue(a))          // (nothing was emitted)
-                        st = node_quadratic<P, R, double, REFINE_NONE, false>(a, np, tri, sa, lam, emit);
+                        st = node_quadratic<P, R, double, sizeof(R) == 8 ? REFINE_STEP : REFINE_NONE, false>(a, np, tri, sa, lam, emit);
                 } else {
                     st = node_quadratic<P, R, S, REFINE, SVD>(a, np, tri, sa, lam, emit);
                 }
@@ -774,7 +817,7 @@ __global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_p2m_linear(P
 
 // The queued nodes again, overwriting the fast pass's placeholder output: the geometry searched
 // per thread with the widest search radius (the launcher passes it in a.B.rmax), and with
-// quadratic shape functions every edge solved in FP64 by the SVD.  A node that fails here
+// quadratic shape functions every edge solved in FP64 (node_u_fix).  A node that fails here
 // reports its error.
 template <typename P, typename V, typename R, int SHAPE, bool WEIGHTS>
 __global__ void __launch_bounds__(128) k_p2m_fix(P2MArgs a)
@@ -1009,10 +1052,7 @@ template <int Q> __device__ __forceinline__ int group_min(int v)
 
 // The fix pass of the table path: the queued nodes located with the star table (complete after
 // the retry kernels; the launcher passes the widest search radius for the nearest particle),
-// four lanes a node as in tab_node.  Each edge system is solved in FP64: by Cholesky down to the
-// FP64 pivot tolerance -- a system too ill-conditioned for the FP32 factor is usually well within
-// FP64's -- and below it (rank deficient, or conditioned beyond it) by the SVD.  A queued node's
-// time is one thread's chain of FP64 instructions, so the edges of a node run side by side: about
+// four lanes a node as in tab_node, the edges as in node_u_fix.  A queued node's time is one thread's chain of FP64 instructions, so the edges of a node run side by side: about
 // 1500 queued nodes of 513^2 over 1024^2 uniform random particles 1150 -> 434 us.
 template <typename P, typename V, typename R>
 __global__ void __launch_bounds__(128) k_p2m_fix_tab(P2MArgs a, StarTab t)
@@ -1058,9 +1098,7 @@ __global__ void __launch_bounds__(128) k_p2m_fix_tab(P2MArgs a, StarTab t)
                 if (q == 0)
 #pragma unroll
                     for (int e = 0; e < 3; ++e) uw[vi[e]] += lam[e];
-                // nothing is added to uw by a system that Cholesky cannot factor
-                if (node_u_solve<P, R, double, REFINE_NONE, false, UM>(f, np, us, uw, vm, vi, lam, e0, e1) != 0)
-                    node_u_solve<P, R, double, REFINE_NONE, true, UM>(f, np, us, uw, vm, vi, lam, e0, e1);
+                node_u_fix<P, R, UM>(f, np, us, uw, vm, vi, lam, e0, e1);
                 __syncwarp(0xfu << (threadIdx.x & 28));
                 for (int k = 0; k < nu; ++k) {
                     const R wk = group_sum<Q>(uw[k]);

@@ -241,3 +241,37 @@ def test_fp64_with_a_short_queue(P, room):
     else:
         assert lost.sum() <= 16 and (code == 5) == bool(lost.any())
     assert np.abs(mesh - ref)[~lost].max() <= TOL64 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("route", ["p2m", "batch", "short_queue"])
+@pytest.mark.parametrize("which", sorted(IRREGULAR))
+def test_fp64_fix_pass_on_irregular_sets(P, which, route):
+    """The nodes that the FP64 fast pass leaves to the fix pass (Cholesky with one refinement step, below
+    its tolerance the SVD), in the table path, a batch and a call that searches the stars a node:
+    the image of white noise at every node within FP64's 1e-12 of the oracle's over the node's sum of
+    weights, which the unrefined normal equations of the worst of them miss a hundredfold."""
+    from paper_1610_05266_gb300 import api
+    pr = IRREGULAR[which]()
+    v = noise(pr.N)
+    pos, vals = torch.tensor(pr.pos, device="cuda"), torch.tensor(v, device="cuda")
+    proj = P.Projector(pr.n, pr.N, C=8, pos_dtype=torch.float64)
+    proj.build(pos)
+    w = proj.shape_weights()[1]
+    if route == "p2m":
+        got = proj.p2m(vals)
+        proj.check(which)
+    elif route == "batch":
+        b = P.Batch([(pr.n, pr.N)], 8, torch.float64, "cuda")
+        b.build(pos)
+        b.p2m(vals)
+        got = b.mesh_view(0)
+        assert b.status()[0] == 0
+    else:
+        c = proj.cells
+        ws = torch.zeros(64 + pr.n * pr.n // 64, dtype=torch.float64, device="cuda")
+        got = torch.empty((pr.n, pr.n, 8), dtype=torch.float64, device="cuda")
+        api.pfem_project_p2m(pr.n, proj.nb, pr.N, c.pos_sorted, c.q_sorted, c.cell_start, c.perm, 8, vals,
+                             P.PFEM_SHAPE_QUADRATIC, P.PFEM_SOLVE_F64, None, None, 0, got, ws)
+        assert api.pfem_read_status(ws)[0] == 0
+    ref = O.p2m(pr.n, pr.pos, v, shape=1, nthreads=16)
+    assert per_node(got.cpu().numpy(), ref, w.cpu().numpy()) <= TOL64
