@@ -273,7 +273,7 @@ __device__ __forceinline__ int bwd_u_solve64(const BwdArgs &b, int Iu, int Ju, c
         EdgeSystem<UMAX> sys(o, vm[e] | vm[f], o[vi[e]], o[vi[f]]);
         long long Y[6], Z[6], u[6] = {0, 0, 0, 0, 0, 0};
         int sy, sz = 0;
-        if (!sys.factor() || !sys.solve_coefficients(Y, sy)) return -PFEM_DEFER;
+        if (!sys.factor(FastTol<float>::v) || !sys.solve_coefficients(Y, sy)) return -PFEM_DEFER;
         const double yu = __hiloint2double((1023 - sy) << 20, 0), ce = 2.0 * lam[e] * lam[f];
         EdgeFix64 Ey, Ez;
         Ey.set(Y);
