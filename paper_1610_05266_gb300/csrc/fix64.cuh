@@ -329,6 +329,8 @@ __device__ __forceinline__ int node_solve64(const longlong2 (&o)[UM], const unsi
         EdgeFix64 E;
         E.set(Y);
         const double coef = 2.0 * lam[e] * lam[f];
+        // a node outside its triangle by the rounding of a sliver: beyond the product's range below
+        if (((__double2hiint(coef) >> 20) & 0x7ff) > 1023) return defer;
         const Split64 cf = split64(__double2ll_rn(coef * 2305843009213693952.0));   // 2^61
         const int sh = W64_SHIFT + 3 - s;                        // product: coef A 2^(s - 3)
         int tm = 0;

@@ -275,3 +275,53 @@ def test_fp64_fix_pass_on_irregular_sets(P, which, route):
         assert api.pfem_read_status(ws)[0] == 0
     ref = O.p2m(pr.n, pr.pos, v, shape=1, nthreads=16)
     assert per_node(got.cpu().numpy(), ref, w.cpu().numpy()) <= TOL64
+
+
+def triangle_weights(pos, node, tri, stars):
+    """Weights of a node in the triangle tri of particles with the given stars, by the pseudo-inverse."""
+    d = pos - node
+
+    def cr(a, b):
+        return d[a][0] * d[b][1] - d[a][1] * d[b][0]
+
+    lam = np.array([cr(tri[1], tri[2]), cr(tri[2], tri[0]), cr(tri[0], tri[1])])
+    lam /= lam.sum()
+    w = dict(zip(tri, lam))
+    for e in range(3):
+        f = (e + 1) % 3
+        ids = sorted({tri[e], tri[f], *stars[e], *stars[f]})
+        m, t = (d[tri[e]] + d[tri[f]]) / 2, d[tri[e]] - d[tri[f]]
+        z, t = (d[ids] - m) / np.hypot(*t), t / np.hypot(*t)
+        p = np.stack([np.ones(len(ids)), z[:, 0], z[:, 1], z[:, 0] ** 2, z[:, 0] * z[:, 1], z[:, 1] ** 2])
+        A = np.linalg.pinv(p) @ np.array([0, 0, 0, -t[0] ** 2 / 2, -t[0] * t[1] / 2, -t[1] ** 2 / 2])
+        for k, a in zip(ids, A):
+            w[k] = w.get(k, 0.0) + 2 * lam[e] * lam[f] * a
+    return w, lam
+
+
+@pytest.mark.parametrize("seed", [26, 415, 1852])
+def test_fp64_node_outside_a_sliver(P, seed):
+    """A node among particles 1.6 units of 2^-32 apart: in the triangulation of the rounded positions it
+    lies in a triangle that it is outside of, with coefficients 2 lambda lambda' of 4 to 16.  FP64 weights
+    (of the triangle that was chosen) and P2M within 1e-12 of the largest."""
+    n, I = 33, 8
+    node = np.array([I, I]) / (n - 1)
+    base = G.jittered_lattice(64, 0.2, G.SEED_BASE + 980)
+    far = base[((base - node) ** 2).sum(1) > (1.2 / 64) ** 2]
+    r = G.uniform01(G.SEED_BASE + 100000 + seed, 98).reshape(49, 2)
+    g = np.stack(np.meshgrid(np.arange(7) - 3, np.arange(7) - 3), -1).reshape(49, 2)
+    pos = np.concatenate([far, node + (1.6 * g + 0.7 * (2 * r - 1)) * 2.0 ** -32])
+    proj = P.Projector(n, len(pos), C=1, pos_dtype=torch.float64)
+    proj.build(torch.tensor(pos, device="cuda"))
+    perm = proj.cells.perm.cpu().numpy()
+    s, w = (x[I * n + I].cpu().numpy() for x in proj.shape_weights())
+    got = dict(zip((int(k) for k in perm[s[s >= 0]]), w))
+    tri = list(got)[:3]
+    cells = O.build_cells(n, pos)
+    ref, lam = triangle_weights(pos, node, tri, [[int(k) for k in O.star(cells, t)] for t in tri])
+    assert max(abs(2 * lam[e] * lam[e - 1]) for e in range(3)) > 2 and set(got) == set(ref)
+    top = max(abs(x) for x in ref.values())
+    for k, x in ref.items():
+        v = torch.zeros(len(pos), 1, dtype=torch.float64, device="cuda")
+        v[k] = 1.0
+        assert abs(got[k] - x) <= TOL64 * top and abs(proj.p2m(v)[I, I, 0].item() - x) <= TOL64 * top, (k, lam)
