@@ -309,16 +309,26 @@ template <int UM> struct EdgeSystem {
 // nodes beyond that take FP64's Cholesky form (k_bwd_fix).
 constexpr float TOL_FIX64 = 3e-5f;
 
-// Weights of the quadratic part in fixed point: w[i] += 2 lambda_nu lambda_sg A_{i e} 2^56 over the
-// edges e0 <= e < e1.  Returns 0, or -PFEM_DEFER for a system below the tolerance, whose refinement
-// stalls, or beyond the fixed-point range.
-constexpr int W64_SHIFT = 56;            // weights up to 2^7
+// Weights of the quadratic part in fixed point: w[i] += 2 lambda_nu lambda_sg A_{i e} / unit over the
+// edges e0 <= e < e1.  The unit is 2^-56 of the node's largest coefficient 2 lambda lambda' or less: a
+// node close to a particle, or to an edge, has small ones, and its weights keep FP64's relative
+// accuracy.  Returns 0, or -PFEM_DEFER for a system below the tolerance, whose refinement stalls, or
+// beyond the fixed-point range, a coefficient of 2 or more (a node outside its triangle by the rounding
+// of a sliver) among them.
+constexpr int W64_SHIFT = 56;            // weights up to 2^7 of the largest coefficient
 constexpr double W64_UNIT = 1.3877787807814457e-17;
 template <int UM>
 __device__ __forceinline__ int node_solve64(const longlong2 (&o)[UM], const unsigned vm[3],
                                             const int vi[3], const double lam[3], int e0, int e1,
-                                            long long *w, int defer)
+                                            long long *w, double &unit, int defer)
 {
+    const double coef[3] = {2.0 * lam[0] * lam[1], 2.0 * lam[1] * lam[2], 2.0 * lam[2] * lam[0]};
+    // 2^up: the largest of |coef| lies in [1/2, 1) 2^-up (zero: any)
+    const int up = min(1022 - max(max((__double2hiint(coef[0]) >> 20) & 0x7ff, (__double2hiint(coef[1]) >> 20) & 0x7ff),
+                                  (__double2hiint(coef[2]) >> 20) & 0x7ff), 100);
+    if (up < -1) return defer;
+    unit = __hiloint2double((1023 - W64_SHIFT - up) << 20, 0);
+    const double to61 = __hiloint2double((1023 + 61 + up) << 20, 0);
 #pragma unroll 1
     for (int e = e0; e < e1; ++e) {
         const int f = e == 2 ? 0 : e + 1;
@@ -328,10 +338,7 @@ __device__ __forceinline__ int node_solve64(const longlong2 (&o)[UM], const unsi
         if (!sys.factor(TOL_FIX64) || !sys.solve_coefficients(Y, s)) return defer;
         EdgeFix64 E;
         E.set(Y);
-        const double coef = 2.0 * lam[e] * lam[f];
-        // a node outside its triangle by the rounding of a sliver: beyond the product's range below
-        if (((__double2hiint(coef) >> 20) & 0x7ff) > 1023) return defer;
-        const Split64 cf = split64(__double2ll_rn(coef * 2305843009213693952.0));   // 2^61
+        const Split64 cf = split64(__double2ll_rn((e == 0 ? coef[0] : e == 1 ? coef[1] : coef[2]) * to61));
         const int sh = W64_SHIFT + 3 - s;                        // product: coef A 2^(s - 3)
         int tm = 0;
         for (unsigned m = sys.mask; m; m &= m - 1) {
@@ -344,8 +351,9 @@ __device__ __forceinline__ int node_solve64(const longlong2 (&o)[UM], const unsi
             const long long ct = mul64(split64(t), cf);
             w[i] += sh >= 0 ? ct << sh : ct >> -sh;
         }
-        // |A| <= (tm + 1) 2^(32 - s): keep the weights well inside their range
-        if (((float)tm + 1.f) * EdgeSystem<UM>::pow2(32 - s) * fabsf((float)coef) > 30.f) return defer;
+        // |A| <= (tm + 1) 2^(32 - s), the coefficient 2^-29 of cf.h + 1: keep the weights well inside their
+        // range
+        if (((float)tm + 1.f) * EdgeSystem<UM>::pow2(32 - s) * (fabsf((float)cf.h) + 1.f) > 30.f * 536870912.f) return defer;
     }
     return 0;
 }

@@ -615,9 +615,10 @@ __device__ __forceinline__ int node_quadratic64(const P2MArgs &a, int Iu, int Ju
     if (node_offsets64<P>(a.pos, Iu, Ju, a.n - 1, us, nu, o) == NOT_FINITE) return -PFEM_DEFER;
     for (int i = 0; i < nu; ++i) w[i] = 0;
     const double l64[3] = {(double)lam[0], (double)lam[1], (double)lam[2]};
-    const int r = node_solve64(o, vm, vi, l64, 0, 3, w, -PFEM_DEFER);
+    double unit;
+    const int r = node_solve64(o, vm, vi, l64, 0, 3, w, unit, -PFEM_DEFER);
     if (r != 0) return r;
-    for (int i = 0; i < nu; ++i) emit(us[i], (R)(__ll2double_rn(w[i]) * W64_UNIT));
+    for (int i = 0; i < nu; ++i) emit(us[i], (R)(__ll2double_rn(w[i]) * unit));
 #pragma unroll
     for (int e = 0; e < 3; ++e) emit(tri[e], lam[e]);
     return 0;
@@ -1158,9 +1159,10 @@ __device__ __forceinline__ int set_solve(const P2MArgs &a, const NodePos<P, R> &
         const bool finite = node_offsets64<P>(a.pos, Iu, Ju, a.n - 1, us, nu, o) != NOT_FINITE;
         for (int i = 0; i < nu; ++i) w[i] = 0;
         const double l64[3] = {(double)lam[0], (double)lam[1], (double)lam[2]};
-        st = group_min<Q>(finite ? node_solve64(o, vm, vi, l64, e0, e1, w, -PFEM_DEFER) : -PFEM_DEFER);
+        double unit = 0.0;
+        st = group_min<Q>(finite ? node_solve64(o, vm, vi, l64, e0, e1, w, unit, -PFEM_DEFER) : -PFEM_DEFER);
         if (st == 0) {
-            for (int i = 0; i < nu; ++i) apply(us[i], (R)(__ll2double_rn(group_sum<Q>(w[i])) * W64_UNIT));
+            for (int i = 0; i < nu; ++i) apply(us[i], (R)(__ll2double_rn(group_sum<Q>(w[i])) * unit));
 #pragma unroll
             for (int e = 0; e < 3; ++e) apply(tri[e], lam[e]);
         }
@@ -1327,8 +1329,9 @@ __global__ void __launch_bounds__(128, tab_min_blocks<REFINE>()) k_shape_tab(P2M
             const bool finite = node_offsets64<P>(a.pos, Iu, Ju, nc, us, nu, o) != NOT_FINITE;
             for (int i = 0; i < nu; ++i) w[i] = 0;
             const double l64[3] = {(double)lam[0], (double)lam[1], (double)lam[2]};
-            st = finite ? node_solve64(o, vm, vi, l64, 0, 3, w, -PFEM_DEFER) : -PFEM_DEFER;
-            for (int i = 0; i < nu; ++i) uw[i] = (R)(__ll2double_rn(w[i]) * W64_UNIT);
+            double unit = 0.0;
+            st = finite ? node_solve64(o, vm, vi, l64, 0, 3, w, unit, -PFEM_DEFER) : -PFEM_DEFER;
+            for (int i = 0; i < nu; ++i) uw[i] = (R)(__ll2double_rn(w[i]) * unit);
 #pragma unroll
             for (int e = 0; e < 3; ++e) uw[vi[e]] += lam[e];
         } else {

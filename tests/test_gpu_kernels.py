@@ -325,3 +325,31 @@ def test_fp64_node_outside_a_sliver(P, seed):
         v = torch.zeros(len(pos), 1, dtype=torch.float64, device="cuda")
         v[k] = 1.0
         assert abs(got[k] - x) <= TOL64 * top and abs(proj.p2m(v)[I, I, 0].item() - x) <= TOL64 * top, (k, lam)
+
+
+@pytest.mark.parametrize("d", [1e-4, 1e-9])
+def test_fp64_weights_of_a_node_close_to_a_particle(P, d):
+    """A node at distance d of a particle on 33^2 nodes: the other particles' weights, of the order of 32 d,
+    within 1e-12 of the largest of them, by the table path's weights and P2M (four lanes a node), as FP64
+    products give them (offsets from the node are exact here)."""
+    n, (I, J) = 33, (16, 20)
+    pos = G.jittered_lattice(64, 0.2, G.SEED_BASE + 990)
+    node = np.array([I, J]) / 32
+    close = int(((pos - node) ** 2).sum(1).argmin())
+    pos[close] = node + d * np.array([1.0, 0.7])
+    idx, ref = O.node_weights(O.build_cells(n, pos), I, J, 1)[:2]
+    proj = P.Projector(n, len(pos), C=1, pos_dtype=torch.float64)
+    proj.build(torch.tensor(pos, device="cuda"))
+    perm = proj.cells.perm.cpu().numpy()
+    s, w = (x[J * n + I].cpu().numpy() for x in proj.shape_weights())
+    proj.check("weights")
+    got = dict(zip((int(k) for k in perm[s[s >= 0]]), w))
+    assert set(got) == {int(k) for k in idx}
+    top = max(abs(x) for k, x in zip(idx, ref) if k != close)
+    assert top < 100 * d
+    for k, x in zip(idx, ref):
+        v = torch.zeros(len(pos), 1, dtype=torch.float64, device="cuda")
+        v[int(k)] = 1.0
+        tol = TOL64 * (1.0 if k == close else top)
+        assert abs(got[int(k)] - x) <= tol and abs(proj.p2m(v)[J, I, 0].item() - x) <= tol, int(k)
+    proj.check("p2m")
