@@ -29,7 +29,7 @@
 
 namespace pfem {
 
-// x mod 1 in Q64 (rounded to nearest below 2^-11, exact above), by integer operations.
+// x mod 1 in Q64 (rounded to nearest below 2^-12, exact above), by integer operations.
 __device__ __forceinline__ long long fx64(double x)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);

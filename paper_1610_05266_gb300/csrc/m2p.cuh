@@ -26,8 +26,11 @@ template <typename R> __device__ __forceinline__ R local_coord(R x, int i, int n
 }
 
 // FP64 positions in fixed point (fix64.cuh: their arithmetic would hold the FP64 pipe): the cell, and the
-// local coordinate in units of 2^-62.  The cell comes from the coordinate rounded to 2^-32, so the
-// local coordinate may lie a rounding outside [0, 1].
+// local coordinate in units of 2^-62 (absolute, where FP64 rounds it to 2^-53 of itself: a weight near
+// zero is a multiple of 2^-62).  The cell comes from the coordinate rounded to 2^-32, so the
+// local coordinate may lie a rounding outside [0, 1].  Below 2^-12 a position has bits beyond 2^-64, whose
+// rounding nc enlarges: with more than 2048 cells a side, where that passes FP64's own rounding, those
+// positions, 2^-12 of all, take the FP64 product.
 __device__ __forceinline__ long long local_fix(double x, int nc, int &i)
 {
     const unsigned long long q = (unsigned long long)fx64(x);
@@ -35,6 +38,8 @@ __device__ __forceinline__ long long local_fix(double x, int nc, int &i)
     unsigned t = (unsigned)(q >> 32);
     t += f > 0x80000000u || (f == 0x80000000u && (t & 1u)) ? 1u : 0u;
     i = bin_of(t, nc);
+    if (nc > 2048 && (unsigned)__double2hiint(x) < 1011u << 20)
+        return __double2ll_rn(fma(x, (double)nc, (double)-i) * 4611686018427387904.0);
     int d = (int)__umul64hi(q, (unsigned long long)nc) - i;
     d -= d > 1 ? nc : 0;
     d += d < -1 ? nc : 0;

@@ -353,3 +353,18 @@ def test_fp64_weights_of_a_node_close_to_a_particle(P, d):
         tol = TOL64 * (1.0 if k == close else top)
         assert abs(got[int(k)] - x) <= tol and abs(proj.p2m(v)[J, I, 0].item() - x) <= tol, int(k)
     proj.check("p2m")
+
+
+def test_fp64_m2p_near_the_origin_of_a_fine_mesh(P):
+    """FP64 particles in the first cell of 16385^2 nodes, where positions have bits below 2^-64: a linear field
+    over that cell within 2^-52, three roundings of FP64 weights (the cell's side is a power of two, so the
+    field's value is exact)."""
+    n = 16385
+    u = G.uniform01(G.SEED_BASE + 995, 2 * 4096).reshape(4096, 2)
+    pos = u / (n - 1)
+    mesh = torch.zeros(n, n, 1, dtype=torch.float64, device="cuda")
+    mesh[:, 1:3] = 1.0
+    got = torch.empty(len(pos), 1, dtype=torch.float64, device="cuda")
+    from paper_1610_05266_gb300 import api
+    api.pfem_interp_m2p(n, len(pos), torch.tensor(pos, device="cuda"), 1, mesh, got)
+    assert np.abs(got[:, 0].cpu().numpy() - pos[:, 0] * (n - 1)).max() <= 2.0 ** -52
