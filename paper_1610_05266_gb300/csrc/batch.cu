@@ -461,7 +461,10 @@ static cudaError_t p2m_batch_t(const void *plan, const P2MArgs &base, int shape_
         const int threads = 16 * TYs[shape_idx];
         if constexpr (SHAPE == PFEM_SHAPE_LINEAR) {
             const size_t lists = (size_t)((threads + STAR_TPB - 1) / STAR_TPB) * HullList::BYTES;
-            e = cudaFuncSetAttribute(k_p2m_batch_linear<P, V, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lists);
+            // the limit is the process's, not the launch's: always that of the largest block, or a call in
+            // another thread with smaller ones could lower it before this launch
+            constexpr int MOST = (256 + STAR_TPB - 1) / STAR_TPB * HullList::BYTES;
+            e = cudaFuncSetAttribute(k_p2m_batch_linear<P, V, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, MOST);
             if (e != cudaSuccess) return e;
             k_p2m_batch_linear<P, V, R><<<blocks, threads, lists, s>>>(pl, shape_idx, base, counter);
         } else {

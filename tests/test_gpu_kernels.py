@@ -368,3 +368,37 @@ def test_fp64_m2p_near_the_origin_of_a_fine_mesh(P):
     from paper_1610_05266_gb300 import api
     api.pfem_interp_m2p(n, len(pos), torch.tensor(pos, device="cuda"), 1, mesh, got)
     assert np.abs(got[:, 0].cpu().numpy() - pos[:, 0] * (n - 1)).max() <= 2.0 ** -52
+
+
+def test_linear_batches_of_two_block_shapes_in_two_threads(P):
+    """Linear batched P2M with 64- and 256-thread blocks from two threads at once, each on its own stream: no
+    launch is refused over shared memory that the other's shape does not need, and the meshes agree."""
+    import threading
+    pr = PROBLEMS["tiny"]()
+    pos, vals = torch.tensor(pr.pos, device="cuda"), torch.tensor(pr.vals, device="cuda")
+    got = {}
+
+    def work(tile_rows):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                b = P.Batch([(pr.n, pr.N)] * 2, pr.C, torch.float64, "cuda")
+                b.build(pos.repeat(2, 1))
+                v = vals.repeat(2, 1)
+                for _ in range(2000):
+                    b.p2m(v, shape=P.PFEM_SHAPE_LINEAR, tile_rows=tile_rows)
+                torch.cuda.current_stream().synchronize()
+                assert b.status()[0] == 0
+                got[tile_rows] = b.mesh.clone()
+        except Exception as e:                   # reported by the main thread
+            got[tile_rows] = e
+
+    torch.cuda.synchronize()
+    ts = [threading.Thread(target=work, args=(t,)) for t in (4, 16)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    torch.cuda.synchronize()
+    for x in got.values():
+        assert torch.is_tensor(x), x
+    assert torch.equal(got[4], got[16])
