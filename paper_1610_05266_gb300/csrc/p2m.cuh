@@ -933,8 +933,30 @@ __device__ __forceinline__ int node_sets8(const StarTab &t, const int tri[3], co
     return nu;
 }
 
+// The lanes of a node (a group of Q consecutive ones that run the same control flow), and the sum
+// and the least of their values.
+template <int Q> __device__ __forceinline__ unsigned group_mask()
+{
+    return ((1u << Q) - 1u) << (threadIdx.x & 31 & ~(Q - 1));
+}
+template <int Q, typename T> __device__ __forceinline__ T group_sum(T v)
+{
+#pragma unroll
+    for (int o = 1; o < Q; o <<= 1) v += __shfl_xor_sync(group_mask<Q>(), v, o);
+    return v;
+}
+template <int Q> __device__ __forceinline__ int group_min(int v)
+{
+#pragma unroll
+    for (int o = 1; o < Q; o <<= 1) v = min(v, __shfl_xor_sync(group_mask<Q>(), v, o));
+    return v;
+}
+
 // node_sets8 where it applies: true when the sets of all nodes of the warp fit (one path a warp: a
-// few nodes with larger sets would otherwise cost it both).  st != 0: no node here.
+// few nodes with larger sets would otherwise cost it both).  st != 0: no node here.  The lanes that vote
+// are those that happen to arrive together, which need not be the whole warp; the Q lanes of a node,
+// which exchange values on the path that is chosen, agree on the answer over their own mask.
+template <int Q>
 __device__ __forceinline__ bool warp_sets8(const StarTab &t, int st, const int tri[3], const TabStar sa[3],
                                            int cap, int *su, int stride, int &nu, unsigned vm[3])
 {
@@ -947,7 +969,7 @@ __device__ __forceinline__ bool warp_sets8(const StarTab &t, int st, const int t
             fits = nu <= min(cap, SET_MAX);
         }
     }
-    return __all_sync(__activemask(), fits);
+    return group_min<Q>(__all_sync(__activemask(), fits) ? 1 : 0) != 0;
 }
 
 // Resident 128-thread blocks per SM of the geometry kernel: its node search waits on memory, and
@@ -978,7 +1000,7 @@ __device__ __forceinline__ void geom_node(const P2MArgs &a, const StarTab &t, co
         }
     int meta = -1, nu = 0;
     unsigned vm[3] = {0u, 0u, 0u};
-    const bool small = warp_sets8(t, st, tri, sa, a.ucap, su, stride, nu, vm);
+    const bool small = warp_sets8<1>(t, st, tri, sa, a.ucap, su, stride, nu, vm);
     if (st == 0) {
         NodePos<P, R> np;
         np.init(Iu, Ju, nc);
@@ -1030,25 +1052,6 @@ __global__ void __launch_bounds__(128, PFEM_GEOM_MIN_BLOCKS) k_p2m_geom(P2MArgs 
     const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
     if (I >= a.n || J >= a.n) return;
     geom_node<P, V, R>(a, t, r, I, J, (long long)J * a.n + I, su + threadIdx.x, 128);
-}
-
-// The lanes of a node (a group of Q consecutive ones that run the same control flow), and the sum
-// and the least of their values.
-template <int Q> __device__ __forceinline__ unsigned group_mask()
-{
-    return ((1u << Q) - 1u) << (threadIdx.x & 31 & ~(Q - 1));
-}
-template <int Q, typename T> __device__ __forceinline__ T group_sum(T v)
-{
-#pragma unroll
-    for (int o = 1; o < Q; o <<= 1) v += __shfl_xor_sync(group_mask<Q>(), v, o);
-    return v;
-}
-template <int Q> __device__ __forceinline__ int group_min(int v)
-{
-#pragma unroll
-    for (int o = 1; o < Q; o <<= 1) v = min(v, __shfl_xor_sync(group_mask<Q>(), v, o));
-    return v;
 }
 
 // The fix pass of the table path: the queued nodes located with the star table (complete after
@@ -1238,7 +1241,7 @@ __device__ __forceinline__ void tab_node(const P2MArgs &a, const StarTab &t, int
     };
     int nu = 0;
     unsigned vm[3] = {0u, 0u, 0u};
-    const bool small = warp_sets8(t, st, tri, sa, a.ucap, su, stride, nu, vm);
+    const bool small = warp_sets8<Q>(t, st, tri, sa, a.ucap, su, stride, nu, vm);
     if (st == 0) {
         NodePos<P, R> np;
         np.init(Iu, Ju, nc);

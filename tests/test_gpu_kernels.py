@@ -402,3 +402,22 @@ def test_linear_batches_of_two_block_shapes_in_two_threads(P):
     for x in got.values():
         assert torch.is_tensor(x), x
     assert torch.equal(got[4], got[16])
+
+
+@pytest.mark.parametrize("solve", ["F32", "F32_REFINED"])
+def test_four_lanes_a_node_over_sets_of_both_sizes(P, solve):
+    """Small meshes (four lanes a node) over uniform random particles, whose warps hold nodes with sets that fit
+    shared memory next to larger ones: bit for bit what one lane a node gives that searches the stars
+    itself, at the nodes which that solves without the fix pass (all but a few)."""
+    from paper_1610_05266_gb300 import api
+    pr, sv = uniform(97, 192, 996), getattr(P, "PFEM_SOLVE_" + solve)
+    proj = P.Projector(pr.n, pr.N, C=pr.C, pos_dtype=torch.float32)
+    proj.build(torch.tensor(pr.pos, dtype=torch.float32, device="cuda"))
+    v = torch.tensor(pr.vals, dtype=torch.float32, device="cuda")
+    four = proj.p2m(v, solve=sv)
+    proj.check("table")
+    c, one = proj.cells, torch.empty_like(four)
+    api.pfem_project_p2m(pr.n, proj.nb, pr.N, c.pos_sorted, c.q_sorted, c.cell_start, c.perm, pr.C, v,
+                         P.PFEM_SHAPE_QUADRATIC, sv, None, None, 0, one, torch.zeros(64, dtype=torch.float64, device="cuda"))
+    done = torch.isfinite(one).all(-1)
+    assert done.float().mean() > 0.97 and torch.equal(four[done], one[done])
