@@ -143,12 +143,11 @@ __global__ void __launch_bounds__(256) k_bin_batch(const BPlanDev *pl, const P *
 
 // ---------------------------------------------------------------- P2M
 
-// The plan and the caller's totals must agree before any table entry is written (nodes < 0: not
-// compared).
+// The plan and the caller's totals must agree before any table entry is written.
 __device__ __forceinline__ bool totals_ok(const BPlanDev *pl, long long nodes, const StarTab &t,
                                           DevStatus *st)
 {
-    const bool ok = (nodes < 0 || nodes == pl->total_nodes) && t.N == pl->total_particles;
+    const bool ok = nodes == pl->total_nodes && t.N == pl->total_particles;
     if (!ok && blockIdx.x == 0 && threadIdx.x == 0) record_error(st, PFEM_ERR_INVALID_ARG, -1);
     return ok;
 }
@@ -216,11 +215,12 @@ __global__ void __launch_bounds__(256) k_p2m_batch_linear(const BPlanDev *pl, in
 
 // Star table of every problem: block b takes 128 consecutive particles of one problem.
 __global__ void __launch_bounds__(BSTAR, PFEM_STAR_MIN_BLOCKS) k_star_list_batch(const BPlanDev *pl,
-                                                                                 P2MArgs base, StarTab t)
+                                                                                 P2MArgs base, StarTab t,
+                                                                                 long long nodes)
 {
     static_assert(BSTAR == STAR_TPB, "HullList's columns");
     __shared__ __align__(16) unsigned char lists[HullList::BYTES];
-    if (!totals_ok(pl, -1, t, base.status)) return;
+    if (!totals_ok(pl, nodes, t, base.status)) return;
     const long long *sp = plan_star_tiles(pl);
     for (long long b = blockIdx.x; b < pl->n_star_tiles; b += gridDim.x) {
         const int p = find_item(sp, pl->P, b);
@@ -434,7 +434,7 @@ size_t batch_p2m_ws_bytes(long long nodes_total, long long N_total)
 
 struct BatchWs {
     StarTab tab;
-    long long nodes;            // the total that the fast pass compares with the plan's, or -1
+    long long nodes;            // the caller's total, compared with the plan's
     bool table;
 };
 
@@ -450,7 +450,7 @@ static cudaError_t p2m_batch_t(const void *plan, const P2MArgs &base, int shape_
     if (SHAPE == PFEM_SHAPE_QUADRATIC && w.table) {
         // a block per tile of 128 particles (the problems' ragged last tiles are taken by the
         // blocks that are done first)
-        k_star_list_batch<<<(unsigned)((w.tab.N + BSTAR - 1) / BSTAR), BSTAR, 0, s>>>(pl, base, w.tab);
+        k_star_list_batch<<<(unsigned)((w.tab.N + BSTAR - 1) / BSTAR), BSTAR, 0, s>>>(pl, base, w.tab, w.nodes);
         k_star_retry_batch<<<num_sms() * RETRY_BLOCKS, RETRY_TPB, 0, s>>>(pl, base, w.tab);
         constexpr int TREF = sizeof(S) == 8 ? REFINE_FIX64 : REF;    // as for one problem
         const size_t su = (size_t)16 * TYs[shape_idx] * tab_rows<TREF>() * sizeof(int);
@@ -530,7 +530,7 @@ cudaError_t launch_batch_p2m(const void *plan, const void *pos_sorted, const uin
         const size_t rb = al256b(node_recs_layout(nullptr, nodes_total, &r, true));
         w.tab = star_tab_layout(base + rb, N_total, (int *)(W + 132));
     }
-    w.nodes = solve == PFEM_SOLVE_F32_REFINED_FF ? nodes_total : -1;
+    w.nodes = nodes_total;
     unsigned long long *counter = (unsigned long long *)(W + 64);
     const bool q = shape == PFEM_SHAPE_QUADRATIC;
     if (val_t == PFEM_F64) {

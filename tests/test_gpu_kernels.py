@@ -421,3 +421,18 @@ def test_four_lanes_a_node_over_sets_of_both_sizes(P, solve):
                          P.PFEM_SHAPE_QUADRATIC, sv, None, None, 0, one, torch.zeros(64, dtype=torch.float64, device="cuda"))
     done = torch.isfinite(one).all(-1)
     assert done.float().mean() > 0.97 and torch.equal(four[done], one[done])
+
+
+@pytest.mark.parametrize("solve", ["F64", "F32", "F32_REFINED", "F32_REFINED_FF"])
+def test_batch_totals_are_compared_for_every_solve(P, solve):
+    """A node total other than the plan's: PFEM_ERR_INVALID_ARG with detail -1, the mesh untouched."""
+    from paper_1610_05266_gb300 import api
+    pr = PROBLEMS["tiny"]()
+    pos, vals = (torch.tensor(x, dtype=torch.float32, device="cuda") for x in (pr.pos, pr.vals))
+    b = P.Batch([(pr.n, pr.N)] * 2, pr.C, torch.float32, "cuda")
+    b.build(pos.repeat(2, 1))
+    b.mesh.fill_(7.0)
+    api.pfem_batch_project_p2m(b.plan, b.nodes_total - 1, b.N_total, b.pos_sorted, b.q_sorted, b.cell_start, b.perm, pr.C,
+                               vals.repeat(2, 1), P.PFEM_SHAPE_QUADRATIC, getattr(P, "PFEM_SOLVE_" + solve), b.mesh, 8,
+                               64, b.ws)
+    assert b.status() == (1, -1) and bool((b.mesh == 7.0).all())
