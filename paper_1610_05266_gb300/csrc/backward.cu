@@ -393,6 +393,100 @@ __global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_bwd_linear(B
     write_entries<R, R, POS>(b, node, nu, us, uw, udx, udy);
 }
 
+// ---------------------------------------------------------------- node records
+// The adjoint runs the table path as two kernels, each with its own register budget: k_p2m_geom
+// locates the node and builds its particle set from the star table (memory latency bound), and
+// the adjoint's solve kernel reads what it found from a per-node record, one array per field so
+// that both kernels access it coalesced.  The forward solves run both halves in k_p2m_tab.
+struct NodeRecs {
+    int *meta;          // [nodes] nu | vi0 << 5 | vi1 << 10 | vi2 << 15, or -1: no record
+    unsigned *mask;     // [3][nodes] vm[e]
+    int *us;            // [UMAX][nodes] slots of the particle set
+    long long nodes;
+};
+
+// Lays the record arrays for `nodes` nodes out from `base` (256-byte aligned arrays; base may be
+// null to size them); returns the bytes they take.
+inline size_t node_recs_layout(char *base, long long nodes, NodeRecs *r)
+{
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t o_meta = 0;
+    const size_t o_mask = al(o_meta + sizeof(int) * (size_t)nodes);
+    const size_t o_us = al(o_mask + 3 * sizeof(unsigned) * (size_t)nodes);
+    const size_t total = al(o_us + UMAX * sizeof(int) * (size_t)nodes);
+    if (base) {
+        r->meta = (int *)(base + o_meta);
+        r->mask = (unsigned *)(base + o_mask);
+        r->us = (int *)(base + o_us);
+    }
+    r->nodes = nodes;
+    return total;
+}
+
+// Resident 128-thread blocks per SM of the geometry kernel: its node search waits on memory, and
+// its particle sets in shared memory and registers want room (the whole gradient step at 1025^2
+// nodes / 2048^2 particles, C = 1, FP32, with 6, 8, 10, 12 blocks: 2395, 2369, 2372, 2391 us).
+#ifndef PFEM_GEOM_MIN_BLOCKS
+#define PFEM_GEOM_MIN_BLOCKS 8
+#endif
+// Node (I, J) of the mesh of a.n nodes per side: locate it and build its particle set from the
+// star table, and write its record at index J * a.n + I.
+__device__ __forceinline__ void geom_node(const P2MArgs &a, const StarTab &t, const NodeRecs &r, int I, int J,
+                                          int *su, int stride)
+{
+    const int nc = a.n - 1;
+    const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
+    const long long rec = (long long)J * a.n + I;
+    const uint2 qn = make_uint2(node_fx(Iu, nc), node_fx(Ju, nc));
+    int tri[3];
+    int st = locate_tab(a.B, t, qn, a.R0, tri);
+    TabStar sa[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+        if (st == 0) {
+            sa[e] = tab_star(t, tri[e]);
+            if (sa[e].n < 0) st = sa[e].n == -1 ? -PFEM_FAR : sa[e].n;
+        }
+    int meta = -1, nu = 0;
+    unsigned vm[3] = {0u, 0u, 0u};
+    const bool small = warp_sets8<1>(t, st, tri, sa, a.ucap, su, stride, nu, vm);
+    if (st == 0) {
+        int vi[3] = {0, 1, 2};
+        auto write = [&](auto us) {
+            // entries up to the warp's largest set, -1 past this node's, so that the warp's
+            // stores to each entry array cover contiguous runs of it
+            const int nw = __reduce_max_sync(__activemask(), nu);
+            for (int i = 0; i < nw; ++i) r.us[i * r.nodes + rec] = i < nu ? us[i] : -1;
+#pragma unroll
+            for (int e = 0; e < 3; ++e) r.mask[e * r.nodes + rec] = vm[e];
+            meta = nu | vi[0] << 5 | vi[1] << 10 | vi[2] << 15;
+        };
+        if (small) {
+            write(Strided<int>{su, stride});
+        } else {
+            int us[UMAX];
+            if (node_u_sets<UMAX>(tri, sa, us, nu, vm, vi, min(a.ucap, UMAX)) != 0)
+                st = a.defer_cap > 0 ? -PFEM_DEFER : -PFEM_ERR_CAPACITY;
+            else
+                write(Strided<int>{us, 1});
+        }
+    }
+    r.meta[rec] = meta;
+    if (st != 0) {
+        st = defer_or_error(a, st, rec);
+        if (st < 0) record_error(a.status, -st, rec);
+    }
+}
+
+__global__ void __launch_bounds__(128, PFEM_GEOM_MIN_BLOCKS) k_p2m_geom(P2MArgs a, StarTab t, NodeRecs r)
+{
+    __shared__ int su[SET_W * 128];
+    const int I = blockIdx.x * 16 + (threadIdx.x & 15);
+    const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
+    if (I >= a.n || J >= a.n) return;
+    geom_node(a, t, r, I, J, su + threadIdx.x, 128);
+}
+
 // The quadratic adjoint as two kernels: k_p2m_geom writes each node's record (particle set, stencil
 // masks), this kernel solves the adjoint of the three edge systems with its own register budget
 // and writes the node's entries.
@@ -527,17 +621,6 @@ static __device__ __noinline__ void edge_adjoint_svd(int k, double (*pt)[6], con
         xb[i] = pb[1] + 2.0 * x[i] * pb[3] + y[i] * pb[4];
         yb[i] = pb[2] + x[i] * pb[4] + 2.0 * y[i] * pb[5];
     }
-}
-
-// Minimal-image offset of slot s from the node, in FP64 from positions of type P.
-template <typename P>
-__device__ __forceinline__ void offset64(const void *pos, int s, double xn, double yn,
-                                         double &dx, double &dy)
-{
-    P px, py;
-    load_pos((const P *)pos, s, px, py);
-    dx = wrap1((double)px - xn);
-    dy = wrap1((double)py - yn);
 }
 
 // With CHOL (FP64 systems) a node first takes the FP64 Cholesky form of the adjoint, down to FP64's
@@ -933,7 +1016,7 @@ static cudaError_t bwd_t(const GeoArgs &g, const int *perm, int C, const void *v
             // looked at the needed ones only: a scratch status word
             DevStatus *st = sizeof(S) == 8 ? (DevStatus *)(ws + 128) : b.f.status;
             launch_star_table(b.f.B, g.R0, g.rmax_far, tab, st, s, 1);     // and the fix-pass counter
-            k_p2m_geom<P, V, R><<<grid, 128, 0, s>>>(b.f, tab, recs);
+            k_p2m_geom<<<grid, 128, 0, s>>>(b.f, tab, recs);
             k_bwd_solve<P, V, R, S, POS><<<(unsigned)((b.nodes + 127) / 128), 128, 0, s>>>(b, recs);
             count_launch(2);
         } else {

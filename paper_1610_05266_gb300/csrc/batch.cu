@@ -422,14 +422,12 @@ cudaError_t launch_batch_build_cells(const void *plan, long long Ntot, long long
 
 // Workspace of the batched P2M: status (byte 0), work counter (byte 64), fix-pass queue counter
 // (byte 128), star-table queue counter (byte 132); the fix-pass queue from byte 256 (8 bytes per
-// node), then a record's space per node and the star table.
+// node), 144 bytes a node that pfem_batch_workspace_size includes and nothing uses, and the star table.
 static size_t al256b(size_t x) { return (x + 255) & ~(size_t)255; }
 
 size_t batch_p2m_ws_bytes(long long nodes_total, long long N_total)
 {
-    NodeRecs r;
-    return al256b(256 + 8 * (size_t)nodes_total) +
-           al256b(node_recs_layout(nullptr, nodes_total, &r, true)) + star_tab_bytes(N_total);
+    return al256b(256 + 8 * (size_t)nodes_total) + al256b(144 * (size_t)nodes_total) + star_tab_bytes(N_total);
 }
 
 struct BatchWs {
@@ -526,9 +524,7 @@ cudaError_t launch_batch_p2m(const void *plan, const void *pos_sorted, const uin
     a.defer_list = a.defer_cap > 0 ? (long long *)(W + 256) : nullptr;
     if (w.table) {
         char *base = W + al256b(256 + 8 * (size_t)nodes_total);
-        NodeRecs r;
-        const size_t rb = al256b(node_recs_layout(nullptr, nodes_total, &r, true));
-        w.tab = star_tab_layout(base + rb, N_total, (int *)(W + 132));
+        w.tab = star_tab_layout(base + al256b(144 * (size_t)nodes_total), N_total, (int *)(W + 132));
     }
     w.nodes = nodes_total;
     unsigned long long *counter = (unsigned long long *)(W + 64);

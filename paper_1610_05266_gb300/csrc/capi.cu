@@ -35,7 +35,7 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Binning scratch for nb*nb bins and N particles; with a mesh (n > 0) the total also covers
 // what quadratic P2M keeps in the workspace once the cells are built (the queue of nodes for
-// the SVD pass, a record's space per node and the star table).
+// the fix pass, 136 unused bytes per node and the star table).
 WsLayout ws_layout(int n, int nb, long long N, int C)
 {
     (void)C;

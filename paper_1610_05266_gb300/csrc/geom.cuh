@@ -288,34 +288,13 @@ __device__ __forceinline__ FCirc make_fcirc(float ax, float ay, float bx, float 
     return c;
 }
 
-// +1 inside, -1 outside, 0 undecided.  Inputs carry at most one rounding each; the bound
-// (2^-19 of the summed magnitudes, 32 roundings) covers inputs, K/P/Q and the evaluation.
-__device__ __forceinline__ int fcirc_filter(const FCirc &c, float x, float y)
-{
-    const float l = fmaf(x, x, y * y);
-    const float det = fmaf(c.K, l, fmaf(c.P, x, c.Q * y));
-    const float mag = fmaf(c.Ka, l, fmaf(c.Pa, fabsf(x), c.Qa * fabsf(y)));
-    const float bound = 1.9073486328125e-06f * mag;
-    return det < -bound ? 1 : (det > bound ? -1 : 0);
-}
-
-// Candidate list of the list-based star: thread-private arrays, or a thread's column of a
-// shared-memory array (entry k of thread t at k * stride + t).
+// Candidate list of the list-based star: thread-private arrays.
 template <int KLC> struct LocalList {
     float2 xy[KLC];
     int s[KLC];
     __device__ __forceinline__ float2 at(int k) const { return xy[k]; }
     __device__ __forceinline__ int slot(int k) const { return s[k]; }
     __device__ __forceinline__ void put(int k, float2 v, int sl) { xy[k] = v; s[k] = sl; }
-};
-
-struct SmemList {
-    float2 *xy;
-    int *s;
-    int stride;
-    __device__ __forceinline__ float2 at(int k) const { return xy[k * stride]; }
-    __device__ __forceinline__ int slot(int k) const { return s[k * stride]; }
-    __device__ __forceinline__ void put(int k, float2 v, int sl) { xy[k * stride] = v; s[k * stride] = sl; }
 };
 
 // The star of v from the candidates within distance D of it (list capacity KLC), written as

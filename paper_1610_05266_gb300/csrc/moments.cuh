@@ -221,10 +221,6 @@ struct FixRes {
     }
 };
 
-template <typename S> struct SolveTol;
-template <> struct SolveTol<double> { static constexpr double v = 1e-13; };
-template <> struct SolveTol<float> { static constexpr float v = 1e-6f; };
-
 // Pivot tolerance (relative to the trace) of the fused P2M's Cholesky solve, which hands a
 // system below it to the FP64 SVD pass: the normal equations square the stencil's condition,
 // so a system is solved fast only while that keeps the precision's accuracy.  Jittered lattices

@@ -74,24 +74,17 @@ static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Workspace layout of P2M after the 256-byte status block: the fix-pass queue counter at byte
 // 256 and the star-table queue counter right before it, the fix-pass queue from byte 512 (8 bytes
-// per node), then a record's space per node (the adjoint's layout) and the star table.
-static size_t recs_offset(long long nodes) { return al256(512 + 8 * (size_t)nodes); }
+// per node), then 136 bytes a node that pfem_workspace_size includes and nothing uses, and the star
+// table.
+static size_t table_offset(long long nodes) { return al256(512 + 8 * (size_t)nodes) + al256(136 * (size_t)nodes); }
 
-size_t p2m_ws_bytes(long long nodes, long long N)
-{
-    NodeRecs r;
-    const size_t recs = al256(node_recs_layout(nullptr, nodes, &r));
-    return recs_offset(nodes) + recs + star_tab_bytes(N);
-}
+size_t p2m_ws_bytes(long long nodes, long long N) { return table_offset(nodes) + star_tab_bytes(N); }
 
-// Records and star table in ws, when it has room for them.
+// Star table in ws, when it has room for it.
 static bool set_table(StarTab &t, void *ws, size_t ws_bytes, long long nodes, long long N)
 {
     if (ws_bytes < p2m_ws_bytes(nodes, N)) return false;
-    char *base = (char *)ws + recs_offset(nodes);
-    NodeRecs r;
-    const size_t recs = al256(node_recs_layout(nullptr, nodes, &r));
-    t = star_tab_layout(base + recs, N, (int *)((char *)ws + 252));
+    t = star_tab_layout((char *)ws + table_offset(nodes), N, (int *)((char *)ws + 252));
     return true;
 }
 

@@ -833,42 +833,7 @@ __global__ void __launch_bounds__(128) k_p2m_fix(P2MArgs a)
     }
 }
 
-// ---------------------------------------------------------------- node records
-// The adjoint runs the table path as two kernels, each with its own register budget: k_p2m_geom
-// locates the node and builds its particle set from the star table (memory latency bound), and
-// the adjoint's solve kernel reads what it found from a per-node record, one array per field so
-// that both kernels access it coalesced.  The forward solves run both halves in k_p2m_tab.
-struct NodeRecs {
-    int *meta;          // [nodes] nu | vi0 << 5 | vi1 << 10 | vi2 << 15, or -1: no record
-    unsigned *mask;     // [3][nodes] vm[e]
-    double *lam;        // [3][nodes] barycentric coordinates (exact in both precisions)
-    int *us;            // [UMAX][nodes] slots of the particle set
-    long long *loc;     // [nodes] Iu | Ju << 21 | nc << 42 (batches of problems), or null
-    long long nodes;
-};
-
-// Lays the record arrays for `nodes` nodes out from `base` (256-byte aligned arrays; base may be
-// null to size them); returns the bytes they take.
-inline size_t node_recs_layout(char *base, long long nodes, NodeRecs *r, bool with_loc = false)
-{
-    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t o_meta = 0;
-    const size_t o_mask = al(o_meta + sizeof(int) * (size_t)nodes);
-    const size_t o_lam = al(o_mask + 3 * sizeof(unsigned) * (size_t)nodes);
-    const size_t o_us = al(o_lam + 3 * sizeof(double) * (size_t)nodes);
-    const size_t o_loc = al(o_us + UMAX * sizeof(int) * (size_t)nodes);
-    const size_t total = with_loc ? al(o_loc + sizeof(long long) * (size_t)nodes) : o_loc;
-    if (base) {
-        r->meta = (int *)(base + o_meta);
-        r->mask = (unsigned *)(base + o_mask);
-        r->lam = (double *)(base + o_lam);
-        r->us = (int *)(base + o_us);
-        r->loc = with_loc ? (long long *)(base + o_loc) : nullptr;
-    }
-    r->nodes = nodes;
-    return total;
-}
-
+// ---------------------------------------------------------------- star table path
 // The node's particle set and stencil masks as node_u_sets gives them (same order), from stars of up
 // to 8 particles held in registers: n the stars' sizes, su the thread's column of shared memory
 // (stride between entries) that receives the slots.  Returns the set's size; the slots are complete
@@ -970,88 +935,6 @@ __device__ __forceinline__ bool warp_sets8(const StarTab &t, int st, const int t
         }
     }
     return group_min<Q>(__all_sync(__activemask(), fits) ? 1 : 0) != 0;
-}
-
-// Resident 128-thread blocks per SM of the geometry kernel: its node search waits on memory, and
-// its particle sets in shared memory and registers want room (the whole gradient step at 1025^2
-// nodes / 2048^2 particles, C = 1, FP32, with 6, 8, 10, 12 blocks: 2395, 2369, 2372, 2391 us).
-#ifndef PFEM_GEOM_MIN_BLOCKS
-#define PFEM_GEOM_MIN_BLOCKS 8
-#endif
-// Node (I, J) of the mesh of a.n nodes per side: locate it and build its particle set from the
-// star table, and write its record at index `rec` (node J * a.n + I of a single problem; the
-// problem's offset plus that in a batch, which also records the node's coordinates).
-template <typename P, typename V, typename R>
-__device__ __forceinline__ void geom_node(const P2MArgs &a, const StarTab &t, const NodeRecs &r,
-                                          int I, int J, long long rec, int *su, int stride)
-{
-    const int nc = a.n - 1;
-    const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
-    const long long node = (long long)J * a.n + I;
-    const uint2 qn = make_uint2(node_fx(Iu, nc), node_fx(Ju, nc));
-    int tri[3];
-    int st = locate_tab(a.B, t, qn, a.R0, tri);
-    TabStar sa[3];
-#pragma unroll
-    for (int e = 0; e < 3; ++e)
-        if (st == 0) {
-            sa[e] = tab_star(t, tri[e]);
-            if (sa[e].n < 0) st = sa[e].n == -1 ? -PFEM_FAR : sa[e].n;
-        }
-    int meta = -1, nu = 0;
-    unsigned vm[3] = {0u, 0u, 0u};
-    const bool small = warp_sets8<1>(t, st, tri, sa, a.ucap, su, stride, nu, vm);
-    if (st == 0) {
-        NodePos<P, R> np;
-        np.init(Iu, Ju, nc);
-        R lam[3];
-        barycentric(a, np, tri, lam);
-        int vi[3] = {0, 1, 2};
-        auto write = [&](auto us) {
-            // entries up to the warp's largest set, -1 past this node's, so that the warp's
-            // stores to each entry array cover contiguous runs of it
-            const int nw = __reduce_max_sync(__activemask(), nu);
-            for (int i = 0; i < nw; ++i) r.us[i * r.nodes + rec] = i < nu ? us[i] : -1;
-#pragma unroll
-            for (int e = 0; e < 3; ++e) {
-                r.mask[e * r.nodes + rec] = vm[e];
-                r.lam[e * r.nodes + rec] = (double)lam[e];
-            }
-            meta = nu | vi[0] << 5 | vi[1] << 10 | vi[2] << 15;
-        };
-        if (small) {
-            write(Strided<int>{su, stride});
-        } else {
-            int us[UMAX];
-            if (node_u_sets<UMAX>(tri, sa, us, nu, vm, vi, min(a.ucap, UMAX)) != 0)
-                st = a.defer_cap > 0 ? -PFEM_DEFER : -PFEM_ERR_CAPACITY;
-            else
-                write(Strided<int>{us, 1});
-        }
-    }
-    r.meta[rec] = meta;
-    if (r.loc) r.loc[rec] = (long long)Iu | (long long)Ju << 21 | (long long)nc << 42;
-    if (st != 0) {
-        st = defer_or_error(a, st, rec);
-        if (st < 0) record_error(a.status, -st, rec);
-        if (a.out) {                    // the adjoint uses this kernel without a mesh output
-            R acc[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) acc[c] = (R)nan_of<R>();
-            store_vals<V, R>((V *)a.out, node, a.C, acc);
-        }
-    }
-}
-
-template <typename P, typename V, typename R>
-__global__ void __launch_bounds__(128, PFEM_GEOM_MIN_BLOCKS) k_p2m_geom(P2MArgs a, StarTab t,
-                                                                        NodeRecs r)
-{
-    __shared__ int su[SET_W * 128];
-    const int I = blockIdx.x * 16 + (threadIdx.x & 15);
-    const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
-    if (I >= a.n || J >= a.n) return;
-    geom_node<P, V, R>(a, t, r, I, J, (long long)J * a.n + I, su + threadIdx.x, 128);
 }
 
 // The fix pass of the table path: the queued nodes located with the star table (complete after
