@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(256) k_bin_batch(const BPlanDev *pl, const P *
 __device__ __forceinline__ bool totals_ok(const BPlanDev *pl, long long nodes, const StarTab &t,
                                           DevStatus *st)
 {
-    const bool ok = nodes == pl->total_nodes && t.N == pl->total_particles;
+    const bool ok = (nodes == pl->total_nodes) & (t.N == pl->total_particles);   // (both loads at once)
     if (!ok && blockIdx.x == 0 && threadIdx.x == 0) record_error(st, PFEM_ERR_INVALID_ARG, -1);
     return ok;
 }
