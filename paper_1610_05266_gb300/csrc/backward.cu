@@ -355,29 +355,29 @@ __device__ __forceinline__ int bwd_u_solve64(const BwdArgs &b, int Iu, int Ju, c
 
 // Linear shape functions: the triangle's vertices are the entries.
 template <typename P, typename V, typename R, bool POS>
-__global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_bwd_linear(BwdArgs b)
+__global__ void __launch_bounds__(STAR_TPB, PFEM_LINEAR_MIN_BLOCKS) k_bwd_linear(BwdArgs b)
 {
     __shared__ __align__(16) unsigned char lists[HullList::BYTES];
     const P2MArgs &a = b.f;
     const int I = blockIdx.x * 16 + (threadIdx.x & 15);
     const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
-    if (I >= a.n || J >= a.n) return;
     const int nc = a.n - 1;
-    const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
+    const bool mesh = I <= nc && J <= nc;
+    const int Iu = I >= nc ? 0 : I, Ju = J >= nc ? 0 : J;
     const long long node = (long long)J * a.n + I;
     R g[8];
     bool any = false;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-        g[c] = c < a.C ? load_val<V, R>((const V *)b.grad_mesh + node * a.C + c) : R(0);
+        g[c] = mesh && c < a.C ? load_val<V, R>((const V *)b.grad_mesh + node * a.C + c) : R(0);
         any |= g[c] != R(0);
     }
     int us[3];
     R uw[3] = {R(0), R(0), R(0)}, ub[3], udx[3] = {R(0), R(0), R(0)}, udy[3] = {R(0), R(0), R(0)};
     int nu = 0;
+    int st = locate_hull(a.B, any, make_uint2(node_fx(Iu, nc), node_fx(Ju, nc)), a.R0,
+                         HullList::at(lists, threadIdx.x), us);       // every lane of the warp
     if (any) {
-        int st = locate_hull(a.B, make_uint2(node_fx(Iu, nc), node_fx(Ju, nc)), a.R0,
-                             HullList::at(lists, threadIdx.x), us);
         if (st == 0) {
             NodePos<P, R> np;
             np.init(Iu, Ju, nc);
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_bwd_linear(B
             if (st < 0) record_error(a.status, -st, node);
         }
     }
-    write_entries<R, R, POS>(b, node, nu, us, uw, udx, udy);
+    if (mesh) write_entries<R, R, POS>(b, node, nu, us, uw, udx, udy);
 }
 
 // ---------------------------------------------------------------- node records

@@ -762,15 +762,17 @@ __global__ void __launch_bounds__(128, PFEM_P2M_MIN_BLOCKS) k_p2m(P2MArgs a)
 // Linear shape functions: one thread a node.  The node's triangle comes from the star of its nearest
 // particle, by the hull over the thread's list in shared memory as in the star table (gift wrapping
 // over lists in local memory took 169 us for 513^2 nodes over 1254^2 particles, this 107); the table itself
-// would hold the stars of every particle, six a node there.
+// would hold the stars of every particle, six a node there.  Every lane of the warp calls (locate_hull).
 template <typename P, typename V, typename R, bool WEIGHTS>
 __device__ __forceinline__ void linear_node(const P2MArgs &a, const HullList &L, int I, int J)
 {
     const int nc = a.n - 1;
-    const int Iu = I == nc ? 0 : I, Ju = J == nc ? 0 : J;
+    const bool mine = I <= nc && J <= nc;
+    const int Iu = I >= nc ? 0 : I, Ju = J >= nc ? 0 : J;
     const long long node = (long long)J * a.n + I;
     int tri[3];
-    int st = locate_hull(a.B, make_uint2(node_fx(Iu, nc), node_fx(Ju, nc)), a.R0, L, tri);
+    int st = locate_hull(a.B, mine, make_uint2(node_fx(Iu, nc), node_fx(Ju, nc)), a.R0, L, tri);
+    if (!mine) return;
     R lam[3] = {R(0), R(0), R(0)}, acc[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) acc[c] = R(0);
@@ -806,13 +808,18 @@ __device__ __forceinline__ void linear_node(const P2MArgs &a, const HullList &L,
     }
 }
 
+// Resident 128-thread blocks per SM: the warp search wants registers (at 64 it spills). 8, 6, 5, 4 blocks:
+// 257^2 nodes over 1024^2 uniform random particles 597, 341, 300, 277 us, 1025^2 over 1025^2 4565, 2715,
+// 2666, 2856, 513^2 over 1254^2 lattice particles 135, 115, 107, 107.
+#ifndef PFEM_LINEAR_MIN_BLOCKS
+#define PFEM_LINEAR_MIN_BLOCKS 5
+#endif
 template <typename P, typename V, typename R, bool WEIGHTS>
-__global__ void __launch_bounds__(STAR_TPB, PFEM_STAR_MIN_BLOCKS) k_p2m_linear(P2MArgs a)
+__global__ void __launch_bounds__(STAR_TPB, PFEM_LINEAR_MIN_BLOCKS) k_p2m_linear(P2MArgs a)
 {
     __shared__ __align__(16) unsigned char lists[HullList::BYTES];
     const int I = blockIdx.x * 16 + (threadIdx.x & 15);
     const int J = blockIdx.y * 8 + (threadIdx.x >> 4);
-    if (I >= a.n || J >= a.n) return;
     linear_node<P, V, R, WEIGHTS>(a, HullList::at(lists, threadIdx.x), I, J);
 }
 

@@ -506,21 +506,6 @@ __device__ __forceinline__ int star_hull(const Bins &B, int v, uint2 pv, const R
     return sp;
 }
 
-// Locate fixed-point point p as locate() does, the star of its nearest particle by the hull over the
-// calling thread's list, and only where that cannot certify it by gift wrapping.
-static __device__ __forceinline__ int locate_hull(const Bins &B, uint2 p, int R0, const HullList &L, int tri[3])
-{
-    const int v0 = nearest_particle(B, p, R0);
-    if (v0 < 0) return v0;
-    const uint2 pv = __ldg(B.q + v0);
-    __align__(16) int star[KMAX];
-    int c = -1;
-    if (B.dmax > 0.f && B.last4 >= 0) c = star_hull(B, v0, pv, make_region(B, pv, R0), B.dmax, L, star);
-    if (c == -1) c = star_region(B, v0, pv, R0, star);
-    if (c < 0) return c;
-    return fan_walk(B, p, v0, ArrStar{star, c}, c, [&](int u, int w) { return apex_of(B, u, w, R0); }, tri);
-}
-
 // The list attempt for slot v (candidates in L): its star into the table, or v queued.
 __device__ __forceinline__ void star_list_slot(const Bins &B, int R0, const StarTab &t, long long v,
                                                const HullList &L, DevStatus *st)
@@ -546,11 +531,14 @@ __device__ __forceinline__ void star_list_slot(const Bins &B, int R0, const Star
 // one keeps the lanes busy.  (A thread per star, over lists in shared and local memory, took 32 us
 // for the lattice's twelve and 1.77 ms for 590,000 of 1024^2 uniform random particles.)
 
-// Candidates of a warp in shared memory: offsets from v and slots.
+// Candidates of a warp in shared memory: offsets from v and slots, in rows of 32 that lie `stride`
+// apart (32: one array).
 constexpr int WSTAR_CAP = 96;
 struct WarpList {
     int2 *d;
     int *s;
+    int stride;
+    __device__ __forceinline__ int at(int k) const { return (k >> 5) * stride + (k & 31); }
 };
 
 // An int whose order is the float's.
@@ -707,8 +695,8 @@ __device__ __forceinline__ int star_warp(const Bins &B, int v, uint2 pv, int R0,
                     if (in) {
                         nearer(d, s);
                         if (at < WSTAR_CAP) {
-                            L.d[at] = d;
-                            L.s[at] = s;
+                            L.d[L.at(at)] = d;
+                            L.s[L.at(at)] = s;
                         }
                     }
                     m += __popc(got);
@@ -720,7 +708,7 @@ __device__ __forceinline__ int star_warp(const Bins &B, int v, uint2 pv, int R0,
             if (m > WSTAR_CAP) break;
             if (m == 0) continue;
             const int c = wrap_warp(B, pv, g, D, u0, d0, [&](auto &&f) {
-                for (int k = lane; k < m; k += 32) f(L.d[k], L.s[k]);
+                for (int k = lane; k < m; k += 32) f(L.d[L.at(k)], L.s[L.at(k)]);
             }, entry);
             if (c != -1) return c;
         }
@@ -741,6 +729,49 @@ __device__ __forceinline__ int star_warp(const Bins &B, int v, uint2 pv, int R0,
         if (c != -1) return c;
     }
     return -PFEM_FAR;
+}
+
+// star_warp out of line, for kernels whose lanes have their registers for the hull attempt.
+static __device__ __noinline__ int star_warp_call(const Bins &B, int v, int R0, WarpList L, int &entry)
+{
+    return star_warp(B, v, __ldg(B.q + v), R0, L, entry);
+}
+
+// Locate fixed-point point p as locate() does, the star of its nearest particle by the hull over the
+// calling thread's list.  Where that cannot certify the star (more than half of a uniform random set's)
+// the warp searches it together, its candidates in the lists' memory: every lane of the warp calls,
+// `mine` where it has a point.  (Gift wrapping a lane instead keeps its candidates in local memory, for
+// which the lists leave no L1: linear P2M of 1024^2 uniform random particles onto 257^2 nodes 1257 us,
+// by gift wrapping alone 780, so 300.)
+static __device__ __forceinline__ int locate_hull(const Bins &B, bool mine, uint2 p, int R0, const HullList &L,
+                                                  int tri[3])
+{
+    static_assert((WSTAR_CAP + 31) / 32 <= HullList::ROWS, "a warp's candidates fit its lists");
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int v0 = mine ? nearest_particle(B, p, R0) : -1;
+    __align__(16) int star[KMAX];
+    int c = v0;
+    if (v0 >= 0) {
+        c = -1;
+        const uint2 pv = __ldg(B.q + v0);
+        if (B.dmax > 0.f && B.last4 >= 0) c = star_hull(B, v0, pv, make_region(B, pv, R0), B.dmax, L, star);
+    }
+    __syncwarp();
+    const WarpList W{reinterpret_cast<int2 *>(L.xy - lane), L.s - lane, HullList::STRIDE};
+    for (unsigned left = __ballot_sync(full, v0 >= 0 && c == -1); left; left &= left - 1) {
+        const int j = __ffs(left) - 1;
+        int entry = -1;
+        const int n = star_warp_call(B, __shfl_sync(full, v0, j), R0, W, entry);
+#pragma unroll
+        for (int k = 0; k < KMAX; ++k) {
+            const int x = __shfl_sync(full, entry, k);
+            if (lane == j) star[k] = x;
+        }
+        if (lane == j) c = n;
+    }
+    if (c < 0) return c;
+    return fan_walk(B, p, v0, ArrStar{star, c}, c, [&](int u, int w) { return apex_of(B, u, w, R0); }, tri);
 }
 
 // Store a queued slot's star (entry of the calling lane) or record its error (an exhausted region as

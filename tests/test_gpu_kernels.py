@@ -436,3 +436,37 @@ def test_batch_totals_are_compared_for_every_solve(P, solve):
                                vals.repeat(2, 1), P.PFEM_SHAPE_QUADRATIC, getattr(P, "PFEM_SOLVE_" + solve), b.mesh, 8,
                                64, b.ws)
     assert b.status() == (1, -1) and bool((b.mesh == 7.0).all())
+
+
+LINEAR = {"uniform": lambda: uniform(70, 256, 901), "sparse": lambda: uniform(129, 60, 902),
+          "dense_disk": lambda: G.Problem("disk", 37, 32, 0.0, 0, _disk(32, 0.1, 700, 920), None)}
+
+
+@pytest.mark.parametrize("which", sorted(LINEAR))
+def test_linear_on_irregular_sets(P, which):
+    """Linear P2M, weights, adjoint and batches (all block shapes) where the hull leaves many stars to the
+    warp, on meshes that leave lanes of a warp without a node, within FP64's bound of the oracle."""
+    pr = LINEAR[which]()
+    n, N, C = pr.n, len(pr.pos), 2
+    v = noise(N, C)
+    ref = O.p2m(n, pr.pos, v, shape=0, nthreads=8)
+    pos, vals = torch.tensor(pr.pos, device="cuda"), torch.tensor(v, device="cuda")
+    proj = P.Projector(n, N, C=C, pos_dtype=torch.float64)
+    proj.build(pos)
+    mesh = proj.p2m(vals, shape=P.PFEM_SHAPE_LINEAR)
+    w = proj.shape_weights(shape=P.PFEM_SHAPE_LINEAR)
+    proj.check(which)
+    assert relerr(mesh.cpu().numpy(), ref) <= TOL64
+    assert relerr(proj.p2m(vals, weights=w).cpu().numpy(), ref) <= TOL64
+    g = 2.0 * G.uniform01(G.SEED_BASE + 961, n * n * C).reshape(n, n, C) - 1.0
+    g[:, ::3] = 0.0                              # nodes without an upstream gradient
+    gv, gp = proj.backward(vals, torch.tensor(g, device="cuda"), shape=P.PFEM_SHAPE_LINEAR)
+    assert proj.backward_status()[0] == 0
+    ov, op = O.p2m_backward(n, pr.pos, v, g, shape=0)
+    assert relerr(gv.cpu().numpy(), ov) <= TOL64 and relerr(gp.cpu().numpy(), op) <= 1e-10
+    b = P.Batch([(n, N)] * 2, C, torch.float64, "cuda")
+    b.build(pos.repeat(2, 1))
+    for rows in (4, 8, 16):
+        b.mesh.fill_(float("nan"))
+        b.p2m(vals.repeat(2, 1), shape=P.PFEM_SHAPE_LINEAR, tile_rows=rows)
+        assert b.status()[0] == 0 and torch.equal(b.mesh_view(0), mesh) and torch.equal(b.mesh_view(1), mesh)
