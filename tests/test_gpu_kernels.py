@@ -470,3 +470,26 @@ def test_linear_on_irregular_sets(P, which):
         b.mesh.fill_(float("nan"))
         b.p2m(vals.repeat(2, 1), shape=P.PFEM_SHAPE_LINEAR, tile_rows=rows)
         assert b.status()[0] == 0 and torch.equal(b.mesh_view(0), mesh) and torch.equal(b.mesh_view(1), mesh)
+
+
+@pytest.mark.parametrize("M", [20, 37, 64])
+def test_adjoint_of_few_particles_on_a_fine_mesh(P, M):
+    """Particles with more entries than a thread sorts by itself (17 to several hundred): linear adjoint
+    against the oracle, the same bits twice, and from checkpointed weights."""
+    n = 65
+    pos = G.jittered_lattice(M, 0.25, G.SEED_BASE + 997)
+    N = len(pos)
+    v, g = noise(N, 2), 2.0 * G.uniform01(G.SEED_BASE + 962, n * n * 2).reshape(n, n, 2) - 1.0
+    proj = P.Projector(n, N, C=2, pos_dtype=torch.float64)
+    proj.build(torch.tensor(pos, device="cuda"))
+    vals, gm = torch.tensor(v, device="cuda"), torch.tensor(g, device="cuda")
+    for shape in (0, 1):
+        gv, gp = proj.backward(vals, gm, shape=shape)
+        again = proj.backward(vals, gm, shape=shape)
+        w = proj.shape_weights(shape=shape)
+        cv, cp = proj.backward(vals, gm, shape=shape, weights=w)
+        assert proj.backward_status()[0] == 0
+        assert torch.equal(gv, again[0]) and torch.equal(gp, again[1]) and torch.equal(gp, cp)
+        ov, op = O.p2m_backward(n, pos, v, g, shape=shape)
+        assert relerr(gv.cpu().numpy(), ov) <= TOL64 and relerr(cv.cpu().numpy(), ov) <= TOL64
+        assert relerr(gp.cpu().numpy(), op) <= TOL64
