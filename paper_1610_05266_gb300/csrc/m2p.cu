@@ -388,17 +388,24 @@ static cudaError_t m2p_q_t(int n, long long N, const void *pos, int C, const voi
 {
     long long blocks = (N + 255) / 256;
     if (blocks > num_sms() * 16LL) blocks = num_sms() * 16LL;
-    // four FP32 components as one 16-byte access when the arrays allow it; one to three (and
-    // four in the other types) with the component loop unrolled
+    // the component loop unrolled; four FP32 components as one 16-byte access when the arrays allow it
+    // (else the loop over eight with a test each)
     const bool aligned = ((reinterpret_cast<uintptr_t>(mesh) | reinterpret_cast<uintptr_t>(vals)) & 15) == 0;
     auto go = [&](auto ct) {
         k_m2p_q<P, V, R, decltype(ct)::value><<<(unsigned)blocks, 256, 0, s>>>(
             n, N, (const P *)pos, C, (const V *)mesh, (V *)vals, mq_table<R>());
     };
-    if (C == 1) go(std::integral_constant<int, 1>());
-    else if (C == 3) go(std::integral_constant<int, 3>());
-    else if (C == 4 && (aligned || sizeof(V) != 4)) go(std::integral_constant<int, 4>());
-    else go(std::integral_constant<int, 0>());
+    switch (C == 4 && sizeof(V) == 4 && !aligned ? 0 : C) {
+    case 1: go(std::integral_constant<int, 1>()); break;
+    case 2: go(std::integral_constant<int, 2>()); break;
+    case 3: go(std::integral_constant<int, 3>()); break;
+    case 4: go(std::integral_constant<int, 4>()); break;
+    case 5: go(std::integral_constant<int, 5>()); break;
+    case 6: go(std::integral_constant<int, 6>()); break;
+    case 7: go(std::integral_constant<int, 7>()); break;
+    case 8: go(std::integral_constant<int, 8>()); break;
+    default: go(std::integral_constant<int, 0>());
+    }
     count_launch();
     return cudaGetLastError();
 }
