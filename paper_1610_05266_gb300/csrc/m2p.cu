@@ -19,13 +19,13 @@ namespace pfem {
 // component 632 -> 314 us with four (their bytes take 104 us), 1254^2 of three FP32 ones 18 -> 13
 // us with two; the round trip of four FP32 ones at 1025^2 / 2048^2 1061 us with one and 1057 with two;
 // four FP64 ones keep enough in flight with one.  FP64 positions in fixed point (m2p.cuh): 1024^2 of three 63 -> 26 us.
-template <typename P, typename V, typename R, int CT, int U>
+template <typename P, typename V, typename R, int CT, int U, bool FINE>
 __global__ void __launch_bounds__(256) k_m2p(int n, long long N, const P *__restrict__ pos,
                                              int Crt, const V *__restrict__ mesh,
                                              V *__restrict__ vals)
 {
     const long long m0 = blockIdx.x * (256LL * U) + threadIdx.x;
-    m2p_particles<P, V, R, CT, U>(n, m0, N, pos, Crt, mesh, vals);
+    m2p_particles<P, V, R, CT, U, FINE>(n, m0, N, pos, Crt, mesh, vals);
 }
 
 template <typename P, typename V, typename R>
@@ -35,8 +35,14 @@ static cudaError_t m2p_t(int n, long long N, const void *pos, int C, const void 
     const bool aligned = ((reinterpret_cast<uintptr_t>(mesh) | reinterpret_cast<uintptr_t>(vals)) & 15) == 0;
     auto go = [&](auto ct, auto u) {
         constexpr int CT = decltype(ct)::value, U = decltype(u)::value;
-        k_m2p<P, V, R, CT, U><<<(unsigned)((N + 256 * U - 1) / (256 * U)), 256, 0, s>>>(
-            n, N, (const P *)pos, C, (const V *)mesh, (V *)vals);
+        auto launch = [&](auto fine) {
+            k_m2p<P, V, R, CT, U, decltype(fine)::value><<<(unsigned)((N + 256 * U - 1) / (256 * U)), 256, 0, s>>>(
+                n, N, (const P *)pos, C, (const V *)mesh, (V *)vals);
+        };
+        // FP64 positions on fine meshes: another look at those near the origin (m2p.cuh), which costs the
+        // others 4 % (2048^2 particles of one component on 1025^2 nodes 73 us, 76 with it)
+        if (sizeof(P) == 8 && n > 2049) launch(std::integral_constant<bool, sizeof(P) == 8>());
+        else launch(std::false_type());
     };
     // the components in registers up to four; four FP32 ones as one 16-byte access when the arrays
     // allow it

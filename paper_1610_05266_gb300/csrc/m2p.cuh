@@ -31,6 +31,12 @@ template <typename R> __device__ __forceinline__ R local_coord(R x, int i, int n
 // local coordinate may lie a rounding outside [0, 1].  Below 2^-12 a position has bits beyond 2^-64, whose
 // rounding nc enlarges: with more than 2048 cells a side, where that passes FP64's own rounding, those
 // positions, 2^-12 of all, take the FP64 product.
+__device__ __forceinline__ bool needs_f64(double x, int nc) { return nc > 2048 && (unsigned)__double2hiint(x) < 1011u << 20; }
+static __device__ __noinline__ long long local_f64(double x, int nc, int i)
+{
+    return __double2ll_rn(fma(x, (double)nc, (double)-i) * 4611686018427387904.0);
+}
+template <bool FINE = true>
 __device__ __forceinline__ long long local_fix(double x, int nc, int &i)
 {
     const unsigned long long q = (unsigned long long)fx64(x);
@@ -38,8 +44,7 @@ __device__ __forceinline__ long long local_fix(double x, int nc, int &i)
     unsigned t = (unsigned)(q >> 32);
     t += f > 0x80000000u || (f == 0x80000000u && (t & 1u)) ? 1u : 0u;
     i = bin_of(t, nc);
-    if (nc > 2048 && (unsigned)__double2hiint(x) < 1011u << 20)
-        return __double2ll_rn(fma(x, (double)nc, (double)-i) * 4611686018427387904.0);
+    if (FINE && needs_f64(x, nc)) return local_f64(x, nc, i);
     int d = (int)__umul64hi(q, (unsigned long long)nc) - i;
     d -= d > 1 ? nc : 0;
     d += d < -1 ? nc : 0;
@@ -53,13 +58,15 @@ __device__ __forceinline__ double unit62(long long x)
     return x == 0 ? 0.0 : __hiloint2double(__double2hiint(d) - (62 << 20), __double2loint(d));
 }
 
-template <typename P, typename R>
+// FINE: with the product of needs_f64 positions in place (out of line, as are all its uses: predicated, its FP64
+// instructions cost M2P of other positions up to a quarter).
+template <typename P, typename R, bool FINE = true>
 __device__ __forceinline__ MeshCell<R> mesh_cell(P px, P py, int n)
 {
     const int nc = n - 1;
     MeshCell<R> c;
     if constexpr (sizeof(P) == 8) {
-        const long long s = local_fix(px, nc, c.i), t = local_fix(py, nc, c.j);
+        const long long s = local_fix<FINE>(px, nc, c.i), t = local_fix<FINE>(py, nc, c.j);
         const long long hi = max(s, t), lo = min(s, t);
         c.mid = s >= t ? 1 : n;
         c.w0 = (R)unit62((1ll << 62) - hi);
@@ -95,8 +102,8 @@ __device__ __forceinline__ bool cell_index(P px, P py, int nc, int &i, int &j)
 }
 
 // M2P of the particles m0 + 256 u < end, u < U, on a mesh of n nodes per side; CT components, or C with
-// CT = 0.
-template <typename P, typename V, typename R, int CT, int U>
+// CT = 0; FINE: n may be above 2049.
+template <typename P, typename V, typename R, int CT, int U, bool FINE = true>
 __device__ __forceinline__ void m2p_particles(int n, long long m0, long long end, const P *__restrict__ pos,
                                               int Crt, const V *__restrict__ mesh, V *__restrict__ vals)
 {
@@ -107,8 +114,16 @@ __device__ __forceinline__ void m2p_particles(int n, long long m0, long long end
         const long long m = min(m0 + 256 * u, end - 1);
         P px, py;
         load_pos(pos, m, px, py);
-        cell[u] = mesh_cell<P, R>(px, py, n);
+        cell[u] = mesh_cell<P, R, false>(px, py, n);
     }
+    if constexpr (sizeof(P) == 8 && FINE)
+        if (n > 2049)                            // again, where a coordinate needs the product
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                P px, py;
+                load_pos(pos, min(m0 + 256 * u, end - 1), px, py);
+                if (needs_f64(px, n - 1) || needs_f64(py, n - 1)) cell[u] = mesh_cell<P, R>(px, py, n);
+            }
     if constexpr (CT == 4 && sizeof(V) == 4 && sizeof(R) == 4) {
         float4 a[U], b[U], c[U];
 #pragma unroll
