@@ -72,11 +72,12 @@ typedef enum {
 typedef enum { PFEM_F64 = 0, PFEM_F32 = 1, PFEM_BF16 = 2 } pfem_dtype;
 typedef enum { PFEM_SHAPE_LINEAR = 0, PFEM_SHAPE_QUADRATIC = 1 } pfem_shape;
 typedef enum {
-    PFEM_SOLVE_F64 = 0,         /* FP64 accuracy: FP32 Cholesky, the solution refined to the last bits
-                                   of 64-bit fixed point; FP64 Cholesky or SVD where that fails */
+    PFEM_SOLVE_F64 = 0,         /* FP64 accuracy: FP32 Cholesky, the solution refined in 64-bit fixed
+                                   point; FP64 Cholesky or SVD where that stalls */
     PFEM_SOLVE_F32 = 1,         /* in FP32 after centring/scaling by the edge length */
     PFEM_SOLVE_F32_REFINED = 2, /* FP32 Cholesky + one refinement step, residual in 64-bit fixed
-                                   point (at least FP64's accuracy) */
+                                   point: coordinates rounded to 32 bits of the stencil's
+                                   largest, the result as accurate as with an FP64 residual */
     PFEM_SOLVE_F32_REFINED_FF = 3 /* FP32 Cholesky + one refinement step, residual in float-float
                                    (~48-bit significand) or better: runs the fixed-point
                                    residual of PFEM_SOLVE_F32_REFINED */
@@ -241,15 +242,17 @@ pfem_status pfem_shape_quadratic(pfem_ctx *ctx, int32_t n, int32_t nb, int64_t N
  * factorisation of its 6x6 moment matrix.  The call runs a fast pass over every node and a fix
  * pass over the nodes the fast pass queued: a node with an edge whose pivot falls below the
  * fast tolerance (rank deficient, e.g. a stencil of five particles, or too ill-conditioned for
- * the FP32 factor: 3e-4 of the trace), with more than the context's
+ * the FP32 factor: 3e-4 of the trace, 3e-5 where the solution is refined to FP64, or a refinement
+ * that stalls), with more than the context's
  * node_capacity distinct particles, or whose search ran out of its first region (a sparse
  * region or a void), is recomputed in FP64, each edge by Cholesky down to a pivot of 1e-6 of the
- * trace and below that with the minimum-norm least-squares solution by SVD (App. A), and
- * searches up to the context's search_radius_max.  Linear shape functions queue
+ * trace (refined once for FP64 weights) and below that with the minimum-norm least-squares solution
+ * by SVD (App. A), and searches up to the context's search_radius_max.  Linear shape functions queue
  * only the last kind.  Workspace layout after the 256-byte status block: the fix-pass queue
  * from byte 512 (8 bytes per node; with ws_bytes < 520 there is no queue and such nodes record
- * PFEM_ERR_DEGENERATE or PFEM_ERR_CAPACITY), then, for the quadratic apply form, 136 bytes of
- * record per node and the star table (72 bytes per particle).  With room for them the fast
+ * PFEM_ERR_DEGENERATE or PFEM_ERR_CAPACITY; where it does not hold every node, nodes that FP64's
+ * Cholesky can solve take no entry but are solved in place), then, for quadratic shape functions,
+ * 136 unused bytes per node and the star table (72 bytes per particle).  With room for them the fast
  * pass is the star table of every particle (see pfem_delaunay_stars) and one kernel that, per
  * node, locates it with the table, builds its particle set and solves the three edge systems.
  * With less room, one kernel
@@ -389,9 +392,10 @@ pfem_status pfem_batch_build_cells(pfem_ctx *ctx, const void *plan, int64_t N_to
  * Values FP32 (FP32 positions) or FP64 (FP64 positions, FP64 solve).  nodes_total and N_total
  * must be totals[2] and totals[0] of the pfem_batch_plan_init call that built `plan`; the
  * workspace (pfem_batch_workspace_size with those totals) holds, after its 256-byte status
- * block, the fix-pass queue (8 bytes per node), the per-node records and the star table.
+ * block, the fix-pass queue (8 bytes per node), 144 unused bytes per node and the star table.
  * Quadratic shape functions then run as for one problem: the star table of every problem, a
- * persistent kernel that locates the nodes and solves the edge systems, and the fix pass over the queued nodes (FP64, SVD solve, widest search radius).  The
+ * persistent kernel that locates the nodes and solves the edge systems, and the fix pass over the
+ * queued nodes (FP64, Cholesky or SVD as for one problem, widest search radius).  For every solve the
  * kernels compare the totals with the plan's own before writing anything and record
  * PFEM_ERR_INVALID_ARG (detail -1) when they differ.  With a smaller workspace (at least 256
  * bytes plus the queue) every node runs a fused per-node kernel; linear shape functions always

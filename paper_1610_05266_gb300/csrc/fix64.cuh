@@ -23,6 +23,10 @@
 //   uniform random, 504,000 edges        median 2e-16 (1e-15), 99.9 % 1e-14 (2e-14), worst 2e-13 (8e-13)
 // Before the shift by h, with a stalled refinement accepted at 2^-36 of the largest |y'|, the uniform
 // random set's were 7e-16, 6e-14 and 2e-11.
+//
+// Measured (round trip, FP64 values; FP64 systems before): 513^2 nodes / 1024^2 particles 1798 -> 624 us,
+// 33^2 / 64^2 200 -> 89 us with four lanes a node; the mesh's error against 64-bit arithmetic 2.6e-16 ->
+// 1.6e-16 of its 2-norm.
 #pragma once
 
 #include "moments.cuh"
