@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(RETRY_TPB, RETRY_BLOCKS) k_star_retry_batch(co
     __shared__ int ss[RETRY_TPB / 32 * WSTAR_CAP];
     const int w = threadIdx.x >> 5;
     const BDesc *D = plan_desc(pl);
-    star_retry(t, lists, WarpList{sd + w * WSTAR_CAP, ss + w * WSTAR_CAP, 32}, base.status, [&](int v, int &R0) {
+    star_retry(t, lists, WarpList{sd + w * WSTAR_CAP, ss + w * WSTAR_CAP}, base.status, [&](int v, int &R0) {
         const BDesc d = D[find_problem(pl->P, v, [&](int k) { return D[k].poff; })];
         P2MArgs a;
         problem_args(a, base, d, pl->total_particles);

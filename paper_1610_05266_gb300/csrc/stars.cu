@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(RETRY_TPB, RETRY_BLOCKS) k_star_retry(Bins B, 
     __shared__ int2 sd[RETRY_TPB / 32 * WSTAR_CAP];
     __shared__ int ss[RETRY_TPB / 32 * WSTAR_CAP];
     const int w = threadIdx.x >> 5;
-    star_retry(t, lists, WarpList{sd + w * WSTAR_CAP, ss + w * WSTAR_CAP, 32}, st, [&](int, int &r) {
+    star_retry(t, lists, WarpList{sd + w * WSTAR_CAP, ss + w * WSTAR_CAP}, st, [&](int, int &r) {
         r = R0;
         return B;
     });

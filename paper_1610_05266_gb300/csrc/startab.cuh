@@ -531,15 +531,16 @@ __device__ __forceinline__ void star_list_slot(const Bins &B, int R0, const Star
 // one keeps the lanes busy.  (A thread per star, over lists in shared and local memory, took 32 us
 // for the lattice's twelve and 1.77 ms for 590,000 of 1024^2 uniform random particles.)
 
-// Candidates of a warp in shared memory: offsets from v and slots, in rows of 32 that lie `stride`
+// Candidates of a warp in shared memory: offsets from v and slots, in rows of 32 that lie STRIDE
 // apart (32: one array).
 constexpr int WSTAR_CAP = 96;
-struct WarpList {
+template <int STRIDE> struct WarpListT {
     int2 *d;
     int *s;
-    int stride;
-    __device__ __forceinline__ int at(int k) const { return (k >> 5) * stride + (k & 31); }
+    static __device__ __forceinline__ int at(int k) { return STRIDE == 32 ? k : (k >> 5) * STRIDE + (k & 31); }
 };
+using WarpList = WarpListT<32>;
+using HullWarpList = WarpListT<HullList::STRIDE>;      // in the lists of the warp's lanes
 
 // An int whose order is the float's.
 __device__ __forceinline__ int ordered(float x)
@@ -649,7 +650,8 @@ __device__ __forceinline__ int wrap_warp(const Bins &B, uint2 pv, const Region &
 // particles 44 % of the stars have a circumcircle wider than 2 mean spacings, 0.3 % wider than
 // 3.5), then every particle of growing regions up to B.rmax.  Lane k receives entry k.  Returns
 // the count or -PFEM_ERR_* / -PFEM_FAR, the same in every lane.
-__device__ __forceinline__ int star_warp(const Bins &B, int v, uint2 pv, int R0, const WarpList &L,
+template <typename List>
+__device__ __forceinline__ int star_warp(const Bins &B, int v, uint2 pv, int R0, const List &L,
                                              int &entry)
 {
     const unsigned full = 0xffffffffu;
@@ -732,7 +734,7 @@ __device__ __forceinline__ int star_warp(const Bins &B, int v, uint2 pv, int R0,
 }
 
 // star_warp out of line, for kernels whose lanes have their registers for the hull attempt.
-static __device__ __noinline__ int star_warp_call(const Bins &B, int v, int R0, WarpList L, int &entry)
+static __device__ __noinline__ int star_warp_call(const Bins &B, int v, int R0, HullWarpList L, int &entry)
 {
     return star_warp(B, v, __ldg(B.q + v), R0, L, entry);
 }
@@ -758,7 +760,7 @@ static __device__ __forceinline__ int locate_hull(const Bins &B, bool mine, uint
         if (B.dmax > 0.f && B.last4 >= 0) c = star_hull(B, v0, pv, make_region(B, pv, R0), B.dmax, L, star);
     }
     __syncwarp();
-    const WarpList W{reinterpret_cast<int2 *>(L.xy - lane), L.s - lane, HullList::STRIDE};
+    const HullWarpList W{reinterpret_cast<int2 *>(L.xy - lane), L.s - lane};
     for (unsigned left = __ballot_sync(full, v0 >= 0 && c == -1); left; left &= left - 1) {
         const int j = __ffs(left) - 1;
         int entry = -1;
