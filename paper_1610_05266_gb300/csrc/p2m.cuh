@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(128, PFEM_P2M_MIN_BLOCKS) k_p2m(P2MArgs a)
 
 // Linear shape functions: one thread a node.  The node's triangle comes from the star of its nearest
 // particle, by the hull over the thread's list in shared memory as in the star table (gift wrapping
-// over lists in local memory took 169 us for 513^2 nodes over 1254^2 particles, this 107); the table itself
+// over lists in local memory took 169 us for 513^2 nodes over 1254^2 particles, this 92); the table itself
 // would hold the stars of every particle, six a node there.  Every lane of the warp calls (locate_hull).
 template <typename P, typename V, typename R, bool WEIGHTS>
 __device__ __forceinline__ void linear_node(const P2MArgs &a, const HullList &L, int I, int J)
